@@ -22,8 +22,11 @@
 #include <vector>
 
 #include "ibim_internal.cuh"
+#include "math64.cuh"
 
 namespace ibim {
+
+constexpr int kStageThreads = 128;
 
 struct LsGrid {
     int64_t lo[3];
@@ -124,39 +127,121 @@ __device__ __forceinline__ void weno_pair(const LsGrid& g, const double* __restr
     pp = weno5(D[5], D[4], D[3], D[2], D[1]);
 }
 
-// One TVD-RK3 stage: out = a base + b (in + dt L(in)).
-//   mode 0: L = |grad phi| with the Godunov form for speed -1 (inward flow);
-//   mode 1: L = -sgn_h(phi0) (|grad phi| - 1) (reinitialisation).
-__global__ void ls_stage_kernel(LsGrid g, const double* __restrict__ in, const double* __restrict__ base,
-                                const double* __restrict__ phi0, double* __restrict__ out, double a, double b,
-                                double dt, int mode)
+// max(-p, 0)^2 of a one-sided WENO5 derivative p (times h: the inputs are plain
+// differences of phi), from its five differences v1..v5 and the three
+// sub-stencil values 6 q1..6 q3.  WENO is homogeneous, so the factor 1/h is
+// applied by the caller.  The weights c_i / (s_i + e)^2 are multiplied through
+// by the three squares, (s_j + e)^2 (s_k + e)^2 c_i, so that one reciprocal
+// serves them all; smoothness and e carry a common factor 4, which cancels.
+__device__ __forceinline__ double weno5_scaled(double v1, double v2, double v3, double v4, double v5, double q1,
+                                               double q2, double q3)
 {
-    const int64_t M = g.n[0] * g.n[1] * g.n[2];
-    const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= M) return;
-    const int64_t i = id % g.n[0], j = (id / g.n[0]) % g.n[1], k = id / (g.n[0] * g.n[1]);
+    const double g1 = v2 - v1, g2 = v3 - v2, g3 = v4 - v3, g4 = v5 - v4;
+    const double d1 = g2 - g1, d2 = g3 - g2, d3 = g4 - g3;
+    const double e1 = fma(3.0, g2, -g1), e2 = g2 + g3, e3 = fma(-3.0, g3, g4);
+    const double m = max_abs64(max_abs64(max_abs64(v1, v2), max_abs64(v3, v4)), v5);
+    // 4 (1e-6 m^2 + tiny); the floor keeps the products below normal numbers
+    const double e = fmax(4e-6 * m * m, 4e-56);
+    const double t1 = fma(13.0 / 3.0 * d1, d1, fma(e1, e1, e));
+    const double t2 = fma(13.0 / 3.0 * d2, d2, fma(e2, e2, e));
+    const double t3 = fma(13.0 / 3.0 * d3, d3, fma(e3, e3, e));
+    const double u1 = t2 * t3, u2 = t1 * t3, u3 = t1 * t2;
+    const double a1 = u1 * u1, a2 = 6.0 * u2 * u2, a3 = 3.0 * u3 * u3;
+    const double num = fma(a1, q1, fma(a2, q2, a3 * q3));
+    const double den = a1 + a2 + a3;
+    return num * rcp64(den);
+}
+
+// Contribution of one axis to (h |grad phi|)^2 by Godunov's rule for fronts
+// that move towards larger phi (the caller flips the sign of f otherwise):
+// max(min(p_-, 0)^2, max(p_+, 0)^2) from the seven values f along the axis.
+// A WENO value is a combination of its three sub-stencil values with positive
+// weights, so it has their sign when they agree: then the side whose term is
+// zero needs no weights, and usually at most one side is left (both only
+// around a minimum of phi).  The one or two evaluations use the same code, so
+// lanes on either side of the front do not diverge.
+__device__ __forceinline__ double godunov_axis(const double (&f)[7])
+{
+    double D[6];
+#pragma unroll
+    for (int m = 0; m < 6; ++m) D[m] = f[m + 1] - f[m];
+    // 6 q of the backward (m) and forward (p) derivative
+    const double m1 = fma(2.0, D[0], fma(-7.0, D[1], 11.0 * D[2]));
+    const double m2 = fma(2.0, D[3], fma(5.0, D[2], -D[1]));
+    const double m3 = fma(2.0, D[2], fma(5.0, D[3], -D[4]));
+    const double p1 = fma(2.0, D[5], fma(-7.0, D[4], 11.0 * D[3]));
+    const double p2 = fma(2.0, D[2], fma(5.0, D[3], -D[4]));
+    const double p3 = fma(2.0, D[3], fma(5.0, D[2], -D[1]));
+    // signs from the high words (a -0 or a positive denormal only costs or saves an evaluation that gives 0)
+    const bool need_m = (__double2hiint(m1) | __double2hiint(m2) | __double2hiint(m3)) < 0;
+    const bool need_p = max(max(__double2hiint(p1), __double2hiint(p2)), __double2hiint(p3)) > 0;
     double s = 0.0;
-    double p0 = 0.0;
-    if (mode == 1) p0 = phi0[id];
-    for (int ax = 0; ax < 3; ++ax) {
-        double pm, pp;
-        weno_pair(g, in, i, j, k, ax, pm, pp);
-        if (mode == 0 || p0 <= 0.0) {  // upwind from the larger phi
-            const double u = pm < 0.0 ? pm : 0.0, v = pp > 0.0 ? pp : 0.0;
-            s += fmax(u * u, v * v);
-        } else {
-            const double u = pm > 0.0 ? pm : 0.0, v = pp < 0.0 ? pp : 0.0;
-            s += fmax(u * u, v * v);
+    if (need_m || need_p) {
+        const bool b = need_m;
+        const double p = weno5_scaled(b ? D[0] : D[5], b ? D[1] : D[4], D[2 + (b ? 0 : 1)], b ? D[3] : D[2],
+                                      b ? D[4] : D[1], b ? m1 : p1, b ? m2 : p2, b ? m3 : p3);
+        const double w = b ? fmin(p, 0.0) : fmax(p, 0.0);
+        s = w * w;
+        if (need_m && need_p) {
+            const double q = fmax(weno5_scaled(D[5], D[4], D[3], D[2], D[1], p1, p2, p3), 0.0);
+            s = fmax(s, q * q);
         }
     }
-    double L;
-    if (mode == 0) {
-        L = sqrt(s);
-    } else {
-        const double sg = p0 / sqrt(p0 * p0 + g.h * g.h);
-        L = -sg * (sqrt(s) - 1.0);
+    return s;  // 36 h^2 times the axis term (the sub-stencil values carry a factor 6)
+}
+
+// sgn_h(phi0) = phi0 / sqrt(phi0^2 + h^2), the fixed sign field of the reinitialisation.
+__global__ void ls_sign_kernel(int64_t M, double h, const double* __restrict__ phi, double* __restrict__ sgn)
+{
+    const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (id >= M) return;
+    const double p = phi[id];
+    sgn[id] = p / sqrt(p * p + h * h);
+}
+
+// One TVD-RK3 stage: out = a base + b (in + dt L(in)).
+//   sgn == NULL: L = |grad phi| with the Godunov form for speed -1 (inward flow);
+//   else:        L = -sgn (|grad phi| - 1) (reinitialisation).
+// Bound by the FP64 pipe (2 lanes per clock and SM).  Against one full WENO5
+// evaluation per side with the textbook divisions (1,600 FP64 instructions per
+// node): one reciprocal per evaluation, constant divisors folded into a common
+// factor 6, 1/h applied once, and the sign rule of godunov_axis.
+__global__ void __launch_bounds__(kStageThreads)
+    ls_stage_kernel(LsGrid g, const double* __restrict__ in, const double* __restrict__ base,
+                    const double* __restrict__ sgn, double* __restrict__ out, double a, double b, double dt,
+                    double inv6h)
+{
+    const int64_t M = g.n[0] * g.n[1] * g.n[2];
+    const int64_t id = (int64_t)blockIdx.x * kStageThreads + threadIdx.x;
+    if (id >= M) return;
+    // grids hold at most 2^31 nodes: 32-bit index arithmetic (unsigned)
+    const unsigned n0 = (unsigned)g.n[0], n1 = (unsigned)g.n[1], n2 = (unsigned)g.n[2], u = (unsigned)id;
+    const unsigned row = u / n0;
+    const int i = (int)(u - row * n0), k = (int)(row / n1), j = (int)(row - (unsigned)k * n1);
+    const double sg = sgn != nullptr ? sgn[id] : 0.0;
+    const bool flip = sg > 0.0;
+    const double c = in[id];
+    const double* __restrict__ p = in + id;
+    const int pos[3] = {i, j, k}, len[3] = {(int)n0, (int)n1, (int)n2};
+    const int64_t stride[3] = {1, (int64_t)n0, (int64_t)n0 * n1};
+    double s = 0.0;
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+        double f[7];
+#pragma unroll
+        for (int q = -3; q <= 3; ++q) {
+            int o = q;  // zero Neumann: indices clamped to the box
+            if (q < 0) o = max(q, -pos[ax]);
+            if (q > 0) o = min(q, len[ax] - 1 - pos[ax]);
+            const double v = q == 0 ? c : p[o * stride[ax]];
+            f[q + 3] = flip ? -v : v;
+        }
+        s += godunov_axis(f);
     }
-    out[id] = a * base[id] + b * (in[id] + dt * L);
+    // |grad phi| = sqrt(s) / (6 h)
+    const double grad = s > 0.0 ? s * rsqrt64(s) * inv6h : 0.0;
+    const double L = sgn == nullptr ? grad : -sg * (grad - 1.0);
+    out[id] = fma(a, base[id], b * fma(dt, L, c));
 }
 
 // --------------------------------------------------------------- cavities
@@ -420,7 +505,7 @@ ibim_status build_levelset(ibim_ctx* c, int64_t Na, const double* z, const doubl
 
     Atom* d_atoms = nullptr;
     int* d_start = nullptr;
-    double *d_phi = nullptr, *d_t1 = nullptr, *d_t2 = nullptr, *d_phi0 = nullptr;
+    double *d_phi = nullptr, *d_t1 = nullptr, *d_t2 = nullptr, *d_sgn = nullptr;
     uint8_t* d_lab = nullptr;
     int* d_flag = nullptr;
     unsigned long long* d_ncav = nullptr;
@@ -430,7 +515,7 @@ ibim_status build_levelset(ibim_ctx* c, int64_t Na, const double* z, const doubl
         cudaFree(d_start);
         cudaFree(d_t1);
         cudaFree(d_t2);
-        cudaFree(d_phi0);
+        cudaFree(d_sgn);
         cudaFree(d_lab);
         cudaFree(d_flag);
         cudaFree(d_ncav);
@@ -450,7 +535,7 @@ ibim_status build_levelset(ibim_ctx* c, int64_t Na, const double* z, const doubl
     c->d_phi = d_phi;
     LS_CUDA(cudaMalloc((void**)&d_t1, sizeof(double) * M));
     LS_CUDA(cudaMalloc((void**)&d_t2, sizeof(double) * M));
-    LS_CUDA(cudaMalloc((void**)&d_phi0, sizeof(double) * M));
+    LS_CUDA(cudaMalloc((void**)&d_sgn, sizeof(double) * M));
     LS_CUDA(cudaMalloc((void**)&d_lab, M));
     LS_CUDA(cudaMalloc((void**)&d_flag, sizeof(int)));
     LS_CUDA(cudaMalloc((void**)&d_ncav, sizeof(unsigned long long)));
@@ -459,6 +544,8 @@ ibim_status build_levelset(ibim_ctx* c, int64_t Na, const double* z, const doubl
 
     const int bs = 256;
     const unsigned nb = (unsigned)((M + bs - 1) / bs);
+    const unsigned ns = (unsigned)((M + kStageThreads - 1) / kStageThreads);
+    const double inv6h = 1.0 / (6.0 * h);
     vdw_kernel<<<nb, bs, 0, c->stream>>>(g, cl, d_atoms, d_start, L, probe, d_phi);
     count_launch(c);
     LS_CUDA(cudaGetLastError());
@@ -468,9 +555,10 @@ ibim_status build_levelset(ibim_ctx* c, int64_t Na, const double* z, const doubl
         const int steps = (int)ceil(probe / (0.5 * h));
         const double dt = probe / steps;
         for (int s = 0; s < steps; ++s) {
-            ls_stage_kernel<<<nb, bs, 0, c->stream>>>(g, d_phi, d_phi, nullptr, d_t1, 0.0, 1.0, dt, 0);
-            ls_stage_kernel<<<nb, bs, 0, c->stream>>>(g, d_t1, d_phi, nullptr, d_t2, 0.75, 0.25, dt, 0);
-            ls_stage_kernel<<<nb, bs, 0, c->stream>>>(g, d_t2, d_phi, nullptr, d_phi, 1.0 / 3.0, 2.0 / 3.0, dt, 0);
+            ls_stage_kernel<<<ns, kStageThreads, 0, c->stream>>>(g, d_phi, d_phi, nullptr, d_t1, 0.0, 1.0, dt, inv6h);
+            ls_stage_kernel<<<ns, kStageThreads, 0, c->stream>>>(g, d_t1, d_phi, nullptr, d_t2, 0.75, 0.25, dt, inv6h);
+            ls_stage_kernel<<<ns, kStageThreads, 0, c->stream>>>(g, d_t2, d_phi, nullptr, d_phi, 1.0 / 3.0, 2.0 / 3.0, dt,
+                                                                 inv6h);
             count_launch(c, 3);
         }
         LS_CUDA(cudaGetLastError());
@@ -512,11 +600,13 @@ ibim_status build_levelset(ibim_ctx* c, int64_t Na, const double* z, const doubl
         const double k0 = 0.5, k1 = eps / h;
         const int steps = (int)ceil((k1 + 4.0) / k0 - 1e-9);
         const double dt = k0 * h;
-        LS_CUDA(cudaMemcpyAsync(d_phi0, d_phi, sizeof(double) * M, cudaMemcpyDeviceToDevice, c->stream));
+        ls_sign_kernel<<<nb, bs, 0, c->stream>>>(M, h, d_phi, d_sgn);
+        count_launch(c);
         for (int s = 0; s < steps; ++s) {
-            ls_stage_kernel<<<nb, bs, 0, c->stream>>>(g, d_phi, d_phi, d_phi0, d_t1, 0.0, 1.0, dt, 1);
-            ls_stage_kernel<<<nb, bs, 0, c->stream>>>(g, d_t1, d_phi, d_phi0, d_t2, 0.75, 0.25, dt, 1);
-            ls_stage_kernel<<<nb, bs, 0, c->stream>>>(g, d_t2, d_phi, d_phi0, d_phi, 1.0 / 3.0, 2.0 / 3.0, dt, 1);
+            ls_stage_kernel<<<ns, kStageThreads, 0, c->stream>>>(g, d_phi, d_phi, d_sgn, d_t1, 0.0, 1.0, dt, inv6h);
+            ls_stage_kernel<<<ns, kStageThreads, 0, c->stream>>>(g, d_t1, d_phi, d_sgn, d_t2, 0.75, 0.25, dt, inv6h);
+            ls_stage_kernel<<<ns, kStageThreads, 0, c->stream>>>(g, d_t2, d_phi, d_sgn, d_phi, 1.0 / 3.0, 2.0 / 3.0, dt,
+                                                                 inv6h);
             count_launch(c, 3);
         }
         LS_CUDA(cudaGetLastError());
