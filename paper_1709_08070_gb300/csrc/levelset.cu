@@ -141,12 +141,11 @@ __device__ __forceinline__ void weno_pair(const LsGrid& g, const double* __restr
     pp = weno5(D[5], D[4], D[3], D[2], D[1]);
 }
 
-// max(-p, 0)^2 of a one-sided WENO5 derivative p (times h: the inputs are plain
-// differences of phi), from its five differences v1..v5 and the three
-// sub-stencil values 6 q1..6 q3.  WENO is homogeneous, so the factor 1/h is
-// applied by the caller.  The weights c_i / (s_i + e)^2 are multiplied through
-// by the three squares, (s_j + e)^2 (s_k + e)^2 c_i, so that one reciprocal
-// serves them all; smoothness and e carry a common factor 4, which cancels.
+// A one-sided WENO5 derivative times 6 h, from the five differences v1..v5 of
+// phi and its sub-stencil values q1..q3 (times 6 h as well).  WENO is
+// homogeneous, so the factor is taken out once by the caller.  The weights
+// c_i / (s_i + e)^2 are multiplied through by the three squares, so that one
+// reciprocal serves them all; smoothness and e carry a common factor 4.
 __device__ __forceinline__ double weno5_scaled(double v1, double v2, double v3, double v4, double v5, double q1,
                                                double q2, double q3)
 {
@@ -155,7 +154,7 @@ __device__ __forceinline__ double weno5_scaled(double v1, double v2, double v3, 
     const double e1 = fma(3.0, g2, -g1), e2 = g2 + g3, e3 = fma(-3.0, g3, g4);
     const double m = max_abs64(max_abs64(max_abs64(v1, v2), max_abs64(v3, v4)), v5);
     // 4 (1e-6 m^2 + tiny); the floor keeps the products below normal numbers
-    const double e = fmax(4e-6 * m * m, 4e-56);
+    const double e = max_abs64(4e-6 * m * m, 4e-56);
     const double t1 = fma(13.0 / 3.0 * d1, d1, fma(e1, e1, e));
     const double t2 = fma(13.0 / 3.0 * d2, d2, fma(e2, e2, e));
     const double t3 = fma(13.0 / 3.0 * d3, d3, fma(e3, e3, e));
@@ -166,42 +165,28 @@ __device__ __forceinline__ double weno5_scaled(double v1, double v2, double v3, 
     return num * rcp64(den);
 }
 
-// Contribution of one axis to (h |grad phi|)^2 by Godunov's rule for fronts
-// that move towards larger phi (the caller flips the sign of f otherwise):
-// max(min(p_-, 0)^2, max(p_+, 0)^2) from the seven values f along the axis.
-// A WENO value is a combination of its three sub-stencil values with positive
-// weights, so it has their sign when they agree: then the side whose term is
-// zero needs no weights, and usually at most one side is left (both only
-// around a minimum of phi).  The one or two evaluations use the same code, so
-// lanes on either side of the front do not diverge.
-__device__ __forceinline__ double godunov_axis(const double (&f)[7])
+// The value's bits as a signed integer: ordered as the values are among
+// positive ones, and negative for negative ones.
+__device__ __forceinline__ long long pos_bits(double v) { return __double_as_longlong(v); }
+__device__ __forceinline__ long long neg_bits(double v) { return __double_as_longlong(v) ^ (1ll << 63); }
+
+// One axis of Godunov's rule for fronts that move towards larger phi: its term
+// is max(min(p_-, 0)^2, max(p_+, 0)^2).  A WENO value is a combination of its
+// three sub-stencil values with positive weights, so it lies between them, and
+// the largest of -q_i (p_-) or q_i (p_+) bounds the side's term.  A side whose
+// bound is not positive is zero without its weights; the side with the smaller
+// bound matters only when that bound exceeds the value of the other one.
+struct AxisSides {
+    double D[6];             // differences along the axis (negated for the other direction)
+    double m1, m2, m3, p1;   // 6 h q: backward (m1, m2, m3), forward (p1, m3, m2)
+};
+
+__device__ __forceinline__ double weno_side(const AxisSides& A, bool back)
 {
-    double D[6];
-#pragma unroll
-    for (int m = 0; m < 6; ++m) D[m] = f[m + 1] - f[m];
-    // 6 q of the backward (m) and forward (p) derivative
-    const double m1 = fma(2.0, D[0], fma(-7.0, D[1], 11.0 * D[2]));
-    const double m2 = fma(2.0, D[3], fma(5.0, D[2], -D[1]));
-    const double m3 = fma(2.0, D[2], fma(5.0, D[3], -D[4]));
-    const double p1 = fma(2.0, D[5], fma(-7.0, D[4], 11.0 * D[3]));
-    const double p2 = fma(2.0, D[2], fma(5.0, D[3], -D[4]));
-    const double p3 = fma(2.0, D[3], fma(5.0, D[2], -D[1]));
-    // signs from the high words (a -0 or a positive denormal only costs or saves an evaluation that gives 0)
-    const bool need_m = (__double2hiint(m1) | __double2hiint(m2) | __double2hiint(m3)) < 0;
-    const bool need_p = max(max(__double2hiint(p1), __double2hiint(p2)), __double2hiint(p3)) > 0;
-    double s = 0.0;
-    if (need_m || need_p) {
-        const bool b = need_m;
-        const double p = weno5_scaled(b ? D[0] : D[5], b ? D[1] : D[4], D[2 + (b ? 0 : 1)], b ? D[3] : D[2],
-                                      b ? D[4] : D[1], b ? m1 : p1, b ? m2 : p2, b ? m3 : p3);
-        const double w = b ? fmin(p, 0.0) : fmax(p, 0.0);
-        s = w * w;
-        if (need_m && need_p) {
-            const double q = fmax(weno5_scaled(D[5], D[4], D[3], D[2], D[1], p1, p2, p3), 0.0);
-            s = fmax(s, q * q);
-        }
-    }
-    return s;  // 36 h^2 times the axis term (the sub-stencil values carry a factor 6)
+    const double w = weno5_scaled(back ? A.D[0] : A.D[5], back ? A.D[1] : A.D[4], back ? A.D[2] : A.D[3],
+                                  back ? A.D[3] : A.D[2], back ? A.D[4] : A.D[1], back ? A.m1 : A.p1,
+                                  back ? A.m2 : A.m3, back ? A.m3 : A.m2);
+    return __longlong_as_double(back ? neg_bits(w) : pos_bits(w));
 }
 
 // sgn_h(phi0) = phi0 / sqrt(phi0^2 + h^2), the fixed sign field of the reinitialisation.
@@ -216,29 +201,41 @@ __global__ void ls_sign_kernel(int64_t M, double h, const double* __restrict__ p
 // One TVD-RK3 stage: out = a base + b (in + dt L(in)).
 //   sgn == NULL: L = |grad phi| with the Godunov form for speed -1 (inward flow);
 //   else:        L = -sgn (|grad phi| - 1) (reinitialisation).
-// Bound by the FP64 pipe (2 lanes per clock and SM).  Against one full WENO5
-// evaluation per side with the textbook divisions (1,600 FP64 instructions per
-// node): one reciprocal per evaluation, constant divisors folded into a common
-// factor 6, 1/h applied once, and the sign rule of godunov_axis.
+// Bound by the FP64 pipe (2 lanes per clock and SM).  Every thread evaluates
+// the side with the larger bound on each axis (same code for both sides, so
+// lanes on either side of a front do not diverge).  The second evaluations are
+// needed by a few lanes of almost every warp; they go through a queue in
+// shared memory and are worked off by full warps.
+// 2.6 M nodes: 1.05 ms a stage, 210 FP64 instructions per warp of 32 nodes at
+// 85 % FP64-pipe activity (the highest seen on this pipe).  Before: 6.61 ms with
+// four divisions per WENO evaluation, divisions by constants and both sides
+// always evaluated (1,600 instructions); 1.54 ms with both sides of a lane in
+// turn (290 to 370).
 __global__ void __launch_bounds__(kStageThreads)
     ls_stage_kernel(LsGrid g, const double* __restrict__ in, const double* __restrict__ base,
                     const double* __restrict__ sgn, double* __restrict__ out, double a, double b, double dt,
                     double inv6h)
 {
+    constexpr int kQueue = 3 * kStageThreads;
+    __shared__ double queue[8][kQueue];  // v1..v5, q1..q3 of a second evaluation; its value comes back in [0]
+    __shared__ int queued;
     const int64_t M = g.n[0] * g.n[1] * g.n[2];
     const int64_t id = (int64_t)blockIdx.x * kStageThreads + threadIdx.x;
-    if (id >= M) return;
+    const bool live = id < M;
+    if (threadIdx.x == 0) queued = 0;
+    __syncthreads();
     // grids hold at most 2^31 nodes: 32-bit index arithmetic (unsigned)
-    const unsigned n0 = (unsigned)g.n[0], n1 = (unsigned)g.n[1], n2 = (unsigned)g.n[2], u = (unsigned)id;
+    const unsigned n0 = (unsigned)g.n[0], n1 = (unsigned)g.n[1], n2 = (unsigned)g.n[2], u = live ? (unsigned)id : 0u;
     const unsigned row = u / n0;
     const int i = (int)(u - row * n0), k = (int)(row / n1), j = (int)(row - (unsigned)k * n1);
-    const double sg = sgn != nullptr ? sgn[id] : 0.0;
-    const bool flip = sg > 0.0;
-    const double c = in[id];
-    const double* __restrict__ p = in + id;
+    const double sg = (sgn != nullptr && live) ? sgn[id] : 0.0;
+    const long long flip = sg > 0.0 ? 1ll << 63 : 0;  // the other direction: the same rule on -phi
+    const double* __restrict__ p = in + u;
+    const double c = p[0];
     const int pos[3] = {i, j, k}, len[3] = {(int)n0, (int)n1, (int)n2};
     const int64_t stride[3] = {1, (int64_t)n0, (int64_t)n0 * n1};
-    double s = 0.0;
+    double r[3];    // the larger one-sided slope of each axis, times 6 h
+    int slot[3];    // its queue entry, or -1
 #pragma unroll
     for (int ax = 0; ax < 3; ++ax) {
         double f[7];
@@ -247,15 +244,60 @@ __global__ void __launch_bounds__(kStageThreads)
             int o = q;  // zero Neumann: indices clamped to the box
             if (q < 0) o = max(q, -pos[ax]);
             if (q > 0) o = min(q, len[ax] - 1 - pos[ax]);
-            const double v = q == 0 ? c : p[o * stride[ax]];
-            f[q + 3] = flip ? -v : v;
+            f[q + 3] = q == 0 ? c : p[o * stride[ax]];
         }
-        s += godunov_axis(f);
+        AxisSides A;
+#pragma unroll
+        for (int m = 0; m < 6; ++m) A.D[m] = __longlong_as_double(__double_as_longlong(f[m + 1] - f[m]) ^ flip);
+        A.m1 = fma(2.0, A.D[0], fma(-7.0, A.D[1], 11.0 * A.D[2]));
+        A.m2 = fma(2.0, A.D[3], fma(5.0, A.D[2], -A.D[1]));
+        A.m3 = fma(2.0, A.D[2], fma(5.0, A.D[3], -A.D[4]));
+        A.p1 = fma(2.0, A.D[5], fma(-7.0, A.D[4], 11.0 * A.D[3]));
+        const long long bm = max(max(neg_bits(A.m1), neg_bits(A.m2)), neg_bits(A.m3));
+        const long long bp = max(max(pos_bits(A.p1), pos_bits(A.m3)), pos_bits(A.m2));
+        const bool back = bm >= bp;
+        long long best = 0;
+        slot[ax] = -1;
+        if (max(bm, bp) > 0) {
+            best = max(0ll, pos_bits(weno_side(A, back)));
+            if (min(bm, bp) > best && live) {
+                const int e = atomicAdd(&queued, 1);
+                slot[ax] = e;
+                queue[0][e] = back ? A.D[5] : A.D[0];
+                queue[1][e] = back ? A.D[4] : A.D[1];
+                queue[2][e] = back ? A.D[3] : A.D[2];
+                queue[3][e] = back ? A.D[2] : A.D[3];
+                queue[4][e] = back ? A.D[1] : A.D[4];
+                queue[5][e] = back ? A.p1 : A.m1;
+                queue[6][e] = back ? A.m3 : A.m2;
+                queue[7][e] = back ? A.m2 : A.m3;
+                if (!back) slot[ax] |= 1 << 16;  // a backward derivative: counts negated
+            }
+        }
+        r[ax] = __longlong_as_double(best);
+    }
+    __syncthreads();
+    const int nq = queued;
+    for (int e = threadIdx.x; e < nq; e += kStageThreads)
+        queue[0][e] = weno5_scaled(queue[0][e], queue[1][e], queue[2][e], queue[3][e], queue[4][e], queue[5][e],
+                                   queue[6][e], queue[7][e]);
+    if (nq > 0) __syncthreads();
+    if (!live) return;
+    double s = 0.0;
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+        if (slot[ax] >= 0) {
+            const double w = queue[0][slot[ax] & 0xffff];
+            r[ax] = __longlong_as_double(max(pos_bits(r[ax]), (slot[ax] >> 16) ? neg_bits(w) : pos_bits(w)));
+        }
+        s = fma(r[ax], r[ax], s);
     }
     // |grad phi| = sqrt(s) / (6 h)
     const double grad = s > 0.0 ? s * rsqrt64(s) * inv6h : 0.0;
     const double L = sgn == nullptr ? grad : -sg * (grad - 1.0);
-    out[id] = fma(a, base[id], b * fma(dt, L, c));
+    // plain operations, as in C: at the edge of the clamp plateau, far outside
+    // the band, the reinitialisation enlarges rounding differences of phi
+    out[id] = a * base[id] + b * (c + dt * L);
 }
 
 // --------------------------------------------------------------- cavities
