@@ -156,19 +156,18 @@ ibim_status timing_collect(ibim_ctx* c)
     return IBIM_OK;
 }
 
-// Source payload and partial-sum buffers large enough for both precisions
-// and every FP32 variant, so operator applications never reallocate them.
+// Source payload and partial-sum buffers large enough for every FP32 variant
+// and the float-float path (and the payload for the FP64 path, whose partial
+// sums are its own), so operator applications never reallocate them.
 ibim_status ensure_operator_workspaces(ibim_ctx* c)
 {
     if (c->ws_sized) return IBIM_OK;
     const int64_t N = c->N;
     IBIM_TRY(ensure(c, &c->d_src, &c->src_bytes,
-                    std::max(std::max((size_t)N * 8 * sizeof(double), (size_t)padded_nodes(N) * 2 * sizeof(float4)),
+                    std::max(std::max(f64_src_bytes(N), (size_t)padded_nodes(N) * 2 * sizeof(float4)),
                              ff_src_bytes(N))));
     IBIM_TRY(ff_prepare_context(c));
-    const PairSchedule s64 = make_schedule(N, kF64TTile, N, kF64STile, f64_grid_cap(c));
-    size_t need = (size_t)s64.grid * s64.max_segs * 2 * kF64TTile * sizeof(double);
-    need = std::max(need, ff_part_doubles(c) * sizeof(double));
+    size_t need = ff_part_doubles(c) * sizeof(double);
     const int keep = c->f32_variant, keep_bps = c->f32_bps;
     c->f32_bps = 0;
     for (int v = 0; v < f32_variant_count(); ++v) {
@@ -198,14 +197,7 @@ ibim_status apply_operator(ibim_ctx* c, const PairConsts& k, int precision, VecR
         return f32_fixup(c, k, s, in, out, d_skip);
     }
     if (precision == IBIM_F32T) return tc_apply(c, k, in, out, d_skip);
-    if (precision == IBIM_F64) {
-        const PairSchedule s = make_schedule(N, kF64TTile, N, kF64STile, f64_grid_cap(c));
-        IBIM_TRY(f64_pack(c, in, d_skip));
-        IBIM_TRY(timing_begin(c));
-        IBIM_TRY(f64_pairs(c, k, s, d_skip));
-        IBIM_TRY(timing_end(c, N * N));
-        return f64_fixup(c, k, s, in, out, d_skip);
-    }
+    if (precision == IBIM_F64) return f64_apply(c, k, in, out, d_skip);
     if (precision == IBIM_FF) {
         const PairSchedule s = ff_schedule(c);
         IBIM_TRY(ff_pack(c, in, d_skip));
@@ -299,6 +291,7 @@ void ibim_destroy(ibim_ctx* c)
     cudaFree(c->d_q);
     cudaFree(c->d_src);
     cudaFree(c->d_part);
+    cudaFree(c->d_part64);
     cudaFree(c->d_red);
     cudaFree(c->d_err);
     cudaFree(c->d_io);

@@ -415,6 +415,7 @@ static ibim_status capture_step(ibim_ctx* c, const PairConsts& k, int precision)
     // precision) touches is sized for both precisions before capture, so that
     // no later call reallocates a buffer the graph holds a pointer to.
     IBIM_TRY(ensure_operator_workspaces(c));
+    if (precision == IBIM_F64) IBIM_TRY(f64_prepare(c));
     if (w->graph_valid && w->graph_prec == precision && memcmp(&w->graph_k, &k, sizeof(k)) == 0 &&
         w->graph_generation == c->ws_generation && w->graph_variant == c->f32_variant && w->graph_bps == c->f32_bps)
         return IBIM_OK;

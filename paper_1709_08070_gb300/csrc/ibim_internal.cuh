@@ -50,10 +50,6 @@ constexpr int kF32MaxTTile = 1024;  // largest target tile of any variant
 constexpr int kPadNodes = 1024;
 static_assert(kPadNodes % kF32STile == 0 && kPadNodes % kF32MaxTTile == 0, "padding");
 __host__ __device__ inline int64_t padded_nodes(int64_t N) { return (N + kPadNodes - 1) / kPadNodes * kPadNodes; }
-// FP64 path: one target per thread, 128 threads, 128 sources per tile.
-constexpr int kF64Threads = 128;
-constexpr int kF64TTile = kF64Threads;
-constexpr int kF64STile = 128;
 
 // Stream-K schedule of a pair-sum launch over (target tile, source tile) steps.
 struct PairSchedule {
@@ -137,6 +133,8 @@ struct ibim_ctx {
     size_t src_bytes = 0;
     double* d_part = nullptr;  // stream-K partial sums
     size_t part_bytes = 0;
+    double* d_part64 = nullptr;  // FP64 path: item counter, exp table, partial sums of the block pairs
+    size_t part64_bytes = 0;
     double* d_red = nullptr;   // small reduction scratch (energy, area, norms)
     size_t red_bytes = 0;
     unsigned* d_err = nullptr; // device error word (kDevErr* bits), zeroed at build
@@ -236,12 +234,10 @@ ibim_status ff_pairs(ibim_ctx* c, const PairConsts& k, const PairSchedule& s, co
 ibim_status ff_fixup(ibim_ctx* c, const PairConsts& k, const PairSchedule& s, VecRef in, OutRef out,
                      const int* d_skip);
 ibim_status ff_prepare_context(ibim_ctx* c);
-// FP64 path pieces (pair_f64.cu)
-ibim_status f64_pack(ibim_ctx* c, VecRef in, const int* d_skip);
-ibim_status f64_pairs(ibim_ctx* c, const PairConsts& k, const PairSchedule& s, const int* d_skip);
-ibim_status f64_fixup(ibim_ctx* c, const PairConsts& k, const PairSchedule& s, VecRef in, OutRef out,
-                      const int* d_skip);
-int f64_grid_cap(ibim_ctx* c);
+// FP64 path (pair_f64.cu): f64_prepare sizes its partial sums (before a capture)
+size_t f64_src_bytes(int64_t N);
+ibim_status f64_prepare(ibim_ctx* c);
+ibim_status f64_apply(ibim_ctx* c, const PairConsts& k, VecRef in, OutRef out, const int* d_skip);
 
 // RHS / energy / area (rhs_energy.cu)
 ibim_status rhs_launch(ibim_ctx* c, double eps_in, double* d_g);
