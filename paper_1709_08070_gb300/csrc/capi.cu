@@ -292,6 +292,7 @@ void ibim_destroy(ibim_ctx* c)
     cudaFree(c->d_src);
     cudaFree(c->d_part);
     cudaFree(c->d_part64);
+    cudaFree(c->d_exptab);
     cudaFree(c->d_red);
     cudaFree(c->d_err);
     cudaFree(c->d_io);

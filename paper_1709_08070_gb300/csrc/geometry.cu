@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "ibim_internal.cuh"
+#include "math64.cuh"
 
 namespace ibim {
 
@@ -332,6 +333,12 @@ static ibim_status compact_order(ibim_ctx* c)
     return IBIM_OK;
 }
 
+__global__ void exp_table_kernel(double* __restrict__ tab)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < kExpTab) tab[i] = exp2((double)i * (1.0 / kExpTab));
+}
+
 ibim_status finish_geometry(ibim_ctx* c, bool reorder)
 {
     if (reorder) IBIM_TRY(compact_order(c));
@@ -347,6 +354,10 @@ ibim_status finish_geometry(ibim_ctx* c, bool reorder)
     const int bs = 256;
     pack_geometry_f32_kernel<<<(unsigned)((n_pad + bs - 1) / bs), bs, 0, c->stream>>>(
         c->d_geo64, N, n_pad, c->centroid[0], c->centroid[1], c->centroid[2], c->d_pos32, c->d_nrm32);
+    count_launch(c);
+    IBIM_CUDA(cudaGetLastError());
+    IBIM_CUDA(cudaMalloc((void**)&c->d_exptab, sizeof(double) * kExpTab));
+    exp_table_kernel<<<kExpTab / 128, 128, 0, c->stream>>>(c->d_exptab);
     count_launch(c);
     IBIM_CUDA(cudaGetLastError());
     IBIM_TRY(f32_chunk_frames(c));  // overwrites d_pos32 with chunk-frame positions

@@ -34,8 +34,7 @@
 namespace ibim {
 
 constexpr int kF64Chunk = 32;
-constexpr int kF64Tab = 512;          // 2^(i/512)
-constexpr int kF64Head = 2 + kF64Tab;  // doubles before the partial slots: item counter, table
+constexpr int kF64Head = 2;  // doubles before the partial slots: the item counter
 // Blocks per side: 160 give about 12,900 items, ten per resident warp, with
 // partial sums of 160 x 16 bytes per node.
 constexpr int64_t kF64Blocks = 160;
@@ -80,24 +79,6 @@ __device__ __forceinline__ F64Node f64_load(const double2* __restrict__ src, int
     const double2* p = src + chunk * (4 * kF64Chunk) + lane;
     const double2 v0 = p[0], v1 = p[kF64Chunk], v2 = p[2 * kF64Chunk], v3 = p[3 * kF64Chunk];
     return F64Node{v0.x, v0.y, v1.x, v1.y, v2.x, v2.y, v3.x, v3.y};
-}
-
-// e^-x for x >= 0: x = -(k ln2/512 + u), |u| <= ln2/1024, e^u by its Taylor
-// series to u^4 (the next term is below 2^-59), 2^(k/512) from the table and
-// the exponent field.  x is held at 700 (e^-x < 1e-304 there).
-__device__ __forceinline__ double exp_neg64(double x, const double* __restrict__ tab)
-{
-    const double xc = __double2hiint(x) > 0x4085e000 ? 700.0 : x;
-    // round(-x 512/ln2) sits in the low word of the sum with 1.5 2^52
-    const double t = fma(xc, -738.6598609351493, 6755399441055744.0);
-    const int k = __double2loint(t);
-    const double kf = t - 6755399441055744.0;
-    double u = fma(kf, -0.0013538030871131923, -xc);  // ln2/512 in two parts, the first of 32 bits
-    u = fma(kf, 8.204912251330243e-14, u);
-    const double p = fma(u * u, fma(u, fma(u, 1.0 / 24.0, 1.0 / 6.0), 0.5), u);
-    const double T = tab[k & (kF64Tab - 1)];
-    const double s = __hiloint2double(__double2hiint(T) + (k >> 9) * 1048576, __double2loint(T));
-    return fma(s, p, s);
 }
 
 // One unordered pair: forward (target T <- source s) into f1, f2, reverse
@@ -167,11 +148,11 @@ __device__ __forceinline__ void f64_chunk_pair(const F64Node& T, double ra, doub
 
 __global__ void __launch_bounds__(128, 4)
     pair_f64_kernel(const double2* __restrict__ src, const float4* __restrict__ frames, F64Plan p, F64Consts k,
-                    double* __restrict__ part, const int* __restrict__ skip)
+                    const double* __restrict__ exptab, double* __restrict__ part, const int* __restrict__ skip)
 {
     if (skip != nullptr && *skip) return;
-    __shared__ double tab[kF64Tab];
-    for (int q = threadIdx.x; q < kF64Tab; q += blockDim.x) tab[q] = part[2 + q];
+    __shared__ double tab[kExpTab];
+    for (int q = threadIdx.x; q < kExpTab; q += blockDim.x) tab[q] = exptab[q];
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -218,14 +199,13 @@ __global__ void __launch_bounds__(128, 4)
 }
 
 // Payload of the chunk-padded node range (past N: the last node's position and
-// normal with zero weights), the table and the cleared item counter.
+// normal with zero weights) and the cleared item counter.
 __global__ void pack_f64_kernel(const double* __restrict__ geo, VecRef in, int64_t N, int64_t n_pad,
                                 double2* __restrict__ src, double* __restrict__ part, const int* __restrict__ skip)
 {
     if (skip != nullptr && *skip) return;
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j == 0) *reinterpret_cast<unsigned long long*>(part) = 0ull;
-    if (j < kF64Tab) part[2 + j] = exp2((double)j * (1.0 / kF64Tab));
     if (j >= n_pad) return;
     const double* p = in.base + (in.kidx ? (int64_t)(*in.kidx + in.koff) * in.stride : 0);
     const int64_t i = j < N ? j : N - 1;
@@ -297,7 +277,7 @@ ibim_status f64_apply(ibim_ctx* c, const PairConsts& k, VecRef in, OutRef out, c
     const F64Plan p = f64_plan(N);
     const int64_t n_pad = p.n_chunks * kF64Chunk;
     const int bs = 256;
-    pack_f64_kernel<<<(unsigned)((std::max<int64_t>(n_pad, kF64Tab) + bs - 1) / bs), bs, 0, c->stream>>>(
+    pack_f64_kernel<<<(unsigned)((n_pad + bs - 1) / bs), bs, 0, c->stream>>>(
         c->d_geo64, in, N, n_pad, (double2*)c->d_src, c->d_part64, d_skip);
     F64Consts kk;
     kk.th1 = k.th1;
@@ -318,7 +298,8 @@ ibim_status f64_apply(ibim_ctx* c, const PairConsts& k, VecRef in, OutRef out, c
     const int64_t cap = (int64_t)std::max(1, occ) * c->num_sms, per = threads / 32;
     const unsigned grid = (unsigned)std::min<int64_t>(cap, (p.items + per - 1) / per);
     IBIM_TRY(timing_begin(c));
-    pair_f64_kernel<<<grid, threads, 0, c->stream>>>((const double2*)c->d_src, c->d_frames, p, kk, c->d_part64, d_skip);
+    pair_f64_kernel<<<grid, threads, 0, c->stream>>>((const double2*)c->d_src, c->d_frames, p, kk, c->d_exptab,
+                                                      c->d_part64, d_skip);
     IBIM_TRY(timing_end(c, N * N));
     fixup_f64_kernel<<<(unsigned)((N + kF64Nodes - 1) / kF64Nodes), kF64Parts * kF64Nodes, 0, c->stream>>>(
         c->d_part64, p, N, k.lambda1, k.lambda2, in, out, d_skip);
