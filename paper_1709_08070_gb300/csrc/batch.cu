@@ -14,8 +14,9 @@
 //                       same arithmetic as the single-molecule kernel; tile
 //                       sums are added to the molecule's output in FP64
 //                       (atomic adds: the few CTAs sharing a target tile)
-//   per molecule        CGS2 orthogonalisation, normalisation and Givens
-//                       (the single-molecule kernels, skipped once done)
+//   gs_kernel, scale    CGS2 orthogonalisation, Givens and normalisation of every
+//                       molecule by the single-molecule kernels (one grid row per
+//                       molecule, skipped once done): four launches a round
 // Molecules that converge drop out of the plan, so later rounds only spend
 // time on the molecules still iterating.
 #include <string.h>
@@ -585,6 +586,8 @@ struct BatchRun {
     BatchMol* d_mols = nullptr;
     BatchPlan* d_plan = nullptr;
     int* d_want = nullptr;
+    GmSys* d_sys = nullptr;
+    int max_nblk = 0, max_C = 0;
     cudaStream_t bs = nullptr;
     cudaGraphExec_t exec = nullptr;
     int variant = 0;
@@ -604,6 +607,7 @@ struct BatchRun {
         cudaFree(d_mols);
         cudaFree(d_plan);
         cudaFree(d_want);
+        cudaFree(d_sys);
         if (bs) cudaStreamDestroy(bs);
     }
 };
@@ -685,6 +689,7 @@ ibim_status batch_solve(int nmol, ibim_ctx* const* ctxs, const ibim_phys* phys, 
     IBIM_CUDA(cudaStreamCreateWithFlags(&R.bs, cudaStreamNonBlocking));
     std::vector<cudaStream_t> user(nmol);
     std::vector<BatchMol> h(nmol);
+    std::vector<GmSys> sys(nmol);
     std::vector<double> gnorm(nmol, 0.0);
     int64_t maxN = 0;
     int sms = ctxs[0]->num_sms;
@@ -738,12 +743,17 @@ ibim_status batch_solve(int nmol, ibim_ctx* const* ctxs, const ibim_phys* phys, 
         b.lambda1 = pk.lambda1;
         b.lambda2 = pk.lambda2;
         b.g64 = Geo64{c->d_geo64, c->d_geo64 + 3 * c->N, 1, c->N};
+        sys[i] = c->gm->sys;
+        R.max_nblk = std::max(R.max_nblk, sys[i].nblk);
+        R.max_C = std::max(R.max_C, sys[i].C);
         maxN = std::max(maxN, c->N);
     }
     IBIM_CUDA(cudaMalloc((void**)&R.d_mols, sizeof(BatchMol) * nmol));
     IBIM_CUDA(cudaMalloc((void**)&R.d_plan, sizeof(BatchPlan)));
     IBIM_CUDA(cudaMalloc((void**)&R.d_want, sizeof(int) * nmol));
     IBIM_CUDA(cudaMemcpyAsync(R.d_mols, h.data(), sizeof(BatchMol) * nmol, cudaMemcpyHostToDevice, R.bs));
+    IBIM_CUDA(cudaMalloc((void**)&R.d_sys, sizeof(GmSys) * nmol));
+    IBIM_CUDA(cudaMemcpyAsync(R.d_sys, sys.data(), sizeof(GmSys) * nmol, cudaMemcpyHostToDevice, R.bs));
     R.sms = sms;
     double sum_n2 = 0.0;
     for (int i = 0; i < nmol; ++i) sum_n2 += (double)ctxs[i]->N * (double)ctxs[i]->N;
@@ -822,10 +832,9 @@ ibim_status batch_solve(int nmol, ibim_ctx* const* ctxs, const ibim_phys* phys, 
             const int64_t before = ctxs[0]->timing.total_launches;
             IBIM_CUDA(cudaStreamBeginCapture(R.bs, cudaStreamCaptureModeThreadLocal));
             ibim_status s = batch_operator(ctxs[0], R, 0);
-            for (int i = 0; i < nmol && s == IBIM_OK; ++i) s = gm_ortho(ctxs[i]);
+            if (s == IBIM_OK) s = gm_ortho_batch(R.d_sys, nmol, R.max_nblk, R.max_C, R.bs);
             cudaError_t e = cudaStreamEndCapture(R.bs, &graph);
             ctxs[0]->timing.total_launches = before;
-            for (int i = 1; i < nmol; ++i) ctxs[i]->timing.total_launches -= 9;
             if (s != IBIM_OK) {
                 if (graph) cudaGraphDestroy(graph);
                 return s;
@@ -837,7 +846,7 @@ ibim_status batch_solve(int nmol, ibim_ctx* const* ctxs, const ibim_phys* phys, 
         }
         for (int round = 0; round <= kMaxRestart + 2; ++round) {
             IBIM_CUDA(cudaGraphLaunch(R.exec, R.bs));
-            count_launch(ctxs[0], 3 + 9 * nmol);
+            count_launch(ctxs[0], 3 + kOrthoLaunches);
             if (round % 2 == 1 || round == kMaxRestart + 2) {
                 for (int i = 0; i < nmol; ++i) IBIM_TRY(gm_fetch_state(ctxs[i]));
                 IBIM_CUDA(cudaStreamSynchronize(R.bs));

@@ -5,10 +5,11 @@
 // k from a device-resident state, so the same sequence can be captured once
 // into a CUDA graph and replayed for every step:
 //   pack/pairs/fixup        w = A v_k                       (operator of the chosen precision)
-//   dots, reduce, update    classical Gram-Schmidt, twice   (CGS2)
-//   norm reduce, scale      v_{k+1} = w / ||w||
-//   givens                  rotate column k of H, update the residual estimate,
-//                           set `done` on convergence / end of cycle
+//   gs_kernel<0>            dots h = V^T w                  (classical Gram-Schmidt,
+//   gs_kernel<1>            w -= V h, dots again             twice: CGS2)
+//   gs_kernel<2>            w -= V h, ||w||, then Givens: rotate column k of H, update
+//                           the residual estimate, set `done` on convergence / end of cycle
+//   scale                   v_{k+1} = w / ||w||
 // Every launch first reads `done` and returns at once when it is set, so the
 // host can replay a few steps ahead and poll the flag only occasionally.
 //
@@ -31,147 +32,291 @@ namespace ibim {
 
 // ------------------------------------------------------------ vector kernels
 
-// part[b * (k+1) + j] = sum over this block's elements of V_j . V_{k+1}, j <= k
-__global__ void __launch_bounds__(kVecThreads)
-    gs_dots_kernel(const double* __restrict__ V, int64_t len, const GmState* __restrict__ st,
-                   double* __restrict__ part)
+// Column k of H by one block: earlier rotations (one serial chain, from shared
+// memory), new rotation, residual estimate |e_{k+1}|, end-of-cycle flags.
+__device__ void givens_column(GmState* __restrict__ st, double hn)
 {
-    if (st->done) return;
-    __shared__ double red[kVecThreads / 32][kMaxRestart + 1];
-    const int k = st->k;
-    const double* w = V + (int64_t)(k + 1) * len;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int j = 0; j <= k; ++j) {
-        const double* v = V + (int64_t)j * len;
-        double s = 0.0;
-        for (int64_t i = (int64_t)blockIdx.x * kVecThreads + threadIdx.x; i < len; i += (int64_t)gridDim.x * kVecThreads)
-            s += v[i] * w[i];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        if (lane == 0) red[warp][j] = s;
-    }
+    __shared__ double h[kMaxRestart + 1], cs[kMaxRestart], sn[kMaxRestart];
+    const int k = st->k, m = st->m;
     __syncthreads();
-    for (int j = threadIdx.x; j <= k; j += kVecThreads) {
-        double s = 0.0;
-        for (int q = 0; q < kVecThreads / 32; ++q) s += red[q][j];
-        part[(int64_t)blockIdx.x * (kMaxRestart + 1) + j] = s;
+    for (int j = threadIdx.x; j <= k; j += blockDim.x) h[j] = __ldcg(st->hcol + j);
+    for (int j = threadIdx.x; j < k; j += blockDim.x) {
+        cs[j] = st->cs[j];
+        sn[j] = st->sn[j];
     }
-}
-
-// coef[j] = sum_b part[b][j]; hcol[j] (+)= coef[j]  (pass 0 sets, pass 1 adds).
-// One warp per coefficient: lane l sums blocks l, l + 32, ..., then a fixed
-// butterfly (the same order every time, so the step is deterministic).
-__global__ void __launch_bounds__(256)
-    gs_reduce_kernel(const double* __restrict__ part, int nblk, GmState* __restrict__ st, int pass)
-{
-    if (st->done) return;
-    const int k = st->k;
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int j = threadIdx.x >> 5; j <= k; j += nw) {
-        double s = 0.0;
-        for (int b = lane; b < nblk; b += 32) s += part[(int64_t)b * (kMaxRestart + 1) + j];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) {
-            st->coef[j] = s;
-            st->hcol[j] = (pass == 0) ? s : st->hcol[j] + s;
-        }
-    }
-}
-
-// V_{k+1} -= sum_j coef[j] V_j; optional per-block partial of ||V_{k+1}||^2 into part[b * (m+1) + 0]
-__global__ void __launch_bounds__(kVecThreads)
-    gs_update_kernel(double* __restrict__ V, int64_t len, const GmState* __restrict__ st,
-                     double* __restrict__ part, int with_norm)
-{
-    if (st->done) return;
-    __shared__ double coef[kMaxRestart + 1];
-    __shared__ double red[kVecThreads / 32];
-    const int k = st->k;
-    for (int j = threadIdx.x; j <= k; j += kVecThreads) coef[j] = st->coef[j];
-    __syncthreads();
-    double* w = V + (int64_t)(k + 1) * len;
-    double nn = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * kVecThreads + threadIdx.x; i < len; i += (int64_t)gridDim.x * kVecThreads) {
-        double s = w[i];
-        for (int j = 0; j <= k; ++j) s -= coef[j] * V[(int64_t)j * len + i];
-        w[i] = s;
-        nn += s * s;
-    }
-    if (!with_norm) return;
-    for (int o = 16; o > 0; o >>= 1) nn += __shfl_down_sync(0xffffffffu, nn, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = nn;
     __syncthreads();
     if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int q = 0; q < kVecThreads / 32; ++q) s += red[q];
-        part[(int64_t)blockIdx.x * (kMaxRestart + 1)] = s;
+        double a = h[0];
+        for (int j = 0; j < k; ++j) {
+            const double b = h[j + 1];
+            h[j] = cs[j] * a + sn[j] * b;
+            a = -sn[j] * a + cs[j] * b;
+        }
+        const double rr = hypot(a, hn);
+        const double c = (rr > 0.0) ? a / rr : 1.0;
+        const double s = (rr > 0.0) ? hn / rr : 0.0;
+        h[k] = rr;
+        st->hn = hn;
+        st->cs[k] = c;
+        st->sn[k] = s;
+        const double e = st->e[k];
+        st->e[k + 1] = -s * e;
+        st->e[k] = c * e;
+        const double resid = fabs(s * e);
+        st->resid = resid;
+        st->k = k + 1;
+        const bool conv = resid <= st->target;
+        if (conv) st->conv = 1;
+        if (conv || k + 1 >= st->kmax || !(hn > 0.0)) st->done = 1;
     }
-}
-
-__global__ void norm_reduce_kernel(const double* __restrict__ part, int nblk, GmState* __restrict__ st)
-{
-    if (st->done) return;
-    __shared__ double red[256];
-    double s = 0.0;
-    for (int b = threadIdx.x; b < nblk; b += blockDim.x) s += part[(int64_t)b * (kMaxRestart + 1)];
-    red[threadIdx.x] = s;
     __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) st->hn = sqrt(red[0]);
+    for (int j = threadIdx.x; j <= k; j += blockDim.x) st->H[j * m + k] = h[j];
+    if (threadIdx.x == 0) st->H[(k + 1) * m + k] = 0.0;
 }
 
-__global__ void scale_kernel(double* __restrict__ V, int64_t len, const GmState* __restrict__ st)
+constexpr int kUpdateLoads = 4;  // element pairs a thread of the update has in flight
+constexpr int kWarps = kVecThreads / 32;
+
+// A pair of basis elements; volatile keeps a batch of these loads together
+// ahead of the arithmetic (left to itself the compiler holds two or three).
+__device__ __forceinline__ double2 load_pair(const double* p)
 {
-    if (st->done) return;
-    const double hn = st->hn;
+    double2 v;
+    asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+    return v;
+}
+
+__device__ __forceinline__ double load_one(const double* p)
+{
+    double v;
+    asm volatile("ld.global.nc.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+
+// One pass of the orthogonalisation of w = V_{k+1} against V_0..V_k.
+//   PASS 0: h = V^T w;  1: w -= V h, then h2 = V^T w (hcol = h + h2);
+//   2: w -= V h2, ||w||, then the Givens step (givens_column).
+// A block owns C consecutive elements of every vector (vectors have even
+// length, so they are read in pairs).  Update: one pair per thread; when C/2 is
+// below the block size, the threads of a pair share the basis vectors.  Dots:
+// a warp takes kDotGroup basis vectors over a slice of the block's elements and
+// reduces their sums together, 9 adds instead of 40 (an FP64 add is as dear as
+// a multiply: the FP64 pipe, 2 lanes per clock and SM, bounds these kernels
+// once the vectors are long, L2 latency before that); while there are fewer
+// groups than warps, the warps of a group share the elements.  The last block
+// to finish a group adds the blocks' partials in a fixed order, so no reduction
+// launch lies between the passes.  gridDim.y systems at once (batched solves).
+// Measured per Arnoldi step (dots twice, updates twice, norm, Givens, scaling):
+// 58 us at 75k elements and 32 vectors on average (117 us as nine launches with
+// one block-wide reduction per dot product and one thread for the Givens
+// column), 28 us at 10k elements (41 us), 56 us at 160k and 8 vectors (58 us),
+// and 106 us for eight molecules of 27k to 46k elements together (456 us as nine
+// launches per molecule).  Sixteen-byte loads in the dots (128 registers, half
+// the warps) were 8 % faster for one system and 14 % slower for eight.
+template <int PASS>
+__global__ void __launch_bounds__(kVecThreads, 4) gs_kernel(GmSys one, const GmSys* __restrict__ many)
+{
+    const GmSys S = many != nullptr ? many[blockIdx.y] : one;
+    GmState* st = S.st;
+    if ((int)blockIdx.x >= S.nblk || st->done) return;
+    constexpr int STRIDE = kMaxRestart + 1;
+    extern __shared__ double2 sw[];  // the block's elements of w
+    __shared__ double coef[kMaxRestart + 1 + kUpdateLoads];
+    __shared__ double2 share[kVecThreads];
+    __shared__ double dsum[kWarps][kMaxRestart + kDotGroup];
+    __shared__ double red[kWarps];
+    __shared__ int last;
+    const int k = st->k, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t base = (int64_t)blockIdx.x * S.C, len = S.len;
+    const int pairs = (int)(len - base < S.C ? len - base : S.C) / 2;
+    const double* V = S.V + base;
+    double2* w = reinterpret_cast<double2*>(S.V + (int64_t)(k + 1) * len + base);
+    double nn = 0.0;
+    if (PASS == 0) {
+        for (int i = tid; i < pairs; i += kVecThreads) sw[i] = w[i];
+    } else {
+        for (int j = tid; j <= k + kUpdateLoads; j += kVecThreads) coef[j] = j <= k ? st->coef[j] : 0.0;
+        __syncthreads();
+        // nh threads per pair, thread h of a pair takes the vectors h, h + nh, ... in batches
+        const int P = S.C / 2, nh = P < kVecThreads ? kVecThreads / P : 1;
+        const int h = nh > 1 ? tid / P : 0, i0 = nh > 1 ? tid - h * P : tid;
+        for (int i = i0; i < P; i += kVecThreads) {  // (one round when nh > 1)
+            double sx = 0.0, sy = 0.0;
+            if (h < nh && i < pairs)
+                for (int j0 = h * kUpdateLoads; j0 <= k; j0 += nh * kUpdateLoads) {
+                    double2 v[kUpdateLoads];  // past k: the last vector again, with weight 0
+#pragma unroll
+                    for (int q = 0; q < kUpdateLoads; ++q) v[q] = load_pair(V + (int64_t)min(j0 + q, k) * len + 2 * i);
+#pragma unroll
+                    for (int q = 0; q < kUpdateLoads; ++q) {
+                        sx = fma(coef[j0 + q], v[q].x, sx);
+                        sy = fma(coef[j0 + q], v[q].y, sy);
+                    }
+                }
+            if (nh > 1) {
+                share[tid] = make_double2(sx, sy);
+                __syncthreads();
+                if (h == 0)
+                    for (int q = 1; q < nh; ++q) {
+                        sx += share[q * P + i].x;
+                        sy += share[q * P + i].y;
+                    }
+            }
+            if (h == 0 && i < pairs) {
+                double2 x = w[i];
+                x.x -= sx;
+                x.y -= sy;
+                w[i] = x;
+                if (PASS == 2) nn = fma(x.x, x.x, fma(x.y, x.y, nn));
+                else sw[i] = x;
+            }
+        }
+    }
+    if (PASS < 2) {
+        __syncthreads();
+        const int ng = k / kDotGroup + 1;
+        const int ns = ng >= kWarps ? 1 : ng > kWarps / 2 ? 1 : ng > kWarps / 4 ? 2 : ng > 1 ? 4 : 8;
+        const int slice = warp % ns;
+        const int i0 = pairs * slice / ns, i1 = pairs * (slice + 1) / ns;
+        for (int g = warp / ns; g < ng; g += kWarps / ns) {
+            double acc[kDotGroup];
+            const double* row[kDotGroup];
+#pragma unroll
+            for (int q = 0; q < kDotGroup; ++q) {
+                acc[q] = 0.0;
+                row[q] = V + (int64_t)min(g * kDotGroup + q, k) * len;  // past k: repeats, not used
+            }
+            const double* ws = reinterpret_cast<const double*>(sw);
+            for (int i = 2 * i0 + lane; i < 2 * i1; i += 32) {
+                double v[kDotGroup];
+#pragma unroll
+                for (int q = 0; q < kDotGroup; ++q) v[q] = load_one(row[q] + i);
+                const double x = ws[i];
+#pragma unroll
+                for (int q = 0; q < kDotGroup; ++q) acc[q] = fma(v[q], x, acc[q]);
+            }
+            // eight sums over 32 lanes: halve the values with the lanes, 4 + 2 + 1 adds, then two more
+#pragma unroll
+            for (int h = kDotGroup / 2, o = 16; h > 0; h >>= 1, o >>= 1) {
+                const bool up = lane & o;
+#pragma unroll
+                for (int q = 0; q < kDotGroup / 2; ++q)
+                    if (q < h) {
+                        const double give = up ? acc[q] : acc[q + h], keep = up ? acc[q + h] : acc[q];
+                        acc[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                    }
+            }
+            double v = acc[0];
+            v += __shfl_xor_sync(0xffffffffu, v, 2);
+            v += __shfl_xor_sync(0xffffffffu, v, 1);
+            if ((lane & 3) == 0) dsum[slice][g * kDotGroup + (lane >> 2)] = v;
+        }
+        __syncthreads();
+        for (int g = warp; g < ng; g += kWarps) {
+            const int j = g * kDotGroup + (lane >> 2);  // four lanes per dot product
+            if ((lane & 3) == 0 && j <= k) {
+                double v = dsum[0][j];
+                for (int q = 1; q < ns; ++q) v += dsum[q][j];
+                S.part[(int64_t)blockIdx.x * STRIDE + j] = v;
+            }
+            __threadfence();
+            __syncwarp();
+            int t = 0;
+            if (lane == 0) t = atomicAdd(&st->dot_ticket[g], 1);
+            if (__shfl_sync(0xffffffffu, t, 0) != S.nblk - 1) continue;
+            __threadfence();
+            double s = 0.0;
+            if (j <= k) {
+                for (int b = lane & 3; b < S.nblk; b += 64) {
+                    double p[16];
+#pragma unroll
+                    for (int q = 0; q < 16; ++q)
+                        p[q] = b + 4 * q < S.nblk ? __ldcg(S.part + (int64_t)(b + 4 * q) * STRIDE + j) : 0.0;
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) s += p[q];
+                }
+            }
+            s += __shfl_xor_sync(0xffffffffu, s, 2);
+            s += __shfl_xor_sync(0xffffffffu, s, 1);
+            if ((lane & 3) == 0 && j <= k) {
+                st->coef[j] = s;
+                st->hcol[j] = PASS == 0 ? s : st->hcol[j] + s;
+            }
+            if (lane == 0) st->dot_ticket[g] = 0;
+        }
+        return;
+    }
+    for (int o = 16; o > 0; o >>= 1) nn += __shfl_down_sync(0xffffffffu, nn, o);
+    if (lane == 0) red[warp] = nn;
+    __syncthreads();
+    if (tid == 0) {
+        double s = 0.0;
+        for (int q = 0; q < kWarps; ++q) s += red[q];
+        S.part[(int64_t)blockIdx.x * STRIDE] = s;
+        __threadfence();
+        last = atomicAdd(&st->norm_ticket, 1) == S.nblk - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double s = 0.0;
+    for (int b = tid; b < S.nblk; b += kVecThreads) s += __ldcg(S.part + (int64_t)b * STRIDE);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    __syncthreads();
+    if (lane == 0) red[warp] = s;
+    __syncthreads();
+    s = 0.0;
+    for (int q = 0; q < kWarps; ++q) s += red[q];
+    if (tid == 0) st->norm_ticket = 0;
+    givens_column(st, sqrt(s));
+}
+
+// v_{k+1} = w / ||w|| (after the Givens step: st->k is the new vector's index)
+__global__ void __launch_bounds__(kVecThreads) scale_kernel(GmSys one, const GmSys* __restrict__ many)
+{
+    const GmSys S = many != nullptr ? many[blockIdx.y] : one;
+    if ((int)blockIdx.x >= S.nblk || S.st->done) return;
+    const double hn = S.st->hn;
     if (!(hn > 0.0)) return;
     const double inv = 1.0 / hn;
-    double* w = V + (int64_t)(st->k + 1) * len;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x)
-        w[i] *= inv;
+    const int64_t base = (int64_t)blockIdx.x * S.C;
+    const int cnt = (int)(S.len - base < S.C ? S.len - base : S.C);
+    double* w = S.V + (int64_t)S.st->k * S.len + base;
+    for (int i = threadIdx.x; i < cnt; i += kVecThreads) w[i] *= inv;
 }
 
-// Column k of H: earlier rotations, new rotation, residual estimate |e_{k+1}|.
-__global__ void givens_kernel(GmState* __restrict__ st)
+// Back substitution H y = e (k x k upper triangular) by one block, column by
+// column: the thread of row i forms y_i, the rows above subtract its column.
+// The columns are staged in shared memory, so a step costs a division and a
+// barrier (k = 64: 32 us; 177 us by one thread reading H from global memory).
+__global__ void __launch_bounds__(kMaxRestart) trisolve_kernel(GmState* __restrict__ st)
 {
-    if (st->done) return;
-    const int k = st->k, m = st->m;
-    double* H = st->H;
-    for (int j = 0; j <= k; ++j) H[j * m + k] = st->hcol[j];
-    const double hn = st->hn;
-    H[(k + 1) * m + k] = hn;
-    for (int j = 0; j < k; ++j) {
-        const double a = H[j * m + k], b = H[(j + 1) * m + k];
-        H[j * m + k] = st->cs[j] * a + st->sn[j] * b;
-        H[(j + 1) * m + k] = -st->sn[j] * a + st->cs[j] * b;
-    }
-    const double a = H[k * m + k], b = H[(k + 1) * m + k];
-    const double rr = hypot(a, b);
-    const double c = (rr > 0.0) ? a / rr : 1.0;
-    const double s = (rr > 0.0) ? b / rr : 0.0;
-    st->cs[k] = c;
-    st->sn[k] = s;
-    H[k * m + k] = rr;
-    H[(k + 1) * m + k] = 0.0;
-    st->e[k + 1] = -s * st->e[k];
-    st->e[k] = c * st->e[k];
-    st->resid = fabs(st->e[k + 1]);
-    st->k = k + 1;
-    if (st->resid <= st->target) st->conv = 1;
-    if (st->conv || st->k >= st->kmax || !(hn > 0.0)) st->done = 1;
-}
-
-// Back substitution H y = e (k x k upper triangular), then nothing else.
-__global__ void trisolve_kernel(GmState* __restrict__ st)
-{
-    const int k = st->k, m = st->m;
+    extern __shared__ double U[];  // column i at i (i + 1) / 2
+    __shared__ double y;
+    const int k = st->k, m = st->m, t = threadIdx.x;
+#pragma unroll 8
+    for (int i = 0; i < k; ++i)
+        if (t <= i) U[i * (i + 1) / 2 + t] = st->H[t * m + i];
+    double e = t < k ? st->e[t] : 0.0;
+    __syncthreads();
     for (int i = k - 1; i >= 0; --i) {
-        double s = st->e[i];
-        for (int j = i + 1; j < k; ++j) s -= st->H[i * m + j] * st->y[j];
-        st->y[i] = s / st->H[i * m + i];
+        if (t == i) {
+            y = e / U[i * (i + 1) / 2 + i];
+            st->y[i] = y;
+        }
+        __syncthreads();
+        if (t < i) e -= U[i * (i + 1) / 2 + t] * y;
+        __syncthreads();
     }
+}
+
+constexpr size_t kTriSmem = sizeof(double) * kMaxRestart * (kMaxRestart + 1) / 2;
+
+static ibim_status trisolve_launch(GmState* st, cudaStream_t stream)
+{
+    IBIM_CUDA(cudaFuncSetAttribute(trisolve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTriSmem));
+    trisolve_kernel<<<1, kMaxRestart, kTriSmem, stream>>>(st);
+    return IBIM_OK;
 }
 
 // x += sum_{j<k} y_j V_j
@@ -184,6 +329,7 @@ __global__ void xupdate_kernel(double* __restrict__ x, const double* __restrict_
     __syncthreads();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x) {
         double s = x[i];
+#pragma unroll 8
         for (int j = 0; j < k; ++j) s += y[j] * V[(int64_t)j * len + i];
         x[i] = s;
     }
@@ -305,29 +451,52 @@ ibim_status gm_alloc(ibim_ctx* c, int m)
     IBIM_CUDA(cudaMalloc((void**)&w->g, sizeof(double) * len));
     IBIM_CUDA(cudaMalloc((void**)&w->xb, sizeof(double) * len));
     IBIM_CUDA(cudaMalloc((void**)&w->gin, sizeof(double) * len));
-    IBIM_CUDA(cudaMalloc((void**)&w->part, sizeof(double) * (size_t)w->nblk * (kMaxRestart + 1)));
+    // blocks of C = 128, 256, ... elements: at most 320 of them (two per SM), so
+    // that the last warp of a group adds few partials, until a block's elements
+    // of w no longer fit shared memory (2.6 million nodes)
+    w->sys.len = len;
+    w->sys.C = 128;
+    while (w->sys.C < 16384 && len > 320 * (int64_t)w->sys.C) w->sys.C *= 2;
+    w->sys.nblk = (int)((len + w->sys.C - 1) / w->sys.C);
+    IBIM_CUDA(cudaMalloc((void**)&w->part,
+                         sizeof(double) * (size_t)std::max(w->nblk, w->sys.nblk) * (kMaxRestart + 1)));
     IBIM_CUDA(cudaMalloc((void**)&w->st, sizeof(GmState)));
+    w->sys.V = w->V;
+    w->sys.st = w->st;
+    w->sys.part = w->part;
     IBIM_CUDA(cudaMallocHost((void**)&w->h_st, sizeof(GmState)));
     IBIM_CUDA(cudaStreamCreateWithFlags(&w->gs, cudaStreamNonBlocking));
     IBIM_CUDA(cudaEventCreateWithFlags(&w->ev, cudaEventDisableTiming));
     return IBIM_OK;
 }
 
-ibim_status gm_ortho(ibim_ctx* c)
+static ibim_status ortho_launch(const GmSys& one, const GmSys* many, int nsys, int nblk, int C, cudaStream_t stream)
 {
-    GmresWork* w = c->gm;
-    const int64_t len = w->len;
-    for (int pass = 0; pass < 2; ++pass) {
-        gs_dots_kernel<<<w->nblk, kVecThreads, 0, c->stream>>>(w->V, len, w->st, w->part);
-        gs_reduce_kernel<<<1, 256, 0, c->stream>>>(w->part, w->nblk, w->st, pass);
-        gs_update_kernel<<<w->nblk, kVecThreads, 0, c->stream>>>(w->V, len, w->st, w->part, pass == 1);
+    const dim3 grid((unsigned)nblk, (unsigned)nsys);
+    const size_t smem = sizeof(double) * C;
+    if (smem > 40 * 1024) {
+        IBIM_CUDA(cudaFuncSetAttribute(gs_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        IBIM_CUDA(cudaFuncSetAttribute(gs_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     }
-    norm_reduce_kernel<<<1, 256, 0, c->stream>>>(w->part, w->nblk, w->st);
-    scale_kernel<<<w->nblk, kVecThreads, 0, c->stream>>>(w->V, len, w->st);
-    givens_kernel<<<1, 1, 0, c->stream>>>(w->st);
-    count_launch(c, 9);
+    gs_kernel<0><<<grid, kVecThreads, smem, stream>>>(one, many);
+    gs_kernel<1><<<grid, kVecThreads, smem, stream>>>(one, many);
+    gs_kernel<2><<<grid, kVecThreads, 0, stream>>>(one, many);
+    scale_kernel<<<grid, kVecThreads, 0, stream>>>(one, many);
     IBIM_CUDA(cudaGetLastError());
     return IBIM_OK;
+}
+
+ibim_status gm_ortho(ibim_ctx* c)
+{
+    const GmSys& S = c->gm->sys;
+    IBIM_TRY(ortho_launch(S, nullptr, 1, S.nblk, S.C, c->stream));
+    count_launch(c, kOrthoLaunches);
+    return IBIM_OK;
+}
+
+ibim_status gm_ortho_batch(const GmSys* d_sys, int nsys, int max_nblk, int max_C, cudaStream_t stream)
+{
+    return ortho_launch(GmSys{}, d_sys, nsys, max_nblk, max_C, stream);
 }
 
 // One Arnoldi step (see the file comment), all launches on c->stream.
@@ -357,7 +526,7 @@ ibim_status gm_cycle_begin(ibim_ctx* c, bool x_zero, double target, int kmax)
 ibim_status gm_cycle_end(ibim_ctx* c)
 {
     GmresWork* w = c->gm;
-    trisolve_kernel<<<1, 1, 0, c->stream>>>(w->st);
+    IBIM_TRY(trisolve_launch(w->st, c->stream));
     xupdate_kernel<<<w->nblk, kVecThreads, 0, c->stream>>>(w->x, w->V, w->len, w->st);
     count_launch(c, 2);
     IBIM_CUDA(cudaGetLastError());
@@ -462,7 +631,7 @@ static ibim_status run_cycle(ibim_ctx* c, const PairConsts& k, int precision, bo
                     return IBIM_ERR_STATE;
                 }
                 IBIM_CUDA(cudaGraphLaunch(w->exec, c->stream));
-                count_launch(c, 12);  // kernels in one captured step
+                count_launch(c, 3 + kOrthoLaunches);  // kernels in one captured step
             } else {
                 IBIM_TRY(arnoldi_step(c, k, precision));
             }
@@ -621,7 +790,7 @@ ibim_status gmres_solve(ibim_ctx* c, const ibim_phys& p, const ibim_solve_opts& 
         info->matvecs_f32 += (prec_in == IBIM_F32C || prec_in == IBIM_F32T) ? steps : 0;
         info->matvecs_f64 += (prec_in == IBIM_F64 || prec_in == IBIM_FF) ? steps : 0;
         if (steps > 0) {
-            trisolve_kernel<<<1, 1, 0, c->stream>>>(w->st);
+            IBIM_TRY(trisolve_launch(w->st, c->stream));
             xupdate_kernel<<<w->nblk, kVecThreads, 0, c->stream>>>(w->x, w->V, len, w->st);
             count_launch(c, 2);
             IBIM_CUDA(cudaGetLastError());
