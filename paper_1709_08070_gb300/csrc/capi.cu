@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "ibim_internal.cuh"
+#include "math64.cuh"
 
 namespace ibim {
 
@@ -233,7 +234,9 @@ static ibim_status ctx_new(void* stream, ibim_ctx** out)
     c->stream = (cudaStream_t)stream;
     cudaError_t e = cudaGetDevice(&c->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_err, sizeof(unsigned));
+    // the error word and, behind it, the table of exp_neg64 (written with the geometry)
+    if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_err, 16 + sizeof(double) * kExpTab);
+    if (e == cudaSuccess) c->d_exptab = reinterpret_cast<double*>(c->d_err + 4);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_err, 0, sizeof(unsigned), c->stream);
     if (e != cudaSuccess) {
         ibim_destroy(c);
@@ -292,7 +295,6 @@ void ibim_destroy(ibim_ctx* c)
     cudaFree(c->d_src);
     cudaFree(c->d_part);
     cudaFree(c->d_part64);
-    cudaFree(c->d_exptab);
     cudaFree(c->d_red);
     cudaFree(c->d_err);
     cudaFree(c->d_io);

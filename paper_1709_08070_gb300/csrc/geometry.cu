@@ -58,6 +58,7 @@ __device__ __forceinline__ bool sphere_node(const SphereBox& B, uint64_t code, d
     return true;
 }
 
+static_assert(kPadNodes >= kExpTab, "one thread per table entry");
 constexpr int kCompactBlock = 1024;
 
 __global__ void __launch_bounds__(kCompactBlock) sphere_count_kernel(SphereBox B, uint64_t ncodes, int* __restrict__ counts)
@@ -194,11 +195,13 @@ ibim_status build_sphere_nodes(ibim_ctx* c, double R, const double* centre, cons
 
 // FP32 copies of the geometry over the padded node range (positions relative
 // to the centroid; the chunk-frame pass replaces them), placeholder normals
-// past N.
+// past N; and the table of exp_neg64.
 __global__ void pack_geometry_f32_kernel(const double* __restrict__ geo, int64_t N, int64_t n_pad, double c0,
-                                         double c1, double c2, float4* __restrict__ pos, float4* __restrict__ nrm)
+                                         double c1, double c2, float4* __restrict__ pos, float4* __restrict__ nrm,
+                                         double* __restrict__ exptab)
 {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < kExpTab) exptab[j] = exp2((double)j * (1.0 / kExpTab));  // n_pad >= kExpTab
     if (j >= n_pad) return;
     if (j >= N) {
         pos[j] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -333,12 +336,6 @@ static ibim_status compact_order(ibim_ctx* c)
     return IBIM_OK;
 }
 
-__global__ void exp_table_kernel(double* __restrict__ tab)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < kExpTab) tab[i] = exp2((double)i * (1.0 / kExpTab));
-}
-
 ibim_status finish_geometry(ibim_ctx* c, bool reorder)
 {
     if (reorder) IBIM_TRY(compact_order(c));
@@ -353,11 +350,8 @@ ibim_status finish_geometry(ibim_ctx* c, bool reorder)
     IBIM_CUDA(cudaMalloc((void**)&c->d_nrm32, sizeof(float4) * n_pad));
     const int bs = 256;
     pack_geometry_f32_kernel<<<(unsigned)((n_pad + bs - 1) / bs), bs, 0, c->stream>>>(
-        c->d_geo64, N, n_pad, c->centroid[0], c->centroid[1], c->centroid[2], c->d_pos32, c->d_nrm32);
-    count_launch(c);
-    IBIM_CUDA(cudaGetLastError());
-    IBIM_CUDA(cudaMalloc((void**)&c->d_exptab, sizeof(double) * kExpTab));
-    exp_table_kernel<<<kExpTab / 128, 128, 0, c->stream>>>(c->d_exptab);
+        c->d_geo64, N, n_pad, c->centroid[0], c->centroid[1], c->centroid[2], c->d_pos32, c->d_nrm32,
+        c->d_exptab);
     count_launch(c);
     IBIM_CUDA(cudaGetLastError());
     IBIM_TRY(f32_chunk_frames(c));  // overwrites d_pos32 with chunk-frame positions

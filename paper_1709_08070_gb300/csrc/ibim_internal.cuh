@@ -133,7 +133,7 @@ struct ibim_ctx {
     size_t src_bytes = 0;
     double* d_part = nullptr;  // stream-K partial sums
     size_t part_bytes = 0;
-    double* d_exptab = nullptr;  // 2^(i/512) for exp_neg64 (math64.cuh), made with the geometry
+    double* d_exptab = nullptr;  // 2^(i/512) for exp_neg64 (math64.cuh): behind d_err, written with the geometry
     double* d_part64 = nullptr;  // FP64 path: item counter, partial sums of the block pairs
     size_t part64_bytes = 0;
     double* d_red = nullptr;   // small reduction scratch (energy, area, norms)
