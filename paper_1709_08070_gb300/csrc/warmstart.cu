@@ -40,8 +40,12 @@ constexpr int kOffB2 = kOffW2 + kWsH * kWsH;
 constexpr int kOffW3 = kOffB2 + kWsH;
 constexpr int kOffB3 = kOffW3 + kWsOut * kWsH;
 constexpr int kWsParams = kOffB3 + kWsOut;  // 4930
-constexpr int kWsThreads = 128;             // nodes per training block
+constexpr int kWsThreads = 128;             // prediction: nodes per block
 constexpr int kHPad = kWsH + 1;             // padded smem row (bank conflicts)
+constexpr int kTrainThreads = 256;
+constexpr int kTrainNodes = 64;             // training: nodes per tile
+constexpr int kTrainRow = kTrainNodes + 4;  // row of a transposed tile (16-byte aligned, rows four banks apart)
+constexpr int kPartStride = kWsParams + 2;  // a CTA's gradient, 16-byte aligned
 
 static_assert(kWsParams == IBIM_WS_NPARAMS, "parameter count");
 
@@ -54,8 +58,9 @@ struct ibim_wsnet {
     __nv_bfloat16* d_wb = nullptr;  // BF16 parameters used by the kernels
     float* d_m = nullptr;           // Adam first moment
     float* d_v = nullptr;           // Adam second moment
-    float* d_g = nullptr;           // gradient accumulator
-    double* d_loss = nullptr;
+    float* d_g = nullptr;           // gradient, then the training CTAs' partial gradients
+    double* d_loss = nullptr;       // loss, then the training CTAs' partial losses
+    int num_sms = 0;
     double* d_scal = nullptr;       // S1, S2 scratch
     float* d_feat = nullptr;        // training features (n_ex x 8)
     float* d_tgt = nullptr;         // training targets (n_ex x 2)
@@ -205,111 +210,249 @@ __device__ __forceinline__ uint64_t mix64(uint64_t z)
     return z ^ (z >> 31);
 }
 
-// Loss and gradient over a batch: node of slot (block, thread) is either
-// consecutive (first + slot, full-batch mode) or drawn at random.
-__global__ void __launch_bounds__(kWsThreads)
-    ws_grad_kernel(const float* __restrict__ feat, const float* __restrict__ tgt, const float* __restrict__ wt,
-                   int64_t n_ex, int64_t first, int64_t count, int random, uint64_t seed, double inv_batch,
-                   const __nv_bfloat16* __restrict__ wb, float* __restrict__ grad, double* __restrict__ loss)
+// Shared memory of the training kernel (floats).
+struct TrainSmem {
+    float W1T[kWsIn][kWsH];          // [input][unit]
+    float W2[kWsH][kWsH];            // [unit 2][unit 1]
+    float W2T[kWsH][kWsH];           // [unit 1][unit 2]
+    float W3[kWsOut][kWsH];
+    float b1[kWsH], b2[kWsH], b3[kWsOut + 2];
+    float X[kWsIn][kTrainRow];       // activations transposed: [unit][node]
+    float H1[kWsH][kTrainRow];
+    float H2[kWsH][kTrainRow];       // then d2
+    float D1[kWsH][kTrainRow];
+    float dO[kWsOut][kTrainRow];
+    float e[kWsOut][kTrainRow];
+    float wt[kTrainNodes], tgt[kWsOut][kTrainNodes];
+    double loss[kTrainNodes];
+};
+
+// acc[i][j] = sum_k A[k][4 ty + i] B[k][4 tx + j] on top of acc's start values, k ascending.
+template <int K, int LDA, int LDB>
+__device__ __forceinline__ void tile_product(const float (*A)[LDA], const float (*B)[LDB], int ty, int tx,
+                                             float (&acc)[4][4])
 {
-    extern __shared__ float smem[];
-    float* sp = smem;                               // params
-    float* X = sp + kWsParams;                      // [128][kWsIn]
-    float* H1 = X + kWsThreads * kWsIn;             // [128][kHPad]
-    float* H2 = H1 + kWsThreads * kHPad;
-    float* D1 = H2 + kWsThreads * kHPad;
-    float* D2 = D1 + kWsThreads * kHPad;
-    float* DO = D2 + kWsThreads * kHPad;            // [128][2]
-    __shared__ double lred[kWsThreads];
-    load_params(wb, sp);
-    __syncthreads();
-    const int t = threadIdx.x;
-    const int64_t slot = (int64_t)blockIdx.x * kWsThreads + t;
-    const bool live = slot < count;
-    float* x = X + t * kWsIn;
-    float* h1 = H1 + t * kHPad;
-    float* h2 = H2 + t * kHPad;
-    float* d1 = D1 + t * kHPad;
-    float* d2 = D2 + t * kHPad;
-    float* dO = DO + t * kWsOut;
-    double l = 0.0;
-    if (live) {
-        const int64_t i = random ? (int64_t)(mix64(seed ^ (uint64_t)slot) % (uint64_t)n_ex) : first + slot;
-        for (int b = 0; b < kWsIn; ++b) x[b] = feat[i * kWsIn + b];
-        float o[kWsOut];
-        ws_forward(sp, x, h1, h2, o);
-        const float w = wt[i];
-        const float e0 = o[0] - tgt[2 * i], e1 = o[1] - tgt[2 * i + 1];
-        l = (double)w * ((double)e0 * e0 + (double)e1 * e1) * inv_batch;
-        dO[0] = (float)(2.0 * inv_batch) * w * e0;
-        dO[1] = (float)(2.0 * inv_batch) * w * e1;
-        for (int a = 0; a < kWsH; ++a) {
-            float s = 0.0f;
-            for (int c = 0; c < kWsOut; ++c) s = fmaf(sp[kOffW3 + c * kWsH + a], dO[c], s);
-            d2[a] = s * (1.0f - h2[a] * h2[a]);
-        }
-        for (int b = 0; b < kWsH; ++b) {
-            float s = 0.0f;
-            for (int a = 0; a < kWsH; ++a) s = fmaf(sp[kOffW2 + a * kWsH + b], d2[a], s);
-            d1[b] = s * (1.0f - h1[b] * h1[b]);
-        }
-    } else {
-        for (int b = 0; b < kWsIn; ++b) x[b] = 0.0f;
-        for (int a = 0; a < kWsH; ++a) h1[a] = h2[a] = d1[a] = d2[a] = 0.0f;
-        dO[0] = dO[1] = 0.0f;
+#pragma unroll 4
+    for (int k = 0; k < K; ++k) {
+        const float4 a = *reinterpret_cast<const float4*>(&A[k][4 * ty]);
+        const float4 b = *reinterpret_cast<const float4*>(&B[k][4 * tx]);
+        const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(bv[j], av[i], acc[i][j]);
     }
-    lred[t] = l;
-    __syncthreads();
-    // weight gradients: contractions over the block's nodes
-    for (int e = t; e < kWsH * kWsH; e += kWsThreads) {  // dW2[a][b] = sum_n d2[n][a] h1[n][b]
-        const int a = e / kWsH, b = e % kWsH;
-        float s = 0.0f;
-        for (int n = 0; n < kWsThreads; ++n) s = fmaf(D2[n * kHPad + a], H1[n * kHPad + b], s);
-        atomicAdd(grad + kOffW2 + e, s);
-    }
-    for (int e = t; e < kWsH * kWsIn; e += kWsThreads) {  // dW1[a][b] = sum_n d1[n][a] x[n][b]
-        const int a = e / kWsIn, b = e % kWsIn;
-        float s = 0.0f;
-        for (int n = 0; n < kWsThreads; ++n) s = fmaf(D1[n * kHPad + a], X[n * kWsIn + b], s);
-        atomicAdd(grad + kOffW1 + e, s);
-    }
-    for (int e = t; e < kWsOut * kWsH; e += kWsThreads) {  // dW3[c][a] = sum_n dO[n][c] h2[n][a]
-        const int c = e / kWsH, a = e % kWsH;
-        float s = 0.0f;
-        for (int n = 0; n < kWsThreads; ++n) s = fmaf(DO[n * kWsOut + c], H2[n * kHPad + a], s);
-        atomicAdd(grad + kOffW3 + e, s);
-    }
-    if (t < kWsH) {
-        float s1 = 0.0f, s2 = 0.0f;
-        for (int n = 0; n < kWsThreads; ++n) {
-            s1 += D1[n * kHPad + t];
-            s2 += D2[n * kHPad + t];
-        }
-        atomicAdd(grad + kOffB1 + t, s1);
-        atomicAdd(grad + kOffB2 + t, s2);
-    }
-    if (t < kWsOut) {
-        float s = 0.0f;
-        for (int n = 0; n < kWsThreads; ++n) s += DO[n * kWsOut + t];
-        atomicAdd(grad + kOffB3 + t, s);
-    }
-    for (int o = kWsThreads / 2; o > 0; o >>= 1) {
-        __syncthreads();
-        if (t < o) lred[t] += lred[t + o];
-    }
-    if (t == 0) atomicAdd(loss, lred[0]);
 }
 
-// Adam (Kingma and Ba 2015) on the FP32 master weights; refreshes the BF16 copy.
-__global__ void ws_adam_kernel(float* __restrict__ w, float* __restrict__ m, float* __restrict__ v,
-                               const float* __restrict__ g, __nv_bfloat16* __restrict__ wb, float lr, float b1,
-                               float b2, float c1, float c2)
+__device__ __forceinline__ float dot4(const float4& a, const float4& b, float s)
 {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= kWsParams) return;
-    const float gq = g[q];
-    const float mq = b1 * m[q] + (1.0f - b1) * gq;
-    const float vq = b2 * v[q] + (1.0f - b2) * gq * gq;
+    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, s))));
+}
+
+// Loss and gradient over a batch: node of slot s is either consecutive (first +
+// s, full-batch mode) or drawn at random.  The three 64 x 64 x 64 products of a
+// 64-node tile (layer 2 forward, its backward, its weight gradient) run as
+// register tiles of 4 x 4 per thread from shared memory, activations stored
+// transposed so that every operand is a float4; a CTA takes tiles blockIdx.x,
+// + gridDim.x, ... and keeps its weight gradients in registers, then writes
+// them as its partial gradient (summed in a fixed order by ws_update_kernel).
+// 242 MFLOP at 8,192 nodes: 3 us of the FP32 pipe; measured @GRAD@ (79.5 us
+// with one thread per node over shared-memory rows and FP32 atomics).
+__global__ void __launch_bounds__(kTrainThreads)
+    ws_grad_kernel(const float* __restrict__ feat, const float* __restrict__ tgt, const float* __restrict__ wt,
+                   int64_t n_ex, int64_t first, int64_t count, int random, uint64_t seed, double inv_batch,
+                   const __nv_bfloat16* __restrict__ wb, float* __restrict__ part, double* __restrict__ part_loss)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    TrainSmem& S = *reinterpret_cast<TrainSmem*>(smem_raw);
+    const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
+    for (int q = t; q < kWsH * kWsH; q += kTrainThreads) {
+        const float v = __bfloat162float(wb[kOffW2 + q]);
+        S.W2[q / kWsH][q % kWsH] = v;
+        S.W2T[q % kWsH][q / kWsH] = v;
+    }
+    for (int q = t; q < kWsH * kWsIn; q += kTrainThreads) S.W1T[q % kWsIn][q / kWsIn] = __bfloat162float(wb[kOffW1 + q]);
+    for (int q = t; q < kWsOut * kWsH; q += kTrainThreads) S.W3[q / kWsH][q % kWsH] = __bfloat162float(wb[kOffW3 + q]);
+    if (t < kWsH) {
+        S.b1[t] = __bfloat162float(wb[kOffB1 + t]);
+        S.b2[t] = __bfloat162float(wb[kOffB2 + t]);
+    }
+    if (t < kWsOut) S.b3[t] = __bfloat162float(wb[kOffB3 + t]);
+
+    float gW2[4][4];                              // units ty + 16 i (layer 2) x tx + 16 j (layer 1)
+    float gW1[3] = {0.0f, 0.0f, 0.0f};            // unit t % 64, inputs t / 64 + 4 i; the bias in the last
+    float gW3 = 0.0f, gB2 = 0.0f, gB3 = 0.0f;     // t < 128: W3[t / 64][t % 64]; 128 <= t < 192: b2; t < 2: b3
+    double l = 0.0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) gW2[i][j] = 0.0f;
+
+    for (int64_t tile = blockIdx.x; tile * kTrainNodes < count; tile += gridDim.x) {
+        __syncthreads();
+        // four threads per node fetch its features, target and weight (zeros past the batch)
+        {
+            const int n = t & (kTrainNodes - 1), part4 = t / kTrainNodes;
+            const int64_t slot = tile * kTrainNodes + n;
+            const bool live = slot < count;
+            int64_t i = 0;
+            if (live) i = random ? (int64_t)(mix64(seed ^ (uint64_t)slot) % (uint64_t)n_ex) : first + slot;
+            for (int b = part4; b < kWsIn; b += 4) S.X[b][n] = live ? feat[i * kWsIn + b] : 0.0f;
+            if (part4 == 0) S.wt[n] = live ? wt[i] : 0.0f;
+            if (part4 >= 1 && part4 <= kWsOut) S.tgt[part4 - 1][n] = live ? tgt[kWsOut * i + part4 - 1] : 0.0f;
+        }
+        __syncthreads();
+        float acc[4][4];  // nodes 4 ty + i, units 4 tx + j
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = S.b1[4 * tx + j];
+        tile_product<kWsIn>(S.X, S.W1T, ty, tx, acc);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            *reinterpret_cast<float4*>(&S.H1[4 * tx + j][4 * ty]) =
+                make_float4(tanhf(acc[0][j]), tanhf(acc[1][j]), tanhf(acc[2][j]), tanhf(acc[3][j]));
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = S.b2[4 * tx + j];
+        tile_product<kWsH>(S.H1, S.W2T, ty, tx, acc);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            *reinterpret_cast<float4*>(&S.H2[4 * tx + j][4 * ty]) =
+                make_float4(tanhf(acc[0][j]), tanhf(acc[1][j]), tanhf(acc[2][j]), tanhf(acc[3][j]));
+        __syncthreads();
+        if (t < kWsOut * kTrainNodes) {  // outputs
+            const int c = t / kTrainNodes, n = t % kTrainNodes;
+            float s = S.b3[c];
+#pragma unroll 8
+            for (int a = 0; a < kWsH; ++a) s = fmaf(S.W3[c][a], S.H2[a][n], s);
+            const float e = tile * kTrainNodes + n < count ? s - S.tgt[c][n] : 0.0f;
+            S.e[c][n] = e;
+            S.dO[c][n] = (float)(2.0 * inv_batch) * S.wt[n] * e;
+        }
+        __syncthreads();
+        if (t < kTrainNodes) {
+            const float w = S.wt[t], e0 = S.e[0][t], e1 = S.e[1][t];
+            l += (double)w * ((double)e0 * e0 + (double)e1 * e1) * inv_batch;
+        }
+        if (t < kWsOut * kWsH) {  // dW3[c][a] += sum_n dO[n][c] h2[n][a]
+            const int c = t / kWsH, a = t % kWsH;
+#pragma unroll 4
+            for (int n = 0; n < kTrainNodes; n += 4)
+                gW3 = dot4(*reinterpret_cast<const float4*>(&S.dO[c][n]), *reinterpret_cast<const float4*>(&S.H2[a][n]), gW3);
+        }
+        if (t < kWsOut)
+            for (int n = 0; n < kTrainNodes; ++n) gB3 += S.dO[t][n];
+        __syncthreads();
+        for (int q = t; q < kWsH * kTrainNodes; q += kTrainThreads) {  // d2 in the place of h2
+            const int a = q / kTrainNodes, n = q % kTrainNodes;
+            const float h = S.H2[a][n];
+            float s = fmaf(S.W3[0][a], S.dO[0][n], 0.0f);
+            s = fmaf(S.W3[1][a], S.dO[1][n], s);
+            S.H2[a][n] = s * (1.0f - h * h);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
+        tile_product<kWsH>(S.H2, S.W2, ty, tx, acc);  // d1 before the derivative of tanh
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float4 h = *reinterpret_cast<const float4*>(&S.H1[4 * tx + j][4 * ty]);
+            *reinterpret_cast<float4*>(&S.D1[4 * tx + j][4 * ty]) =
+                make_float4(acc[0][j] * (1.0f - h.x * h.x), acc[1][j] * (1.0f - h.y * h.y),
+                            acc[2][j] * (1.0f - h.z * h.z), acc[3][j] * (1.0f - h.w * h.w));
+        }
+#pragma unroll 2
+        for (int n = 0; n < kTrainNodes; n += 4) {  // dW2[a][b] += sum_n d2[n][a] h1[n][b]
+            float4 d[4], h[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                d[i] = *reinterpret_cast<const float4*>(&S.H2[ty + 16 * i][n]);
+                h[i] = *reinterpret_cast<const float4*>(&S.H1[tx + 16 * i][n]);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) gW2[i][j] = dot4(d[i], h[j], gW2[i][j]);
+        }
+        if (t >= 2 * kWsH && t < 3 * kWsH)
+            for (int n = 0; n < kTrainNodes; ++n) gB2 += S.H2[t - 2 * kWsH][n];
+        __syncthreads();
+        {  // dW1[a][b] += sum_n d1[n][a] x[n][b], the bias as one more input
+            const int a = t % kWsH, b0 = t / kWsH;
+#pragma unroll 4
+            for (int n = 0; n < kTrainNodes; n += 4) {
+                const float4 d = *reinterpret_cast<const float4*>(&S.D1[a][n]);
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    const int b = b0 + 4 * i;
+                    if (b < kWsIn) gW1[i] = dot4(d, *reinterpret_cast<const float4*>(&S.X[b][n]), gW1[i]);
+                    else if (b == kWsIn) gW1[i] += (d.x + d.y) + (d.z + d.w);
+                }
+            }
+        }
+    }
+
+    float* g = part + (int64_t)blockIdx.x * kPartStride;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) g[kOffW2 + (ty + 16 * i) * kWsH + tx + 16 * j] = gW2[i][j];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int a = t % kWsH, b = t / kWsH + 4 * i;
+        if (b < kWsIn) g[kOffW1 + a * kWsIn + b] = gW1[i];
+        else if (b == kWsIn) g[kOffB1 + a] = gW1[i];
+    }
+    if (t < kWsOut * kWsH) g[kOffW3 + t] = gW3;
+    if (t >= 2 * kWsH && t < 3 * kWsH) g[kOffB2 + t - 2 * kWsH] = gB2;
+    if (t < kWsOut) g[kOffB3 + t] = gB3;
+    if (t < kTrainNodes) S.loss[t] = l;
+    for (int o = kTrainNodes / 2; o > 0; o >>= 1) {
+        __syncthreads();
+        if (t < o) S.loss[t] += S.loss[t + o];
+    }
+    if (t == 0) part_loss[blockIdx.x] = S.loss[0];
+}
+
+// Sums the CTAs' partial gradients (kSumParts threads per parameter over fixed
+// shares) and losses; with adam, one Adam step (Kingma and Ba 2015) on the FP32
+// master weights, which refreshes the BF16 copy; else the gradient goes to grad.
+constexpr int kSumParts = 8, kSumParams = 32;
+__global__ void __launch_bounds__(kSumParts * kSumParams)
+    ws_update_kernel(const float* __restrict__ part, const double* __restrict__ part_loss, int nparts, int adam,
+                     float* __restrict__ w, float* __restrict__ m, float* __restrict__ v, __nv_bfloat16* __restrict__ wb,
+                     float lr, float b1, float b2, float c1, float c2, float* __restrict__ grad,
+                     double* __restrict__ loss)
+{
+    __shared__ float sh[kSumParts][kSumParams];
+    const int ql = threadIdx.x % kSumParams, pr = threadIdx.x / kSumParams;
+    const int q = blockIdx.x * kSumParams + ql;
+    float s = 0.0f;
+    if (q < kWsParams) {
+#pragma unroll 8
+        for (int p = pr; p < nparts; p += kSumParts) s += part[(int64_t)p * kPartStride + q];
+    }
+    sh[pr][ql] = s;
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
+        double d = 0.0;
+        for (int p = threadIdx.x; p < nparts; p += 32) d += part_loss[p];
+        for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+        if (threadIdx.x == 0) *loss = d;
+    }
+    __syncthreads();
+    if (pr != 0 || q >= kWsParams) return;
+    for (int p = 1; p < kSumParts; ++p) s += sh[p][ql];
+    if (!adam) {
+        grad[q] = s;
+        return;
+    }
+    const float mq = b1 * m[q] + (1.0f - b1) * s;
+    const float vq = b2 * v[q] + (1.0f - b2) * s * s;
     m[q] = mq;
     v[q] = vq;
     const float wq = w[q] - lr * (mq / c1) / (sqrtf(vq / c2) + 1e-8f);
@@ -323,7 +466,15 @@ __global__ void ws_to_bf16_kernel(const float* __restrict__ w, __nv_bfloat16* __
     if (q < kWsParams) wb[q] = __float2bfloat16_rn(w[q]);
 }
 
-static size_t grad_smem() { return sizeof(float) * (kWsParams + kWsThreads * (kWsIn + 4 * kHPad + kWsOut)); }
+static size_t grad_smem() { return sizeof(TrainSmem); }
+// CTAs of a training launch: one per SM, each over its share of the tiles
+static unsigned grad_ctas(const ibim_wsnet* n, int64_t count)
+{
+    return (unsigned)std::min<int64_t>(n->num_sms, (count + kTrainNodes - 1) / kTrainNodes);
+}
+// the partial gradients behind the gradient, the partial losses behind the loss
+static float* grad_parts(const ibim_wsnet* n) { return n->d_g + kPartStride; }
+static double* loss_parts(const ibim_wsnet* n) { return n->d_loss + 2; }
 static size_t predict_smem() { return sizeof(float) * (kWsParams + kWsThreads * 2 * kHPad); }
 
 // Features (into c->d_io as floats after the RHS) and scales of one context.
@@ -419,8 +570,9 @@ ibim_status ibim_wsnet_create(uint64_t seed, void* stream, ibim_wsnet** out)
     if (e == cudaSuccess) e = cudaMalloc((void**)&n->d_wb, sizeof(__nv_bfloat16) * kWsParams);
     if (e == cudaSuccess) e = cudaMalloc((void**)&n->d_m, sizeof(float) * kWsParams);
     if (e == cudaSuccess) e = cudaMalloc((void**)&n->d_v, sizeof(float) * kWsParams);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&n->d_g, sizeof(float) * kWsParams);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&n->d_loss, sizeof(double));
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n->num_sms, cudaDevAttrMultiProcessorCount, n->device);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&n->d_g, sizeof(float) * kPartStride * (1 + (size_t)n->num_sms));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&n->d_loss, sizeof(double) * (2 + (size_t)n->num_sms));
     if (e == cudaSuccess) e = cudaMalloc((void**)&n->d_scal, sizeof(double) * 4);
     if (e == cudaSuccess) e = cudaMemcpyAsync(n->d_w, w.data(), sizeof(float) * kWsParams, cudaMemcpyHostToDevice, n->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(n->d_m, 0, sizeof(float) * kWsParams, n->stream);
@@ -555,12 +707,13 @@ ibim_status ibim_wsnet_gradient(ibim_wsnet* n, int64_t first, int64_t count, dou
         set_error("need a net and 0 <= first, first + count <= number of examples, count >= 1");
         return IBIM_ERR_ARG;
     }
-    IBIM_CUDA(cudaMemsetAsync(n->d_g, 0, sizeof(float) * kWsParams, n->stream));
-    IBIM_CUDA(cudaMemsetAsync(n->d_loss, 0, sizeof(double), n->stream));
-    const unsigned blocks = (unsigned)((count + kWsThreads - 1) / kWsThreads);
-    ws_grad_kernel<<<blocks, kWsThreads, grad_smem(), n->stream>>>(n->d_feat, n->d_tgt, n->d_wt, n->n_ex, first, count,
-                                                                   0, 0, 1.0 / (double)count, n->d_wb, n->d_g,
-                                                                   n->d_loss);
+    const unsigned ctas = grad_ctas(n, count);
+    ws_grad_kernel<<<ctas, kTrainThreads, grad_smem(), n->stream>>>(n->d_feat, n->d_tgt, n->d_wt, n->n_ex, first, count,
+                                                                    0, 0, 1.0 / (double)count, n->d_wb, grad_parts(n),
+                                                                    loss_parts(n));
+    ws_update_kernel<<<(kWsParams + kSumParams - 1) / kSumParams, kSumParts * kSumParams, 0, n->stream>>>(
+        grad_parts(n), loss_parts(n), (int)ctas, 0, n->d_w, n->d_m, n->d_v, n->d_wb, 0.0f, 0.0f, 0.0f, 1.0f, 1.0f,
+        n->d_g, n->d_loss);
     IBIM_CUDA(cudaGetLastError());
     IBIM_CUDA(cudaMemcpyAsync(h_grad, n->d_g, sizeof(float) * kWsParams, cudaMemcpyDeviceToHost, n->stream));
     IBIM_CUDA(cudaMemcpyAsync(loss, n->d_loss, sizeof(double), cudaMemcpyDeviceToHost, n->stream));
@@ -578,19 +731,18 @@ ibim_status ibim_wsnet_train(ibim_wsnet* n, int steps, int batch_nodes, double l
         set_error("no training examples");
         return IBIM_ERR_STATE;
     }
-    const unsigned blocks = (unsigned)((batch_nodes + kWsThreads - 1) / kWsThreads);
+    const unsigned ctas = grad_ctas(n, batch_nodes);
     const double b1 = 0.9, b2 = 0.999;
     for (int s = 0; s < steps; ++s) {
         ++n->step;
-        IBIM_CUDA(cudaMemsetAsync(n->d_g, 0, sizeof(float) * kWsParams, n->stream));
-        IBIM_CUDA(cudaMemsetAsync(n->d_loss, 0, sizeof(double), n->stream));
         const uint64_t sd = n->seed * 0x9e3779b97f4a7c15ull + (uint64_t)n->step * 0xd1b54a32d192ed03ull;
-        ws_grad_kernel<<<blocks, kWsThreads, grad_smem(), n->stream>>>(n->d_feat, n->d_tgt, n->d_wt, n->n_ex, 0,
-                                                                       batch_nodes, 1, sd, 1.0 / (double)batch_nodes,
-                                                                       n->d_wb, n->d_g, n->d_loss);
+        ws_grad_kernel<<<ctas, kTrainThreads, grad_smem(), n->stream>>>(n->d_feat, n->d_tgt, n->d_wt, n->n_ex, 0,
+                                                                        batch_nodes, 1, sd, 1.0 / (double)batch_nodes,
+                                                                        n->d_wb, grad_parts(n), loss_parts(n));
         const float c1 = (float)(1.0 - pow(b1, (double)n->step)), c2 = (float)(1.0 - pow(b2, (double)n->step));
-        ws_adam_kernel<<<(kWsParams + 255) / 256, 256, 0, n->stream>>>(n->d_w, n->d_m, n->d_v, n->d_g, n->d_wb,
-                                                                       (float)lr, (float)b1, (float)b2, c1, c2);
+        ws_update_kernel<<<(kWsParams + kSumParams - 1) / kSumParams, kSumParts * kSumParams, 0, n->stream>>>(
+            grad_parts(n), loss_parts(n), (int)ctas, 1, n->d_w, n->d_m, n->d_v, n->d_wb, (float)lr, (float)b1, (float)b2,
+            c1, c2, n->d_g, n->d_loss);
         IBIM_CUDA(cudaGetLastError());
     }
     if (last_loss) {
