@@ -111,6 +111,12 @@ __device__ __forceinline__ double rsqrt_approx64(double x)
     return y;
 }
 
+// Programmatic dependent launch: allow the next kernel of the stream to be set
+// up, and wait until the kernel before this one has finished (its writes
+// visible).  Both do nothing in a launch without the attribute.
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ float rsqrt_approx(float x)
 {
     float y;

@@ -29,6 +29,7 @@
 #include <vector>
 
 #include "ibim_internal.cuh"
+#include "ptx.cuh"
 
 namespace ibim {
 
@@ -256,8 +257,11 @@ __device__ __forceinline__ float dot4(const float4& a, const float4& b, float s)
 // transposed so that every operand is a float4; a CTA takes tiles blockIdx.x,
 // + gridDim.x, ... and keeps its weight gradients in registers, then writes
 // them as its partial gradient (summed in a fixed order by ws_update_kernel).
-// 242 MFLOP at 8,192 nodes: 3 us of the FP32 pipe; measured @GRAD@ (79.5 us
-// with one thread per node over shared-memory rows and FP32 atomics).
+// 242 MFLOP at 8,192 nodes: 3 us of the FP32 pipe; bound by the latency of its
+// eight phases.  Measured 20 us a step with the Adam kernel, launches overlapped
+// (27 us before the overlap and the transposed read of W2, whose copy stored
+// with 32-way bank conflicts; 92 us with one thread per node over shared-memory
+// rows, FP32 atomics and two memsets).
 __global__ void __launch_bounds__(kTrainThreads)
     ws_grad_kernel(const float* __restrict__ feat, const float* __restrict__ tgt, const float* __restrict__ wt,
                    int64_t n_ex, int64_t first, int64_t count, int random, uint64_t seed, double inv_batch,
@@ -266,12 +270,33 @@ __global__ void __launch_bounds__(kTrainThreads)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     TrainSmem& S = *reinterpret_cast<TrainSmem*>(smem_raw);
     const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-    for (int q = t; q < kWsH * kWsH; q += kTrainThreads) {
-        const float v = __bfloat162float(wb[kOffW2 + q]);
-        S.W2[q / kWsH][q % kWsH] = v;
-        S.W2T[q % kWsH][q / kWsH] = v;
+    // four threads per node fetch its features, target and weight (zeros past the batch)
+    auto fetch = [&](int64_t tile) {
+        const int n = t & (kTrainNodes - 1), part4 = t / kTrainNodes;
+        const int64_t slot = tile * kTrainNodes + n;
+        const bool live = slot < count;
+        int64_t i = 0;
+        if (live) i = random ? (int64_t)(mix64(seed ^ (uint64_t)slot) % (uint64_t)n_ex) : first + slot;
+        for (int b = part4; b < kWsIn; b += 4) S.X[b][n] = live ? feat[i * kWsIn + b] : 0.0f;
+        if (part4 == 0) S.wt[n] = live ? wt[i] : 0.0f;
+        if (part4 >= 1 && part4 <= kWsOut) S.tgt[part4 - 1][n] = live ? tgt[kWsOut * i + part4 - 1] : 0.0f;
+    };
+    ptx::grid_dep_launch();  // the Adam kernel may be set up; it waits for this grid
+    // this step's first tile of features while the previous Adam step finishes
+    fetch(blockIdx.x);
+    ptx::grid_dep_wait();
+    const __nv_bfloat162* w2 = reinterpret_cast<const __nv_bfloat162*>(wb + kOffW2);
+#pragma unroll 4
+    for (int q = t; q < kWsH * kWsH / 2; q += kTrainThreads) {
+        // once along the rows, once across them, so that neither copy stores with bank conflicts
+        const int r = q / (kWsH / 2), c = q % (kWsH / 2);
+        *reinterpret_cast<float2*>(&S.W2[r][2 * c]) = __bfloat1622float2(w2[q]);
+        const int a = q % kWsH, p = q / kWsH;
+        const float2 v = __bfloat1622float2(w2[a * (kWsH / 2) + p]);
+        S.W2T[2 * p][a] = v.x;
+        S.W2T[2 * p + 1][a] = v.y;
     }
-    for (int q = t; q < kWsH * kWsIn; q += kTrainThreads) S.W1T[q % kWsIn][q / kWsIn] = __bfloat162float(wb[kOffW1 + q]);
+    for (int q = t; q < kWsH * kWsIn; q += kTrainThreads) S.W1T[q / kWsH][q % kWsH] = __bfloat162float(wb[kOffW1 + (q % kWsH) * kWsIn + q / kWsH]);
     for (int q = t; q < kWsOut * kWsH; q += kTrainThreads) S.W3[q / kWsH][q % kWsH] = __bfloat162float(wb[kOffW3 + q]);
     if (t < kWsH) {
         S.b1[t] = __bfloat162float(wb[kOffB1 + t]);
@@ -289,17 +314,9 @@ __global__ void __launch_bounds__(kTrainThreads)
         for (int j = 0; j < 4; ++j) gW2[i][j] = 0.0f;
 
     for (int64_t tile = blockIdx.x; tile * kTrainNodes < count; tile += gridDim.x) {
-        __syncthreads();
-        // four threads per node fetch its features, target and weight (zeros past the batch)
-        {
-            const int n = t & (kTrainNodes - 1), part4 = t / kTrainNodes;
-            const int64_t slot = tile * kTrainNodes + n;
-            const bool live = slot < count;
-            int64_t i = 0;
-            if (live) i = random ? (int64_t)(mix64(seed ^ (uint64_t)slot) % (uint64_t)n_ex) : first + slot;
-            for (int b = part4; b < kWsIn; b += 4) S.X[b][n] = live ? feat[i * kWsIn + b] : 0.0f;
-            if (part4 == 0) S.wt[n] = live ? wt[i] : 0.0f;
-            if (part4 >= 1 && part4 <= kWsOut) S.tgt[part4 - 1][n] = live ? tgt[kWsOut * i + part4 - 1] : 0.0f;
+        if (tile != blockIdx.x) {
+            __syncthreads();
+            fetch(tile);
         }
         __syncthreads();
         float acc[4][4];  // nodes 4 ty + i, units 4 tx + j
@@ -430,6 +447,8 @@ __global__ void __launch_bounds__(kSumParts * kSumParams)
                      double* __restrict__ loss)
 {
     __shared__ float sh[kSumParts][kSumParams];
+    ptx::grid_dep_launch();  // the next step's gradient may be set up; it waits for this grid
+    ptx::grid_dep_wait();
     const int ql = threadIdx.x % kSumParams, pr = threadIdx.x / kSumParams;
     const int q = blockIdx.x * kSumParams + ql;
     float s = 0.0f;
@@ -733,17 +752,33 @@ ibim_status ibim_wsnet_train(ibim_wsnet* n, int steps, int batch_nodes, double l
     }
     const unsigned ctas = grad_ctas(n, batch_nodes);
     const double b1 = 0.9, b2 = 0.999;
+    // Each launch may begin while the one before it ends (programmatic dependent
+    // launch): the kernels wait for it themselves before they touch what it wrote.
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t grad_cfg = {}, sum_cfg = {};
+    grad_cfg.gridDim = dim3(ctas);
+    grad_cfg.blockDim = dim3(kTrainThreads);
+    grad_cfg.dynamicSmemBytes = grad_smem();
+    sum_cfg.gridDim = dim3((kWsParams + kSumParams - 1) / kSumParams);
+    sum_cfg.blockDim = dim3(kSumParts * kSumParams);
+    grad_cfg.stream = sum_cfg.stream = n->stream;
+    grad_cfg.attrs = sum_cfg.attrs = &attr;
+    grad_cfg.numAttrs = sum_cfg.numAttrs = 1;
     for (int s = 0; s < steps; ++s) {
         ++n->step;
         const uint64_t sd = n->seed * 0x9e3779b97f4a7c15ull + (uint64_t)n->step * 0xd1b54a32d192ed03ull;
-        ws_grad_kernel<<<ctas, kTrainThreads, grad_smem(), n->stream>>>(n->d_feat, n->d_tgt, n->d_wt, n->n_ex, 0,
-                                                                        batch_nodes, 1, sd, 1.0 / (double)batch_nodes,
-                                                                        n->d_wb, grad_parts(n), loss_parts(n));
+        // (the first launch of a call follows whatever the stream holds in full)
+        grad_cfg.numAttrs = s > 0 ? 1 : 0;
+        IBIM_CUDA(cudaLaunchKernelEx(&grad_cfg, ws_grad_kernel, (const float*)n->d_feat, (const float*)n->d_tgt,
+                                     (const float*)n->d_wt, n->n_ex, (int64_t)0, (int64_t)batch_nodes, 1, sd,
+                                     1.0 / (double)batch_nodes, (const __nv_bfloat16*)n->d_wb, grad_parts(n),
+                                     loss_parts(n)));
         const float c1 = (float)(1.0 - pow(b1, (double)n->step)), c2 = (float)(1.0 - pow(b2, (double)n->step));
-        ws_update_kernel<<<(kWsParams + kSumParams - 1) / kSumParams, kSumParts * kSumParams, 0, n->stream>>>(
-            grad_parts(n), loss_parts(n), (int)ctas, 1, n->d_w, n->d_m, n->d_v, n->d_wb, (float)lr, (float)b1, (float)b2,
-            c1, c2, n->d_g, n->d_loss);
-        IBIM_CUDA(cudaGetLastError());
+        IBIM_CUDA(cudaLaunchKernelEx(&sum_cfg, ws_update_kernel, (const float*)grad_parts(n),
+                                     (const double*)loss_parts(n), (int)ctas, 1, n->d_w, n->d_m, n->d_v, n->d_wb,
+                                     (float)lr, (float)b1, (float)b2, c1, c2, n->d_g, n->d_loss));
     }
     if (last_loss) {
         IBIM_CUDA(cudaMemcpyAsync(last_loss, n->d_loss, sizeof(double), cudaMemcpyDeviceToHost, n->stream));
