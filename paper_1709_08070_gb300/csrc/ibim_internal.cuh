@@ -209,13 +209,14 @@ size_t f32_part_doubles(ibim_ctx* c);  // partial-sum doubles of the current var
 int sym_variant_count();
 void sym_variant_info(int v, int* tpt, int* minb, int* threads, int* scheme);
 int sym_occupancy(int v);
-size_t sym_part_doubles(int64_t N, int ttile, int grid_cap);
+int sym_stile(int v);  // source tile of symmetric variant v
+size_t sym_part_doubles(int64_t N, int ttile, int stile, int grid_cap);
 size_t sym_yrev_bytes(int64_t N);
 ibim_status sym_pack(ibim_ctx* c, VecRef in, const int* d_skip);
 ibim_status sym_pairs(ibim_ctx* c, int sv, int grid_cap, const PairConsts& k, const int* d_skip);
 ibim_status sym_fixup(ibim_ctx* c, int sv, int grid_cap, const PairConsts& k, VecRef in, OutRef out,
                       const int* d_skip);
-ibim_status sym_fixup_tiles(ibim_ctx* c, int ttile, int grid_cap, const PairConsts& k, VecRef in, OutRef out,
+ibim_status sym_fixup_tiles(ibim_ctx* c, int ttile, int stile, int grid_cap, const PairConsts& k, VecRef in, OutRef out,
                             const int* d_skip);
 PairSchedule f32_schedule(ibim_ctx* c);
 ibim_status f32_chunk_frames(ibim_ctx* c);

@@ -48,7 +48,7 @@
 
 namespace ibim {
 
-template <int TPT, int MINB, int THREADS>
+template <int TPT, int MINB, int THREADS, int STAGES = kF32Stages, bool FLATNEAR = false>
 __global__ void __launch_bounds__(THREADS, MINB)
     pair_f32_kernel(const float4* __restrict__ tpos, const float4* __restrict__ tnrm,
                     const float4* __restrict__ src, const float4* __restrict__ frames, int64_t N, PairSchedule s,
@@ -57,9 +57,9 @@ __global__ void __launch_bounds__(THREADS, MINB)
 {
     constexpr int TTILE = THREADS * TPT;
     constexpr int NW = THREADS / 32;
-    static_assert(TTILE <= kF32MaxTTile, "target tile");
+    static_assert(TTILE <= kF32MaxTTile && STAGES <= kF32Stages, "tile, stages");
     if (skip != nullptr && *skip) return;
-    __shared__ __align__(128) SourceStage stg[kF32Stages];
+    __shared__ __align__(128) SourceStage stg[STAGES];
     __shared__ __align__(16) float4 tfrm[NW][2 * TPT];
     __shared__ __align__(8) StagePipe pipe;
 
@@ -76,12 +76,12 @@ __global__ void __launch_bounds__(THREADS, MINB)
 
     auto issue = [&](int64_t u) {
         const int64_t st = ((u % s.n_stiles) * s.sperm) % s.n_stiles;
-        const int stage = (int)((u - s0) % kF32Stages);
+        const int stage = (int)((u - s0) % STAGES);
         pipe_issue(pipe, stg[stage], stage, src + st * (kF32STile / 2) * kPairF4,
                    have_frames ? frames + st * 2 * kChunksPerTile : nullptr);
     };
     if (tid == 0)
-        for (int q = 0; q < kF32Stages && s0 + q < s1; ++q) issue(s0 + q);
+        for (int q = 0; q < STAGES && s0 + q < s1; ++q) issue(s0 + q);
 
     const int64_t t_first = s0 / s.n_stiles;
     int64_t t = t_first;
@@ -117,8 +117,8 @@ __global__ void __launch_bounds__(THREADS, MINB)
     load_targets(t);
 
     for (int64_t u = s0; u < s1; ++u) {
-        const int stage = (int)((u - s0) % kF32Stages);
-        const uint32_t parity = (uint32_t)(((u - s0) / kF32Stages) & 1);
+        const int stage = (int)((u - s0) % STAGES);
+        const uint32_t parity = (uint32_t)(((u - s0) / STAGES) & 1);
         if (!__all_sync(0xffffffffu, ptx::mbar_wait_bounded(&pipe.full[stage], parity, kWaitLimitNs))) {
             if (lane == 0) atomicOr(err, kDevErrTimeout);
             return;
@@ -129,8 +129,9 @@ __global__ void __launch_bounds__(THREADS, MINB)
 #pragma unroll
         for (int q = 0; q < TPT; ++q) S1[q] = C1[q] = S2[q] = C2[q] = 0.0f;
         if (!idle)
-            tile_sums<TPT>(T, &tfrm[warp][0], have_frames, stg[stage].buf, stg[stage].frm, k, S1, C1, S2, C2, g64,
-                           gi0, THREADS, st * kF32STile, N);
+            tile_sums<TPT, false, kChunksPerTile, FLATNEAR>(T, &tfrm[warp][0], have_frames, stg[stage].buf,
+                                                            stg[stage].frm, k, S1, C1, S2, C2, g64, gi0, THREADS,
+                                                            st * kF32STile, N);
 #pragma unroll
         for (int q = 0; q < TPT; ++q) {
             D1[q] += (double)S1[q] - (double)C1[q];
@@ -138,16 +139,16 @@ __global__ void __launch_bounds__(THREADS, MINB)
         }
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(&pipe.empty[stage]);
-        // thread 0 refills the stage of step u - 1 with step u - 1 + kF32Stages
+        // thread 0 refills the stage of step u - 1 with step u - 1 + STAGES
         if (warp == 0) {
             bool ok = true;
-            if (lane == 0 && u > s0 && u - 1 + kF32Stages < s1) {
+            if (lane == 0 && u > s0 && u - 1 + STAGES < s1) {
                 const int64_t v = u - 1 - s0;
-                ok = ptx::mbar_wait_bounded(&pipe.empty[(int)(v % kF32Stages)], (uint32_t)((v / kF32Stages) & 1),
+                ok = ptx::mbar_wait_bounded(&pipe.empty[(int)(v % STAGES)], (uint32_t)((v / STAGES) & 1),
                                             kWaitLimitNs);
                 if (ok) {
                     ptx::fence_proxy_async_smem();
-                    issue(u - 1 + kF32Stages);
+                    issue(u - 1 + STAGES);
                 } else {
                     atomicOr(err, kDevErrTimeout);
                 }
@@ -239,27 +240,47 @@ __global__ void pack_f32_kernel(const float4* __restrict__ pos, const float4* __
     write_source_pair(src + kPairF4 * pr, y[0], y[1], m[0], m[1], a[0], a[1], b[0], b[1]);
 }
 
-// y = Lambda p + (1/(4 pi)) sum of the partials of every CTA that touched the tile.
-__global__ void fixup_kernel(const double* __restrict__ part, PairSchedule s, int ttile, int64_t N,
-                             double lambda1, double lambda2, VecRef in, OutRef out,
-                             const int* __restrict__ skip)
+// y = Lambda p + (1/(4 pi)) sum of the partials of every CTA that touched the
+// tile.  kFixShares threads per target, each over a fixed share of the CTAs,
+// the shares added in a fixed order: deterministic.  Only the first of a row's
+// CTAs can have begun in an earlier row; in the others the row is segment 0.
+// (3,001 nodes, 47 CTAs a row: 3.8 us; 11.7 us with one thread per target and
+// its divisions per slot.)
+constexpr int kFixShares = 8, kFixNodes = 32;
+__global__ void __launch_bounds__(kFixShares * kFixNodes)
+    fixup_kernel(const double* __restrict__ part, PairSchedule s, int ttile, int64_t N, double lambda1,
+                 double lambda2, VecRef in, OutRef out, const int* __restrict__ skip)
 {
     if (skip != nullptr && *skip) return;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const double* p = in.base + (in.kidx ? (int64_t)(*in.kidx + in.koff) * in.stride : 0);
-    double* y = out.base + (out.kidx ? (int64_t)(*out.kidx + out.koff) * out.stride : 0);
-    const int64_t t = i / ttile;
+    __shared__ double sh[2][kFixShares][kFixNodes];
+    const int tl = threadIdx.x % kFixNodes, pr = threadIdx.x / kFixNodes;
+    const int64_t i = (int64_t)blockIdx.x * kFixNodes + tl;
+    // kFixNodes divides every target tile: a block lies in one row
+    const int64_t t = (int64_t)blockIdx.x * kFixNodes / ttile;
     const int64_t l = i - t * ttile;
     const int64_t c0 = (t * s.n_stiles) / s.per_cta;
-    const int64_t c1 = ((t + 1) * s.n_stiles - 1) / s.per_cta;
+    const int64_t n = ((t + 1) * s.n_stiles - 1) / s.per_cta - c0 + 1;
     double a1 = 0.0, a2 = 0.0;
-    for (int64_t c = c0; c <= c1; ++c) {
-        const int64_t seg = t - (c * s.per_cta) / s.n_stiles;
-        const double* src = part + (c * s.max_segs + seg) * 2 * ttile;
-        a1 += src[l];
-        a2 += src[ttile + l];
+    if (i < N) {
+        const int64_t seg0 = t - (c0 * s.per_cta) / s.n_stiles, stride = 2 * (int64_t)s.max_segs * ttile;
+        const double* base = part + c0 * stride + l;
+#pragma unroll 4
+        for (int64_t c = n * pr / kFixShares; c < n * (pr + 1) / kFixShares; ++c) {
+            const double* src = base + c * stride + (c == 0 ? seg0 * 2 * ttile : 0);
+            a1 += src[0];
+            a2 += src[ttile];
+        }
     }
+    sh[0][pr][tl] = a1;
+    sh[1][pr][tl] = a2;
+    __syncthreads();
+    if (pr != 0 || i >= N) return;
+    for (int q = 1; q < kFixShares; ++q) {
+        a1 += sh[0][q][tl];
+        a2 += sh[1][q][tl];
+    }
+    const double* p = in.base + (in.kidx ? (int64_t)(*in.kidx + in.koff) * in.stride : 0);
+    double* y = out.base + (out.kidx ? (int64_t)(*out.kidx + out.koff) * out.stride : 0);
     y[i] = lambda1 * p[i] + kInv4Pi * a1;
     y[N + i] = lambda2 * p[N + i] + kInv4Pi * a2;
 }
@@ -279,11 +300,11 @@ struct PairArgs {
     Geo64 g64;
 };
 
-template <int TPT, int MINB, int THREADS>
+template <int TPT, int MINB, int THREADS, int STAGES = kF32Stages, bool FLATNEAR = false>
 static void launch_variant(const PairArgs& a, cudaStream_t stream)
 {
-    pair_f32_kernel<TPT, MINB, THREADS><<<a.s.grid, THREADS, 0, stream>>>(a.tpos, a.tnrm, a.src, a.frames, a.N, a.s,
-                                                                          a.k, a.part, a.err, a.skip, a.g64);
+    pair_f32_kernel<TPT, MINB, THREADS, STAGES, FLATNEAR><<<a.s.grid, THREADS, 0, stream>>>(
+        a.tpos, a.tnrm, a.src, a.frames, a.N, a.s, a.k, a.part, a.err, a.skip, a.g64);
 }
 
 struct F32Variant {
@@ -298,6 +319,17 @@ static const F32Variant kVariants[] = {
     IBIM_F32_VARIANT(1, 1, 512),
 };
 #undef IBIM_F32_VARIANT
+// Small launches of variant 0, the choice of a context that was not tuned:
+// below kSmallSteps steps of its own kernel (about 15,000 nodes) they run
+// 64-target tiles, four times as many steps, so that the chip is filled, and the
+// branch-free near formula, as most chunk pairs are near.  The source tiles,
+// within which a target's sums are compensated, stay the same, and with them
+// the result.  Jittered-sphere clouds, own kernel against this one:
+// 300 nodes 67.5 / 33.5 us, 3,001 70.5 / 34.7, 5,000 94.7 / 62.3, 8,000 165 / 127,
+// 12,000 279 / 233; at 17,000 the two meet.
+constexpr int64_t kSmallSteps = 3600;
+static const F32Variant kSmallVariant = {1, 8, 64, (const void*)pair_f32_kernel<1, 8, 64, 2, true>,
+                                         launch_variant<1, 8, 64, 2, true>};
 constexpr int kNumVariants = (int)(sizeof(kVariants) / sizeof(kVariants[0]));
 
 // Variants kNumVariants.. are the symmetric kernel's (pair_sym.cu).
@@ -319,18 +351,31 @@ void f32_variant_info(int v, int* tpt, int* minb, int* threads, int* symmetric)
     *symmetric = 0;
 }
 
-static int occupancy_of(int v)
+// The one-directional kernel that variant v runs on N nodes.
+static bool runs_small(int v, int64_t N)
 {
-    if (is_sym(v)) return sym_occupancy(v - kNumVariants);
+    if (v != 0) return false;
+    const int64_t tt = kVariants[0].tpt * kVariants[0].threads;
+    return ((N + tt - 1) / tt) * ((N + kF32STile - 1) / kF32STile) < kSmallSteps;
+}
+static const F32Variant& one_directional(const ibim_ctx* c)
+{
+    return runs_small(c->f32_variant, c->N) ? kSmallVariant : kVariants[c->f32_variant];
+}
+
+static int occupancy_of(const F32Variant& k)
+{
     int occ = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kVariants[v].fn, kVariants[v].threads, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k.fn, k.threads, 0);
     return occ < 1 ? 1 : occ;
 }
 
-int f32_max_bps(int v) { return occupancy_of(v); }
+int f32_max_bps(int v) { return is_sym(v) ? sym_occupancy(v - kNumVariants) : occupancy_of(kVariants[v]); }
 
+// Target tile of the context's FP32 kernel.
 int f32_ttile(const ibim_ctx* c)
 {
+    if (!is_sym(c->f32_variant)) return one_directional(c).threads * one_directional(c).tpt;
     int tpt, minb, threads, sym;
     f32_variant_info(c->f32_variant, &tpt, &minb, &threads, &sym);
     return threads * tpt;
@@ -338,7 +383,7 @@ int f32_ttile(const ibim_ctx* c)
 
 int f32_grid_cap(ibim_ctx* c)
 {
-    const int occ = occupancy_of(c->f32_variant);
+    const int occ = is_sym(c->f32_variant) ? f32_max_bps(c->f32_variant) : occupancy_of(one_directional(c));
     const int bps = (c->f32_bps > 0 && c->f32_bps < occ) ? c->f32_bps : occ;
     return bps * c->num_sms;
 }
@@ -346,8 +391,8 @@ int f32_grid_cap(ibim_ctx* c)
 // Partial-sum doubles the current variant needs.
 size_t f32_part_doubles(ibim_ctx* c)
 {
-    if (is_sym(c->f32_variant)) return sym_part_doubles(c->N, f32_ttile(c), f32_grid_cap(c));
-    const PairSchedule s = make_schedule(c->N, f32_ttile(c), c->N, kF32STile, f32_grid_cap(c));
+    if (is_sym(c->f32_variant)) return sym_part_doubles(c->N, f32_ttile(c), sym_stile(c->f32_variant - kNumVariants), f32_grid_cap(c));
+    const PairSchedule s = f32_schedule(c);
     return (size_t)s.grid * s.max_segs * 2 * f32_ttile(c);
 }
 
@@ -391,7 +436,7 @@ ibim_status f32_pairs(ibim_ctx* c, const PairConsts& k, const PairSchedule& s, c
     if (is_sym(c->f32_variant)) return sym_pairs(c, c->f32_variant - kNumVariants, f32_grid_cap(c), k, d_skip);
     const PairArgs a{c->d_pos32, c->d_nrm32, (const float4*)c->d_src, c->d_frames, c->N, s, f32_consts(k),
                      c->d_part, c->d_err, d_skip, Geo64{c->d_geo64, c->d_geo64 + 3 * c->N, 1, c->N}};
-    kVariants[c->f32_variant].launch(a, c->stream);
+    one_directional(c).launch(a, c->stream);
     count_launch(c);
     IBIM_CUDA(cudaGetLastError());
     return IBIM_OK;
@@ -400,8 +445,7 @@ ibim_status f32_pairs(ibim_ctx* c, const PairConsts& k, const PairSchedule& s, c
 ibim_status fixup_launch(ibim_ctx* c, const PairConsts& k, const PairSchedule& s, int ttile, VecRef in,
                          OutRef out, const int* d_skip)
 {
-    const int bs = 256;
-    fixup_kernel<<<(unsigned)((c->N + bs - 1) / bs), bs, 0, c->stream>>>(
+    fixup_kernel<<<(unsigned)((c->N + kFixNodes - 1) / kFixNodes), kFixShares * kFixNodes, 0, c->stream>>>(
         c->d_part, s, ttile, c->N, k.lambda1, k.lambda2, in, out, d_skip);
     count_launch(c);
     IBIM_CUDA(cudaGetLastError());
@@ -451,8 +495,7 @@ cudaError_t launch_pair_f32_raw(const float4* tpos, const float4* tnrm, const fl
 cudaError_t launch_fixup_raw(const double* part, const PairSchedule& s, int64_t N, const PairConsts& k,
                              const double* d_in, double* d_out, cudaStream_t stream)
 {
-    const int bs = 256;
-    fixup_kernel<<<(unsigned)((N + bs - 1) / bs), bs, 0, stream>>>(part, s, kF32TTile, N, k.lambda1, k.lambda2,
+    fixup_kernel<<<(unsigned)((N + kFixNodes - 1) / kFixNodes), kFixShares * kFixNodes, 0, stream>>>(part, s, kF32TTile, N, k.lambda1, k.lambda2,
                                                                   VecRef{d_in, nullptr, 0, 0},
                                                                   OutRef{d_out, nullptr, 0, 0}, nullptr);
     return cudaGetLastError();

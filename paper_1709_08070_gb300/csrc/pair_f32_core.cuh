@@ -3,6 +3,8 @@
 // pair_f32.cu for the formulas, the chunk frames, the near/far split and the
 // accumulation.
 #pragma once
+#include <type_traits>
+
 #include "ibim_internal.cuh"
 #include "ptx.cuh"
 
@@ -190,20 +192,61 @@ static __device__ __noinline__ bool tube_f64(const Geo64& g, int64_t i, int64_t 
 // FP32 tube test defers to tube_f64.
 constexpr float kTieBand = 1e-5f;
 
+// Margins of the tube test, packed: p = tau^2 - rho^2 (to which s_x^2 is added:
+// positive inside the tangent-plane cylinder) and q = (4 tau^2 - rho^2) / 4
+// (+inf for tube rule 1), so that both have the tie band kTieBand tau^2.
+struct TubeTest {
+    float2 p, q;
+};
+__device__ __forceinline__ TubeTest tube_margins(float2 rr, const F32Consts& k)
+{
+    TubeTest t;
+    t.p = __ffma2_rn(rr, f2(-1.0f), f2(k.tau2));
+    t.q = __ffma2_rn(rr, f2(-0.25f), f2(0.25f * k.four_tau2));
+    return t;
+}
+
+// g from its series (g_series, both lanes at once) and fn = -(1 - E) = E xn - g
+// where kappa rho < 0.5; formed always and selected, so that the loops around
+// it have no branch.
+__device__ __forceinline__ void series_where_small(float2 xn, float2 En, const FarConsts& c, float2& g, float2& fn)
+{
+    const float2 x = __fmul2_rn(xn, c.neg1);
+    float2 p = __ffma2_rn(f2(-1.0f / 45360.0f), x, f2(1.0f / 5760.0f));
+    p = __ffma2_rn(p, x, f2(-1.0f / 840.0f));
+    p = __ffma2_rn(p, x, f2(1.0f / 144.0f));
+    p = __ffma2_rn(p, x, f2(-1.0f / 30.0f));
+    p = __ffma2_rn(p, x, f2(1.0f / 8.0f));
+    p = __ffma2_rn(p, x, f2(-1.0f / 3.0f));
+    p = __ffma2_rn(p, x, f2(0.5f));
+    const float2 gs = __fmul2_rn(__fmul2_rn(p, x), x);
+    const float2 fs = __ffma2_rn(gs, c.neg1, En);
+    g.x = x.x < 0.5f ? gs.x : g.x;
+    g.y = x.y < 0.5f ? gs.y : g.y;
+    fn.x = x.x < 0.5f ? fs.x : fn.x;
+    fn.y = x.y < 0.5f ? fs.y : fn.y;
+}
+
 // Near pairs, packed over the two sources of a payload pair (one target):
 // pair_far2's formula with, per lane, g from its series where kappa rho <
 // 0.5 (f = 1 - E = g + E x there) and the tube test (Sec. 2.2.1): a
 // regularised pair keeps only K12's tube value, by selects on rho^-3 and on
 // the 1/rho factor of the first sum.  rho^2 is kept >= 1e-12, so that
 // coincident nodes (the self pair among them, always in the tube) leave
-// every product finite.  When a test lies within kTieBand of a threshold,
-// both sources are decided again in FP64 (tube_f64), which the FP32 test
-// agrees with outside the band.  i: the target's node index, j: the first
-// source's.
+// every product finite.  A test within kTieBand of a threshold has to be
+// decided in FP64 (tube_f64, which the FP32 test agrees with outside the
+// band).  Without FLAT that is done on the spot, by a branch, and the series by
+// another; FLAT has no branch and keeps the smallest distance to a threshold in
+// tmin: the caller repeats the chunk without FLAT when it lies in the band.
+// (One-directional kernel, 5k-node sphere, almost every chunk near: 79 us flat,
+// 97 us with the branches; on large surfaces, where near chunks are few, the
+// flat loop costs the far loop registers: 80k nodes 8.01 against 7.88 ms.)
+// i: the target's node index, j: the first source's.
+template <bool FLAT>
 __device__ __forceinline__ void pair_near2(float2 Xx, float2 Xy, float2 Xz, float2 nx, float2 ny, float2 nz,
                                            const float4& A, const float4& B, const float4& C, const float4& D,
                                            const FarConsts& c, const F32Consts& k, float2& t1, float2& t2,
-                                           const Geo64& g64, int64_t i, int64_t j, int64_t N)
+                                           float& tmin, const Geo64& g64, int64_t i, int64_t j, int64_t N)
 {
     const float2 rx = __fadd2_rn(Xx, make_float2(A.x, A.y));
     const float2 ry = __fadd2_rn(Xy, make_float2(A.z, A.w));
@@ -222,14 +265,24 @@ __device__ __forceinline__ void pair_near2(float2 Xx, float2 Xy, float2 Xz, floa
     float2 ca = __fmul2_rn(nx, mx);
     ca = __ffma2_rn(ny, my, ca);
     ca = __ffma2_rn(nz, mz, ca);
-    const float2 rp = __ffma2_rn(__fmul2_rn(sx, c.neg1), sx, rr);
-    bool t0 = (rp.x < k.tau2) & (rr.x < k.four_tau2), t1b = (rp.y < k.tau2) & (rr.y < k.four_tau2);
-    const float bt = kTieBand * k.tau2, b4 = kTieBand * k.four_tau2;
-    const bool tie = (fabsf(rp.x - k.tau2) < bt) | (fabsf(rp.y - k.tau2) < bt) | (fabsf(rr.x - k.four_tau2) < b4) |
-                     (fabsf(rr.y - k.four_tau2) < b4);
-    if (tie && g64.x != nullptr && i < N) {
-        if (j < N) t0 = tube_f64(g64, i, j, k.tau2_d, k.four_tau2_d);
-        if (j + 1 < N) t1b = tube_f64(g64, i, j + 1, k.tau2_d, k.four_tau2_d);
+    bool t0, t1b;
+    if (FLAT) {
+        const TubeTest tt = tube_margins(rr, k);
+        const float2 mf = __ffma2_rn(sx, sx, tt.p);
+        t0 = (mf.x > 0.0f) & (tt.q.x > 0.0f);
+        t1b = (mf.y > 0.0f) & (tt.q.y > 0.0f);
+        tmin = fminf(tmin, fminf(fminf(fabsf(mf.x), fabsf(tt.q.x)), fminf(fabsf(mf.y), fabsf(tt.q.y))));
+    } else {
+        const float2 rp = __ffma2_rn(__fmul2_rn(sx, c.neg1), sx, rr);
+        t0 = (rp.x < k.tau2) & (rr.x < k.four_tau2);
+        t1b = (rp.y < k.tau2) & (rr.y < k.four_tau2);
+        const float bt = kTieBand * k.tau2, b4 = kTieBand * k.four_tau2;
+        const bool tie = (fabsf(rp.x - k.tau2) < bt) | (fabsf(rp.y - k.tau2) < bt) | (fabsf(rr.x - k.four_tau2) < b4) |
+                         (fabsf(rr.y - k.four_tau2) < b4);
+        if (tie && g64.x != nullptr && i < N) {
+            if (j < N) t0 = tube_f64(g64, i, j, k.tau2_d, k.four_tau2_d);
+            if (j + 1 < N) t1b = tube_f64(g64, i, j + 1, k.tau2_d, k.four_tau2_d);
+        }
     }
     const float2 rrs = make_float2(fmaxf(rr.x, 1.0e-12f), fmaxf(rr.y, 1.0e-12f));
     const float2 inv = make_float2(ptx::rsqrt_approx(rrs.x), ptx::rsqrt_approx(rrs.y));
@@ -240,13 +293,17 @@ __device__ __forceinline__ void pair_near2(float2 Xx, float2 Xy, float2 Xz, floa
     const float2 En = __fmul2_rn(E, xn);
     float2 fn = __fadd2_rn(E, c.neg1);
     float2 g = __ffma2_rn(fn, c.neg1, En);
-    if (-xn.x < 0.5f) {  // kappa rho < 0.5: series of g, fn = -(g + E x)
-        g.x = g_series(-xn.x);
-        fn.x = En.x - g.x;
-    }
-    if (-xn.y < 0.5f) {
-        g.y = g_series(-xn.y);
-        fn.y = En.y - g.y;
+    if (FLAT) {
+        series_where_small(xn, En, c, g, fn);
+    } else {
+        if (-xn.x < 0.5f) {  // kappa rho < 0.5: series of g, fn = -(g + E x)
+            g.x = g_series(-xn.x);
+            fn.x = En.x - g.x;
+        }
+        if (-xn.y < 0.5f) {
+            g.y = g_series(-xn.y);
+            fn.y = En.y - g.y;
+        }
     }
     const float2 hn = __ffma2_rn(g, c.neg3, __fmul2_rn(En, xn));
     const float2 inv2 = __fmul2_rn(inv, inv);
@@ -272,15 +329,16 @@ struct Targets {
 };
 
 // All interactions of one thread's targets with one staged source tile
-// (kF32STile nodes as kF32STile / 2 payload pairs at sb, chunk frames at
-// sfrm).  tfrm: the frames of the warp's target blocks (2 float4 per slot).
+// (CH chunks of kChunk nodes as payload pairs at sb, chunk frames at sfrm).
+// tfrm: the frames of the warp's target blocks (2 float4 per slot).
 // Adds the tile's sums to the compensated pairs (S, C).  gi0: node index of
 // the thread's slot-0 target, slot q adding q * qstride.  LIST kernels may
 // pass force_far for a tile whose every source is known to lie at least
 // far_dist from every target (treecode proxies): it then takes the far-field
 // branch without the per-chunk distance test; n_chunks < kChunksPerTile
-// skips the tile's trailing chunks (all padding).
-template <int TPT, bool LIST = false>
+// skips the tile's trailing chunks (all padding).  FLATNEAR: near chunks by the
+// branch-free form of pair_near2.
+template <int TPT, bool LIST = false, int CH = kChunksPerTile, bool FLATNEAR = false>
 __device__ __forceinline__ void tile_sums(const Targets<TPT>& T, const float4* tfrm, bool have_frames,
                                           const float4* sb, const float4* sfrm, const F32Consts& k,
                                           float (&S1)[TPT], float (&C1)[TPT], float (&S2)[TPT], float (&C2)[TPT],
@@ -289,7 +347,7 @@ __device__ __forceinline__ void tile_sums(const Targets<TPT>& T, const float4* t
 {
     const FarConsts fc = far_consts(k);
 #pragma unroll 1
-    for (int c = 0; c < (LIST ? n_chunks : kChunksPerTile); ++c) {
+    for (int c = 0; c < (LIST ? n_chunks : CH); ++c) {
         // targets in the source chunk's frame; far test on the two bounding spheres
         float3 X[TPT];
         const bool forced = LIST && force_far;
@@ -345,18 +403,29 @@ __device__ __forceinline__ void tile_sums(const Targets<TPT>& T, const float4* t
                 Xz[q] = f2(X[q].z);
             }
             const int64_t jc = j0 + (int64_t)c * kChunk;
-#pragma unroll 1
-            for (int p = 0; p < kPairsPerChunk; ++p) {
-                const float4 A = cb[kPairF4 * p], B = cb[kPairF4 * p + 1];
-                const float4 C = cb[kPairF4 * p + 2], D = cb[kPairF4 * p + 3];
+            float tmin = __builtin_huge_valf();
+            auto near_loop = [&](auto flat) {
+                constexpr bool FLAT = decltype(flat)::value;
+#pragma unroll(FLAT && TPT == 1 ? 2 : 1)
+                for (int p = 0; p < kPairsPerChunk; ++p) {
+                    const float4 A = cb[kPairF4 * p], B = cb[kPairF4 * p + 1];
+                    const float4 C = cb[kPairF4 * p + 2], D = cb[kPairF4 * p + 3];
 #pragma unroll
-                for (int q = 0; q < TPT; ++q) {
-                    if (TPT > 1 && farq[q])  // (one slot: this loop runs near chunks only)
-                        pair_far2(Xx[q], Xy[q], Xz[q], T.nx[q], T.ny[q], T.nz[q], A, B, C, D, fc, t1[q], t2[q]);
-                    else
-                        pair_near2(Xx[q], Xy[q], Xz[q], T.nx[q], T.ny[q], T.nz[q], A, B, C, D, fc, k, t1[q], t2[q],
-                                   g64, gi0 + (int64_t)q * qstride, jc + 2 * p, N);
+                    for (int q = 0; q < TPT; ++q) {
+                        if (TPT > 1 && farq[q])  // (one slot: this loop runs near chunks only)
+                            pair_far2(Xx[q], Xy[q], Xz[q], T.nx[q], T.ny[q], T.nz[q], A, B, C, D, fc, t1[q], t2[q]);
+                        else
+                            pair_near2<FLAT>(Xx[q], Xy[q], Xz[q], T.nx[q], T.ny[q], T.nz[q], A, B, C, D, fc, k, t1[q],
+                                             t2[q], tmin, g64, gi0 + (int64_t)q * qstride, jc + 2 * p, N);
+                    }
                 }
+            };
+            if (FLATNEAR) near_loop(std::true_type{});
+            // (with FLATNEAR only after a tie: the chunk again, its tests decided in FP64)
+            if (!FLATNEAR || __any_sync(0xffffffffu, tmin < kTieBand * k.tau2)) {
+#pragma unroll
+                for (int q = 0; q < TPT; ++q) t1[q] = t2[q] = make_float2(0.0f, 0.0f);
+                near_loop(std::false_type{});
             }
         }
 #pragma unroll
@@ -374,12 +443,14 @@ __device__ __forceinline__ void tile_sums(const Targets<TPT>& T, const float4* t
 // warp once it is done with the stage).  Warps consume stages independently;
 // thread 0 refills the stage of step u - 1 while at step u, so warps never
 // meet at a CTA-wide barrier inside the step loop.
-struct SourceStage {
-    float4 buf[kF32STile / 2 * kPairF4];
-    float4 frm[2 * kChunksPerTile];
+// A stage holds CH chunks: kChunksPerTile, or fewer where a launch would
+// otherwise have too few steps to fill the chip.
+template <int CH>
+struct SourceStageT {
+    float4 buf[CH * kPairsPerChunk * kPairF4];
+    float4 frm[2 * CH];
 };
-constexpr uint32_t kStagePayloadBytes = kF32STile / 2 * kPairF4 * sizeof(float4);
-constexpr uint32_t kStageFrameBytes = 2 * kChunksPerTile * sizeof(float4);
+using SourceStage = SourceStageT<kChunksPerTile>;
 
 struct StagePipe {
     uint64_t full[kF32Stages];
@@ -396,12 +467,14 @@ __device__ __forceinline__ void pipe_init(StagePipe& P, int nwarps)
 }
 
 // Stage a source tile (payload at src, frames at frm or none).
-__device__ __forceinline__ void pipe_issue(StagePipe& P, SourceStage& S, int stage, const float4* src,
+template <int CH>
+__device__ __forceinline__ void pipe_issue(StagePipe& P, SourceStageT<CH>& S, int stage, const float4* src,
                                            const float4* frm)
 {
-    const uint32_t fbytes = frm != nullptr ? kStageFrameBytes : 0u;
-    ptx::mbar_arrive_expect_tx(&P.full[stage], kStagePayloadBytes + fbytes);
-    ptx::bulk_g2s(&S.buf[0], src, kStagePayloadBytes, &P.full[stage]);
+    constexpr uint32_t kPayloadBytes = sizeof(S.buf);
+    const uint32_t fbytes = frm != nullptr ? (uint32_t)sizeof(S.frm) : 0u;
+    ptx::mbar_arrive_expect_tx(&P.full[stage], kPayloadBytes + fbytes);
+    ptx::bulk_g2s(&S.buf[0], src, kPayloadBytes, &P.full[stage]);
     if (frm != nullptr) ptx::bulk_g2s(&S.frm[0], frm, fbytes, &P.full[stage]);
 }
 

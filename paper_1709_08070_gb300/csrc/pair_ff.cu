@@ -825,7 +825,7 @@ int ffs_grid_cap(ibim_ctx* c)
     return (occ < 1 ? 1 : occ) * c->num_sms;
 }
 
-size_t ffs_part_doubles(ibim_ctx* c) { return sym_part_doubles(c->N, kFFSThreads, ffs_grid_cap(c)); }
+size_t ffs_part_doubles(ibim_ctx* c) { return sym_part_doubles(c->N, kFFSThreads, kFFSTile, ffs_grid_cap(c)); }
 
 ibim_status ff_pack(ibim_ctx* c, VecRef in, const int* d_skip)
 {
@@ -843,7 +843,7 @@ ibim_status ff_pack(ibim_ctx* c, VecRef in, const int* d_skip)
 ibim_status ff_pairs(ibim_ctx* c, const PairConsts& k, const PairSchedule& s, const int* d_skip)
 {
     if (c->ff_symmetric) {
-        const SymSchedule ss = make_sym_schedule(c->N, kFFSThreads, ffs_grid_cap(c));
+        const SymSchedule ss = make_sym_schedule(c->N, kFFSThreads, kFFSTile, ffs_grid_cap(c));
         pair_ffs_kernel<<<ss.grid, kFFSThreads, 0, c->stream>>>(
             (const float4*)c->d_src, c->d_frames, c->d_fftab, c->d_geo64, c->N, padded_nodes(c->N), ss, ff_consts(k),
             c->d_part, c->d_yrev, c->d_err, d_skip);
@@ -860,7 +860,7 @@ ibim_status ff_pairs(ibim_ctx* c, const PairConsts& k, const PairSchedule& s, co
 ibim_status ff_fixup(ibim_ctx* c, const PairConsts& k, const PairSchedule& s, VecRef in, OutRef out,
                      const int* d_skip)
 {
-    if (c->ff_symmetric) return sym_fixup_tiles(c, kFFSThreads, ffs_grid_cap(c), k, in, out, d_skip);
+    if (c->ff_symmetric) return sym_fixup_tiles(c, kFFSThreads, kFFSTile, ffs_grid_cap(c), k, in, out, d_skip);
     return fixup_launch(c, k, s, kFFTTile, in, out, d_skip);
 }
 

@@ -65,7 +65,7 @@
 namespace ibim {
 
 
-template <int TPT, int MINB, int THREADS, bool ROT, int UNR>
+template <int TPT, int MINB, int THREADS, bool ROT, int UNR, int CH>
 __global__ void __launch_bounds__(THREADS, MINB)
     pair_sym_kernel(const float4* __restrict__ tpos, const float4* __restrict__ tnrm,
                     const float4* __restrict__ src, const float4* __restrict__ frames, int64_t N, int64_t n_pad,
@@ -74,13 +74,14 @@ __global__ void __launch_bounds__(THREADS, MINB)
 {
     constexpr int TTILE = THREADS * TPT;
     constexpr int NW = THREADS / 32;
-    static_assert(TTILE <= kF32MaxTTile && TTILE % kF32STile == 0, "target tile");
+    constexpr int STILE = CH * kChunk;
+    static_assert(TTILE <= kF32MaxTTile && TTILE % STILE == 0 && kPadNodes % STILE == 0, "tiles");
     if (skip != nullptr && *skip) return;
-    __shared__ __align__(128) SourceStage stg[kF32Stages];
+    __shared__ __align__(128) SourceStageT<CH> stg[kF32Stages];
     __shared__ __align__(16) float4 tfrm[NW][2 * TPT];
     __shared__ __align__(8) StagePipe pipe;
-    constexpr int REVOFF = sym_rev_off(ROT);
-    __shared__ float racc[kF32Stages][sym_rev_row(ROT)];
+    constexpr int REVOFF = sym_rev_off(ROT, CH), REVROW = sym_rev_row(ROT, CH);
+    __shared__ float racc[kF32Stages][REVROW];
     __shared__ int64_t stage_st[kF32Stages];
 
     __shared__ int64_t seg_next[2];
@@ -91,7 +92,7 @@ __global__ void __launch_bounds__(THREADS, MINB)
     const int lane = tid & 31;
     unsigned long long* seg_ctr = reinterpret_cast<unsigned long long*>(yrev + 2 * n_pad);
 
-    for (int q = tid; q < kF32Stages * sym_rev_row(ROT); q += THREADS) (&racc[0][0])[q] = 0.0f;
+    for (int q = tid; q < kF32Stages * REVROW; q += THREADS) (&racc[0][0])[q] = 0.0f;
     if (tid == 0) {
         pipe_init(pipe, NW);
         abort_sh = 0;
@@ -108,7 +109,7 @@ __global__ void __launch_bounds__(THREADS, MINB)
         const int64_t st = s.R * t + pos;
         const int stage = (int)((u + off) % kF32Stages);
         stage_st[stage] = st;
-        pipe_issue(pipe, stg[stage], stage, src + st * (kF32STile / 2) * kPairF4, frames + st * 2 * kChunksPerTile);
+        pipe_issue(pipe, stg[stage], stage, src + st * (STILE / 2) * kPairF4, frames + st * 2 * CH);
     };
 
     int64_t t, rho, pos;
@@ -151,8 +152,8 @@ __global__ void __launch_bounds__(THREADS, MINB)
     // warp 0: add the reverse sums of step v to the global vector and clear them
     auto flush = [&](int64_t v) {
         const int sv = (int)((v + off) % kF32Stages);
-        const int64_t j0 = stage_st[sv] * kF32STile;
-        for (int jj = lane; jj < kF32STile; jj += 32) {
+        const int64_t j0 = stage_st[sv] * STILE;
+        for (int jj = lane; jj < STILE; jj += 32) {
             const float v1 = racc[sv][jj], v2 = racc[sv][REVOFF + jj];
             if (v1 != 0.0f) atomicAdd(yrev + j0 + jj, (double)v1);
             if (v2 != 0.0f) atomicAdd(yrev + n_pad + j0 + jj, (double)v2);
@@ -208,8 +209,8 @@ __global__ void __launch_bounds__(THREADS, MINB)
 #pragma unroll
             for (int q = 0; q < TPT; ++q) S1[q] = C1[q] = S2[q] = C2[q] = 0.0f;
             if (!idle)
-                tile_sums_sym<TPT, ROT, UNR>(T, &tfrm[warp][0], stg[stage].buf, stg[stage].frm, k, S1, C1, S2, C2, g64, gi0,
-                                   THREADS, st * kF32STile, N, Ablk, st * kChunksPerTile, &racc[stage][0]);
+                tile_sums_sym<TPT, ROT, UNR, CH>(T, &tfrm[warp][0], stg[stage].buf, stg[stage].frm, k, S1, C1, S2, C2, g64, gi0,
+                                   THREADS, st * STILE, N, Ablk, st * CH, &racc[stage][0]);
 #pragma unroll
             for (int q = 0; q < TPT; ++q) {
                 D1[q] += (double)S1[q] - (double)C1[q];
@@ -365,28 +366,39 @@ struct SymArgs {
     Geo64 g64;
 };
 
-template <int TPT, int MINB, int THREADS, bool ROT, int UNR>
+template <int TPT, int MINB, int THREADS, bool ROT, int UNR, int CH>
 static void launch_sym(const SymArgs& a, cudaStream_t st)
 {
-    pair_sym_kernel<TPT, MINB, THREADS, ROT, UNR><<<a.s.grid, THREADS, 0, st>>>(
+    pair_sym_kernel<TPT, MINB, THREADS, ROT, UNR, CH><<<a.s.grid, THREADS, 0, st>>>(
         a.tpos, a.tnrm, a.src, a.frames, a.N, a.n_pad, a.s, a.k, a.part, a.yrev, a.err, a.skip, a.g64);
 }
 
 // scheme: 1 = warp reduction of the reverse sums, 2 = rotation (see the file comment)
 struct SymVariant {
-    int tpt, minb, threads, scheme;
+    int tpt, minb, threads, scheme, stile;
     const void* fn;
     void (*launch)(const SymArgs&, cudaStream_t);
 };
-#define IBIM_SYM_VARIANT(T, M, W, R, U) \
-    {T, M, W, (R) ? 2 : 1, (const void*)pair_sym_kernel<T, M, W, R, U>, launch_sym<T, M, W, R, U>}
+#define IBIM_SYM_VARIANT(T, M, W, R, U, C)                                                              \
+    {T, M, W, (R) ? 2 : 1, (C) * kChunk, (const void*)pair_sym_kernel<T, M, W, R, U, C>,                \
+     launch_sym<T, M, W, R, U, C>}
+// The last three, with smaller source tiles and target tiles, are for small
+// molecules: a launch of 512-target tiles on 5,000 nodes has 110 steps for 152
+// SMs.  Measured per application (us; the best of the first four, then these):
+// 862 nodes 66 / 21.7 33 63; 4,982 68 / 50.8 56 67; 12,754 201 / 198 186 191;
+// 21,651 467 / 531 504 445; 37,657 1245 / 1515 1417 1244; 80,358 5334 / 6459
+// 6102 5583 (the smaller target tile reads every source more often).  The
+// autotuner picks.
 static const SymVariant kSymVariants[] = {
-    IBIM_SYM_VARIANT(2, 1, 512, false, 2), IBIM_SYM_VARIANT(1, 1, 512, false, 2),
-    IBIM_SYM_VARIANT(2, 1, 512, true, 1), IBIM_SYM_VARIANT(1, 1, 512, true, 4),
+    IBIM_SYM_VARIANT(2, 1, 512, false, 2, 8), IBIM_SYM_VARIANT(1, 1, 512, false, 2, 8),
+    IBIM_SYM_VARIANT(2, 1, 512, true, 1, 8),  IBIM_SYM_VARIANT(1, 1, 512, true, 4, 8),
+    IBIM_SYM_VARIANT(1, 4, 128, true, 4, 2),  IBIM_SYM_VARIANT(1, 2, 256, true, 4, 4),
+    IBIM_SYM_VARIANT(2, 1, 512, true, 1, 4),
 };
 #undef IBIM_SYM_VARIANT
 constexpr int kNumSymVariants = (int)(sizeof(kSymVariants) / sizeof(kSymVariants[0]));
 
+int sym_stile(int v) { return kSymVariants[v].stile; }
 int sym_variant_count() { return kNumSymVariants; }
 void sym_variant_info(int v, int* tpt, int* minb, int* threads, int* scheme)
 {
@@ -406,12 +418,12 @@ int sym_occupancy(int v)
 // the rest is cut into about kSymSmallPerCta small segments per CTA.
 constexpr int64_t kSymBigShare = 9, kSymShareDen = 10, kSymSmallPerCta = 16;
 
-SymSchedule make_sym_schedule(int64_t N, int ttile, int grid_cap)
+SymSchedule make_sym_schedule(int64_t N, int ttile, int stile, int grid_cap)
 {
     SymSchedule s;
     s.n_t = (N + ttile - 1) / ttile;
-    s.n_s = (N + kF32STile - 1) / kF32STile;
-    s.R = ttile / kF32STile;
+    s.n_s = (N + stile - 1) / stile;
+    s.R = ttile / stile;
     s.npairs = s.n_t / 2;
     s.L2 = 2 * s.n_s - s.R * (s.n_t - 1);
     s.total = s.npairs * s.L2 + ((s.n_t & 1) ? sym_row_len(s, s.npairs) : 0);
@@ -427,9 +439,9 @@ SymSchedule make_sym_schedule(int64_t N, int ttile, int grid_cap)
 }
 
 // Partial slots (segment + row sequence index < nseg + n_t).
-size_t sym_part_doubles(int64_t N, int ttile, int grid_cap)
+size_t sym_part_doubles(int64_t N, int ttile, int stile, int grid_cap)
 {
-    const SymSchedule s = make_sym_schedule(N, ttile, grid_cap);
+    const SymSchedule s = make_sym_schedule(N, ttile, stile, grid_cap);
     return (size_t)(s.nseg + s.n_t) * 2 * ttile;
 }
 
@@ -452,7 +464,7 @@ ibim_status sym_pack(ibim_ctx* c, VecRef in, const int* d_skip)
 ibim_status sym_pairs(ibim_ctx* c, int sv, int grid_cap, const PairConsts& k, const int* d_skip)
 {
     const SymVariant& v = kSymVariants[sv];
-    const SymSchedule s = make_sym_schedule(c->N, v.tpt * v.threads, grid_cap);
+    const SymSchedule s = make_sym_schedule(c->N, v.tpt * v.threads, v.stile, grid_cap);
     const int64_t n_pad = padded_nodes(c->N);
     const F32Consts kk = f32_consts(k);
     const Geo64 g64{c->d_geo64, c->d_geo64 + 3 * c->N, 1, c->N};
@@ -468,16 +480,16 @@ ibim_status sym_fixup(ibim_ctx* c, int sv, int grid_cap, const PairConsts& k, Ve
                       const int* d_skip)
 {
     const SymVariant& v = kSymVariants[sv];
-    return sym_fixup_tiles(c, v.tpt * v.threads, grid_cap, k, in, out, d_skip);
+    return sym_fixup_tiles(c, v.tpt * v.threads, v.stile, grid_cap, k, in, out, d_skip);
 }
 
 // y = Lambda p + (1/(4 pi)) (forward partials + reverse sums) for a symmetric
 // launch of `ttile`-target tiles on a grid of at most grid_cap CTAs.
-ibim_status sym_fixup_tiles(ibim_ctx* c, int ttile, int grid_cap, const PairConsts& k, VecRef in, OutRef out,
+ibim_status sym_fixup_tiles(ibim_ctx* c, int ttile, int stile, int grid_cap, const PairConsts& k, VecRef in, OutRef out,
                             const int* d_skip)
 {
-    const SymSchedule s = make_sym_schedule(c->N, ttile, grid_cap);
-    static_assert(kFixParts == 4 && kF32STile % kFixTargets == 0, "fixup shares");
+    const SymSchedule s = make_sym_schedule(c->N, ttile, stile, grid_cap);
+    static_assert(kFixParts == 4 && 128 % kFixTargets == 0, "fixup shares");
     fixup_sym_kernel<<<(unsigned)((c->N + kFixTargets - 1) / kFixTargets), kFixParts * kFixTargets, 0, c->stream>>>(
         c->d_part, s, ttile, c->N, padded_nodes(c->N), k.lambda1, k.lambda2, in, out, c->d_yrev, d_skip);
     count_launch(c);

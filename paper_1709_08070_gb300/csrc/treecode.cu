@@ -410,7 +410,7 @@ __global__ void __launch_bounds__(THREADS, MINB)
 #pragma unroll
             for (int q = 0; q < TPT; ++q) S1[q] = C1[q] = S2[q] = C2[q] = 0.0f;
             if (!idle)
-                tile_sums<TPT, true>(T, &tfrm[warp][0], true, stg[stage].buf, stg[stage].frm, k, S1, C1, S2, C2,
+                tile_sums<TPT, true, kChunksPerTile, true>(T, &tfrm[warp][0], true, stg[stage].buf, stg[stage].frm, k, S1, C1, S2, C2,
                                      g64, gi0, THREADS, st * kF32STile, N, st >= s.n_real_tiles,
                                      st >= s.n_real_tiles ? s.proxy_chunks : kChunksPerTile);
 #pragma unroll
