@@ -3,11 +3,10 @@
 //
 // The pair geometry (r, |r|, e^{-kappa rho}, g, 3 - B, rho^-3, the theta
 // terms) is the same for the ordered pairs (i <- j) and (j <- i), so one
-// evaluation of an unordered pair gives both contributions: 48 FP32
-// lane-operations per pair instead of 2 x 36 (28 shared and 10 per direction
-// in pair_far_sym; 36 shared and 6 per direction in the rotation scheme's
-// pair_far_sym_acc, which forms the factors common to both directions
-// once).  Each aligned 32-node block pair
+// evaluation of an unordered pair gives both contributions: 46 FP32
+// lane-operations per pair instead of 2 x 36 (38 shared and 4 per direction in
+// the rotation scheme's pair_far_sym_acc, which forms the factors common to both
+// directions once; 28 and 10 in pair_far_sym).  Each aligned 32-node block pair
 // (A, B) is evaluated once: by the warp holding target block A when B > A
 // (both directions), B == A gives the forward direction only (it holds the
 // self pairs), and B < A is skipped (the warp holding B covered it).

@@ -159,14 +159,16 @@ __device__ __forceinline__ void pair_far_sym(float2 Xx, float2 Xy, float2 Xz, fl
 }
 
 // pair_far_sym with the reverse sums accumulated into (nR1, R2) (rotation
-// scheme): nR1 -= first reverse sum, R2 += second.  The factors common to both
-// directions are formed once, P u1, P u2, P g c and P hn rho^-2, and rho^-2 is
-// the square of the MUFU rsqrt (two MUFU operations per source, 48 packed
-// operations per source pair as in pair_far_sym: 36 shared, 6 per direction):
-//   t1 += (P u1) s_a + qf b,   t2 += s_x [(P hn rho^-2) s_a + (P u2) b] + (P g c) a
-// and the reverse sums likewise with (s_a, b, s_x, a) -> (a_i s_x, -b_i, s_y, a_i).
-// (Measured against pair_far_sym's order of operations inside the rotation
-// loop: 5.66 against 5.74 ms per application on the 80k-node sphere.)
+// scheme): nR1 -= first reverse sum, R2 += second.  The a-part of the second sum
+// is the same in both directions, W = [g c - (3 - B) s_x s_y / rho^2] / rho^3:
+//   t1 += (P u1 s_y) a_j + qf b_j,  t2 += (P u2 s_x) b_j + W a_j,  P = rho^-3,
+// and the reverse sums likewise with (s_y, b_j, s_x, a_j) -> (s_x, -b_i, s_y,
+// a_i): 46 packed operations per source pair, 38 shared and 4 per direction, and
+// three MUFU operations per source: rho is the hardware square root, not rho^2
+// times the rsqrt, as the XU pipe has room (12 % busy).  211k / 80k nodes:
+// 35.76 / 5.19 ms per application, 36.73 / 5.33 with 48 operations (each direction
+// its own s_x s_y product) and two MUFU; rho^-2 by a hardware reciprocal as well
+// (45 operations) 36.01 / 5.22.
 __device__ __forceinline__ void pair_far_sym_acc(float2 Xx, float2 Xy, float2 Xz, float2 nx, float2 ny, float2 nz,
                                                  float2 ai, float2 nbi, const float4& A, const float4& B,
                                                  const float4& C, const float4& D, const FarConsts& c, float2& t1,
@@ -191,7 +193,7 @@ __device__ __forceinline__ void pair_far_sym_acc(float2 Xx, float2 Xy, float2 Xz
     cc = __ffma2_rn(ny, my, cc);
     cc = __ffma2_rn(nz, mz, cc);
     const float2 inv = make_float2(ptx::rsqrt_approx(rr.x), ptx::rsqrt_approx(rr.y));
-    const float2 rho = __fmul2_rn(rr, inv);
+    const float2 rho = make_float2(ptx::sqrt_approx(rr.x), ptx::sqrt_approx(rr.y));
     const float2 ea = __fmul2_rn(rho, c.kl2e);
     const float2 xn = __fmul2_rn(rho, c.nkappa);
     const float2 E = make_float2(ptx::ex2_approx(ea.x), ptx::ex2_approx(ea.y));
@@ -203,21 +205,18 @@ __device__ __forceinline__ void pair_far_sym_acc(float2 Xx, float2 Xy, float2 Xz
     const float2 P = __fmul2_rn(inv2, inv);
     const float2 Pu1 = __fmul2_rn(P, __ffma2_rn(c.th1, g, c.omth1));
     const float2 Pu2 = __fmul2_rn(P, __ffma2_rn(c.th2, g, c.omth2));
-    const float2 Pgc = __fmul2_rn(__fmul2_rn(P, g), cc);
-    const float2 Phi = __fmul2_rn(hn, __fmul2_rn(inv2, P));
+    const float2 W = __fmul2_rn(P, __ffma2_rn(__fmul2_rn(hn, inv2), __fmul2_rn(sx, sy), __fmul2_rn(g, cc)));
     const float2 qf = __fmul2_rn(fn, inv);
     // forward
-    const float2 sa = __fmul2_rn(aj, sy);
-    t1 = __ffma2_rn(Pu1, sa, t1);
+    t1 = __ffma2_rn(__fmul2_rn(Pu1, sy), aj, t1);
     t1 = __ffma2_rn(qf, bj, t1);
-    t2 = __ffma2_rn(sx, __ffma2_rn(Phi, sa, __fmul2_rn(Pu2, bj)), t2);
-    t2 = __ffma2_rn(Pgc, aj, t2);
+    t2 = __ffma2_rn(__fmul2_rn(Pu2, sx), bj, t2);
+    t2 = __ffma2_rn(W, aj, t2);
     // reverse, accumulated
-    const float2 psa = __fmul2_rn(ai, sx);
-    nR1 = __ffma2_rn(Pu1, psa, nR1);
+    nR1 = __ffma2_rn(__fmul2_rn(Pu1, sx), ai, nR1);
     nR1 = __ffma2_rn(qf, nbi, nR1);
-    R2 = __ffma2_rn(sy, __ffma2_rn(Phi, psa, __fmul2_rn(Pu2, nbi)), R2);
-    R2 = __ffma2_rn(Pgc, ai, R2);
+    R2 = __ffma2_rn(__fmul2_rn(Pu2, sy), nbi, R2);
+    R2 = __ffma2_rn(W, ai, R2);
 }
 
 // Near pairs in the rotation scheme, both directions, packed over the two
@@ -327,27 +326,24 @@ __device__ __forceinline__ void pair_near_sym_acc(float2 Xx, float2 Xy, float2 X
     const float2 P = __fmul2_rn(inv2, inv);
     const float2 Pu1 = __fmul2_rn(P, __ffma2_rn(c.th1, g, c.omth1));
     const float2 Pu2 = __fmul2_rn(P, __ffma2_rn(c.th2, g, c.omth2));
-    const float2 Pgc = __fmul2_rn(__fmul2_rn(P, g), cc);
-    const float2 Phi = __fmul2_rn(hn, __fmul2_rn(inv2, P));
+    const float2 W = __fmul2_rn(P, __ffma2_rn(__fmul2_rn(hn, inv2), __fmul2_rn(sx, sy), __fmul2_rn(g, cc)));
     const float2 qf = __fmul2_rn(fn, inv);
     // forward; a regularised pair adds -K12_tube b only
     const float2 ajf = make_float2(tf0 ? 0.0f : aj.x, tf1 ? 0.0f : aj.y);
     const float2 bjt = make_float2(tf0 ? 0.0f : bj.x, tf1 ? 0.0f : bj.y);
     const float2 qff = make_float2(tf0 ? -k.k12t : qf.x, tf1 ? -k.k12t : qf.y);
-    const float2 sa = __fmul2_rn(ajf, sy);
-    t1 = __ffma2_rn(Pu1, sa, t1);
+    t1 = __ffma2_rn(__fmul2_rn(Pu1, sy), ajf, t1);
     t1 = __ffma2_rn(qff, bj, t1);
-    t2 = __ffma2_rn(sx, __ffma2_rn(Phi, sa, __fmul2_rn(Pu2, bjt)), t2);
-    t2 = __ffma2_rn(Pgc, ajf, t2);
+    t2 = __ffma2_rn(__fmul2_rn(Pu2, sx), bjt, t2);
+    t2 = __ffma2_rn(W, ajf, t2);
     // reverse, accumulated (nbi = -b_i)
     const float2 air = make_float2(tr0 ? 0.0f : ai.x, tr1 ? 0.0f : ai.y);
     const float2 nbt = make_float2(tr0 ? 0.0f : nbi.x, tr1 ? 0.0f : nbi.y);
     const float2 qfr = make_float2(tr0 ? -k.k12t : qf.x, tr1 ? -k.k12t : qf.y);
-    const float2 psa = __fmul2_rn(air, sx);
-    nR1 = __ffma2_rn(Pu1, psa, nR1);
+    nR1 = __ffma2_rn(__fmul2_rn(Pu1, sx), air, nR1);
     nR1 = __ffma2_rn(qfr, nbi, nR1);
-    R2 = __ffma2_rn(sy, __ffma2_rn(Phi, psa, __fmul2_rn(Pu2, nbt)), R2);
-    R2 = __ffma2_rn(Pgc, air, R2);
+    R2 = __ffma2_rn(__fmul2_rn(Pu2, sy), nbt, R2);
+    R2 = __ffma2_rn(W, air, R2);
 }
 
 // One ordered near pair (target <- source), scalar: tube test on the target's
