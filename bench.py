@@ -48,19 +48,18 @@ F32_OPS_PER_INTERACTION = 36
 # products, rho^-3, theta terms, hi, qf) is 28 lane-operations and each
 # direction's two sums 10 more, 48 for two interactions.
 F32_OPS_PER_INTERACTION_SYM = 24
-# The float-float operator (IBIM_FF, pair_ff_kernel), counted from ff_pair's
-# far branch: r 6, |r|^2 31, s_x, s_y and n.m 31 each, 1/rho 11, rho, kappa rho
-# and the exponent argument 4 each, exp 25, E x 4, 1 - E 4, g 11, 1 - th A
-# 15 twice, 3 - B 18, rho^-2 and rho^-3 8, the y1 term 31, the y2 term 54 and
-# the two float-float accumulations 22 FP32-pipe operations per interaction
-# (plus one MUFU, about six integer operations and five shared loads).
-FF_OPS_PER_INTERACTION = 366
-# The symmetric float-float kernel (pair_ffs_kernel, the default IBIM_FF kernel),
-# counted from ffs_pair: 296 shared operations per unordered pair (the above up
-# to rho^-3, plus the combination g c - (3 - B) s_x s_y / rho^2 27 and four
-# products with the powers of 1/rho 16) and 68 per direction (the two terms 46,
-# their float-float accumulation 22): 432 per unordered pair, 216 per interaction.
-FFS_OPS_PER_INTERACTION = 216
+# The float-float operator (IBIM_FF, pair_ff_kernel), counted from ff_pairs2's
+# far form (lane-operations per interaction): r 6, |r|^2, s_x and s_y 31 each,
+# n.m 28, 1/rho 11, rho 7, kappa rho and the exponent argument 4 each, exp 25, E x
+# 4, 1 - E 4, g 11, 1 - th A 12 twice, 3 - B 15, rho^-2 and rho^-3 8, the
+# combination g c - (3 - B) s_x s_y / rho^2 24, four products with the powers of
+# 1/rho 16: 284; the two terms 20 each and their float-float accumulation 22 (plus
+# one MUFU, about six integer operations and four shared loads).
+FF_OPS_PER_INTERACTION = 346
+# The symmetric float-float kernel (pair_ffs_kernel, the default IBIM_FF kernel):
+# the 284 shared operations once per unordered pair and 62 per direction, 408 per
+# unordered pair.
+FFS_OPS_PER_INTERACTION = 204
 FP32_LANES_PER_SM = 128
 # dram__bytes_read.sum + dram__bytes_write.sum of one pair-kernel launch on this
 # workload, by variant (targets/thread, min CTAs/SM, threads/CTA, symmetric scheme), from

@@ -210,14 +210,16 @@ int sym_variant_count();
 void sym_variant_info(int v, int* tpt, int* minb, int* threads, int* scheme);
 int sym_occupancy(int v);
 int sym_stile(int v);  // source tile of symmetric variant v
-size_t sym_part_doubles(int64_t N, int ttile, int stile, int grid_cap);
+// Large segments of a symmetric schedule: this many tenths of an even share per CTA.
+constexpr int kSymBigShare = 9;
+size_t sym_part_doubles(int64_t N, int ttile, int stile, int grid_cap, int big_share = kSymBigShare);
 size_t sym_yrev_bytes(int64_t N);
 ibim_status sym_pack(ibim_ctx* c, VecRef in, const int* d_skip);
 ibim_status sym_pairs(ibim_ctx* c, int sv, int grid_cap, const PairConsts& k, const int* d_skip);
 ibim_status sym_fixup(ibim_ctx* c, int sv, int grid_cap, const PairConsts& k, VecRef in, OutRef out,
                       const int* d_skip);
 ibim_status sym_fixup_tiles(ibim_ctx* c, int ttile, int stile, int grid_cap, const PairConsts& k, VecRef in, OutRef out,
-                            const int* d_skip);
+                            const int* d_skip, int big_share = kSymBigShare);
 PairSchedule f32_schedule(ibim_ctx* c);
 ibim_status f32_chunk_frames(ibim_ctx* c);
 ibim_status f32_pack_to(ibim_ctx* c, VecRef in, float4* dst, const int* d_skip);

@@ -54,14 +54,22 @@ constexpr int kFFChunksPerTile = kFFSTile / kFFChunk;
 constexpr int kFFTab = 256;      // table of 2^(i/256)
 constexpr uint64_t kFFWaitNs = 2000000000ull;  // 2 s
 static_assert(kPadNodes % kFFSTile == 0 && kPadNodes % kFFTTile == 0, "padding");
-// payload per node: (xh, ah), (xl, al), (nh, bh), (nl, bl), stored per aligned
-// 32-node chunk component by component (the chunk's 32 first float4, then its
-// 32 second ones, ...), so that 32 lanes reading 32 different nodes of a chunk
-// touch 512 contiguous bytes
+// Payload: the nodes p and p + 16 of an aligned 32-node chunk form a pair whose
+// values lie side by side, as the packed FP32 instructions take them.  A pair
+// has eight float4:
+//   0 (xh0 xh0' xh1 xh1')  1 (xh2 xh2' ah ah')  2, 3 the same of xl, al
+//   4 (nh0 nh0' nh1 nh1')  5 (nh2 nh2' bh bh')  6, 7 the same of nl, bl
+// stored per chunk component by component (the chunk's 16 first float4, then
+// its 16 second ones, ...), so that 16 lanes reading the 16 pairs of a chunk
+// touch 256 contiguous bytes.
 constexpr int kFFNodeF4 = 4;
-__host__ __device__ __forceinline__ int64_t ff_off(int64_t j, int comp)
+constexpr int kFFPairs = kFFChunk / 2;
+// Float offset of value c of field f of node j: fields (xh, ah), (xl, al), (nh,
+// bh), (nl, bl), values 0..2 the components and 3 the scalar.
+__host__ __device__ __forceinline__ int64_t ff_off(int64_t j, int f, int c)
 {
-    return (j >> 5) * (32 * kFFNodeF4) + comp * 32 + (j & 31);
+    const int64_t f4 = (j >> 5) * (32 * kFFNodeF4) + (2 * f + (c >> 1)) * kFFPairs + (j & (kFFPairs - 1));
+    return 4 * f4 + 2 * (c & 1) + ((j >> 4) & 1);
 }
 constexpr uint32_t kFFStageBytes = kFFSTile * kFFNodeF4 * sizeof(float4);
 constexpr uint32_t kFFFrameBytes = 2 * kFFChunksPerTile * sizeof(float4);
@@ -69,120 +77,181 @@ constexpr float kFFPad = 1.0e4f;  // placeholder coordinate (sources +, targets 
 
 // ------------------------------------------------------ float-float arithmetic
 
+// Two pairs of nodes per lane in the packed FP32 instructions (add, mul and fma
+// of two values; negating an operand costs nothing, measured).  One pair per
+// lane took 444 instructions a pair and stood at 0.84 of the issue slots and 0.75
+// of the FMA pipe; packed it is 252 (209 of them FMA-pipe instructions of two
+// cycles each), so the FMA pipe bounds it (39,406 nodes 10.9 -> 9.8 ms with the
+// finer segments below).
+__device__ __forceinline__ float2 vneg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __fadd2_rn(a, vneg(b)); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 vset(float a) { return make_float2(a, a); }
+
 struct ff {
     float h, l;
 };
+struct ff2 {
+    float2 h, l;
+};
 
-__device__ __forceinline__ ff ff_of(float2 v) { return ff{v.x, v.y}; }
+// Constant (h, h, l, l): one 64-bit operand each.
+__device__ __forceinline__ ff2 ff_of(const float4& v) { return ff2{make_float2(v.x, v.y), make_float2(v.z, v.w)}; }
+
+__device__ __forceinline__ ff2 ff_wide(ff v) { return ff2{vset(v.h), vset(v.l)}; }
+__device__ __forceinline__ ff ff_half(ff2 v, int q) { return q ? ff{v.h.y, v.l.y} : ff{v.h.x, v.l.x}; }
 
 // Knuth's two-sum: s + e == a + b exactly.
-__device__ __forceinline__ ff two_sum(float a, float b)
+__device__ __forceinline__ ff2 two_sum(float2 a, float2 b)
 {
-    const float s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-    return ff{s, e};
+    const float2 s = vadd(a, b);
+    const float2 bb = vsub(s, a);
+    const float2 e = vadd(vsub(a, vsub(s, bb)), vsub(b, bb));
+    return ff2{s, e};
 }
 
 // Dekker's fast two-sum (exact when |a| >= |b|, or a == 0).
-__device__ __forceinline__ ff fast_two_sum(float a, float b)
+__device__ __forceinline__ ff2 fast_two_sum(float2 a, float2 b)
 {
-    const float s = __fadd_rn(a, b);
-    return ff{s, __fsub_rn(b, __fsub_rn(s, a))};
+    const float2 s = vadd(a, b);
+    return ff2{s, vsub(b, vsub(s, a))};
 }
+
+__device__ __forceinline__ ff2 ff_norm(ff2 a) { return fast_two_sum(a.h, a.l); }
 
 // a b with the l l' term dropped (result nearly normalised).
-__device__ __forceinline__ ff ff_mul(ff a, ff b)
+__device__ __forceinline__ ff2 ff_mul(ff2 a, ff2 b)
 {
-    const float p = __fmul_rn(a.h, b.h);
-    float e = __fmaf_rn(a.h, b.h, -p);
-    e = __fmaf_rn(a.h, b.l, e);
-    e = __fmaf_rn(a.l, b.h, e);
-    return ff{p, e};
+    const float2 p = vmul(a.h, b.h);
+    float2 e = vfma(a.h, b.h, vneg(p));
+    e = vfma(a.h, b.l, e);
+    e = vfma(a.l, b.h, e);
+    return ff2{p, e};
 }
 
-// a b for a plain float b.
-__device__ __forceinline__ ff ff_mulf(ff a, float b)
+// a b for a plain number b.
+__device__ __forceinline__ ff2 ff_mulf(ff2 a, float2 b)
 {
-    const float p = __fmul_rn(a.h, b);
-    float e = __fmaf_rn(a.h, b, -p);
-    e = __fmaf_rn(a.l, b, e);
-    return ff{p, e};
+    const float2 p = vmul(a.h, b);
+    float2 e = vfma(a.h, b, vneg(p));
+    e = vfma(a.l, b, e);
+    return ff2{p, e};
+}
+
+__device__ __forceinline__ ff2 ff_neg(ff2 a) { return ff2{vneg(a.h), vneg(a.l)}; }
+
+// a + b without the final renormalisation: l may reach a few ulps of max(|a.h|,
+// |b.h|), which the products and sums that take it keep (they drop only l l').
+// A sum whose parts cancel, or that meets another unnormalised factor, is
+// normalised (s_x, s_y, |r|^2, 1/rho, rho, E, g and the running sums: without
+// these the error against FP64 grows, up to thirtyfold where g takes an
+// unnormalised E).  Against normalising every sum but not E and 1/rho: 432 -> 408
+// operations a pair, and the error against FP64 falls by a fifth to a half with
+// screening (20,000 nodes, kappa 0.1257: 5.6e-13 -> 4.5e-13) and stays without.
+__device__ __forceinline__ ff2 ff_add_u(ff2 a, ff2 b)
+{
+    const ff2 s = two_sum(a.h, b.h);
+    return ff2{s.h, vadd(s.l, vadd(a.l, b.l))};
 }
 
 // a + b, renormalised (absolute error about 2^-47 max(|a|, |b|)).
-__device__ __forceinline__ ff ff_add(ff a, ff b)
+__device__ __forceinline__ ff2 ff_add(ff2 a, ff2 b) { return ff_norm(ff_add_u(a, b)); }
+
+__device__ __forceinline__ ff2 ff_sub(ff2 a, ff2 b) { return ff_add(a, ff_neg(b)); }
+
+// a b + c d without the final renormalisation.
+__device__ __forceinline__ ff2 ff_dot2_u(ff2 a, ff2 b, ff2 c, ff2 d)
 {
-    const ff s = two_sum(a.h, b.h);
-    return fast_two_sum(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+    return ff_add_u(ff_mul(a, b), ff_mul(c, d));
 }
 
-__device__ __forceinline__ ff ff_sub(ff a, ff b) { return ff_add(a, ff{-b.h, -b.l}); }
-
-// a0 b0 + a1 b1 + a2 b2 for float-float vectors (the l l' terms dropped).
-__device__ __forceinline__ ff ff_dot3(float ah0, float al0, float ah1, float al1, float ah2, float al2, float bh0,
-                                      float bl0, float bh1, float bl1, float bh2, float bl2)
+// a0 b0 + a1 b1 + a2 b2 (the l l' terms dropped; not renormalised).
+__device__ __forceinline__ ff2 ff_dot3(const ff2 (&a)[3], const ff2 (&b)[3])
 {
-    const ff p0 = ff_mul(ff{ah0, al0}, ff{bh0, bl0});
-    const ff p1 = ff_mul(ff{ah1, al1}, ff{bh1, bl1});
-    const ff p2 = ff_mul(ff{ah2, al2}, ff{bh2, bl2});
-    const ff s = two_sum(p0.h, p1.h);
-    const ff t = two_sum(s.h, p2.h);
-    const float lo = __fadd_rn(__fadd_rn(s.l, t.l), __fadd_rn(__fadd_rn(p0.l, p1.l), p2.l));
-    return fast_two_sum(t.h, lo);
+    const ff2 p0 = ff_mul(a[0], b[0]);
+    const ff2 p1 = ff_mul(a[1], b[1]);
+    const ff2 p2 = ff_mul(a[2], b[2]);
+    const ff2 s = two_sum(p0.h, p1.h);
+    const ff2 t = two_sum(s.h, p2.h);
+    return ff2{t.h, vadd(vadd(s.l, t.l), vadd(vadd(p0.l, p1.l), p2.l))};
 }
 
-// (h + l)^2 summed over three components.
-__device__ __forceinline__ ff ff_norm2(float h0, float l0, float h1, float l1, float h2, float l2)
+// (h + l)^2 summed over three components (not renormalised).
+__device__ __forceinline__ ff2 ff_norm2(const ff2 (&r)[3])
 {
-    const float p0 = __fmul_rn(h0, h0), p1 = __fmul_rn(h1, h1), p2 = __fmul_rn(h2, h2);
-    // (h + l)^2 - h h rounded = fma error of h h + (2 h + l) l
-    const float e0 = __fmaf_rn(__fmaf_rn(2.0f, h0, l0), l0, __fmaf_rn(h0, h0, -p0));
-    const float e1 = __fmaf_rn(__fmaf_rn(2.0f, h1, l1), l1, __fmaf_rn(h1, h1, -p1));
-    const float e2 = __fmaf_rn(__fmaf_rn(2.0f, h2, l2), l2, __fmaf_rn(h2, h2, -p2));
-    const ff s = two_sum(p0, p1);
-    const ff t = two_sum(s.h, p2);
-    const float lo = __fadd_rn(__fadd_rn(s.l, t.l), __fadd_rn(__fadd_rn(e0, e1), e2));
-    return fast_two_sum(t.h, lo);
+    float2 p[3], e[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        // (h + l)^2 - h h rounded = fma error of h h + (2 h + l) l
+        p[q] = vmul(r[q].h, r[q].h);
+        e[q] = vfma(vfma(vset(2.0f), r[q].h, r[q].l), r[q].l, vfma(r[q].h, r[q].h, vneg(p[q])));
+    }
+    const ff2 s = two_sum(p[0], p[1]);
+    const ff2 t = two_sum(s.h, p[2]);
+    return ff2{t.h, vadd(vadd(s.l, t.l), vadd(vadd(e[0], e[1]), e[2]))};
+}
+
+__device__ __forceinline__ float2 vrsqrt(float2 a)
+{
+    return make_float2(ptx::rsqrt_approx(a.x), ptx::rsqrt_approx(a.y));
+}
+__device__ __forceinline__ float2 vmax(float2 a, float b) { return make_float2(fmaxf(a.x, b), fmaxf(a.y, b)); }
+
+// Table entry 2^((ki mod 256)/256) and the power 2^floor(ki/256) of ki, the
+// integer in the low mantissa bits of t (ki >= -30720).
+__device__ __forceinline__ void ff_exp2_parts(float t, const float2* __restrict__ tab, float& Th, float& Tl, float& sc)
+{
+    const int ki = __float_as_int(t) - 0x4B400000;
+    const float2 T = tab[ki & (kFFTab - 1)];
+    Th = T.x;
+    Tl = T.y;
+    sc = __int_as_float(((ki >> 8) + 127) << 23);
+}
+__device__ __forceinline__ void ff_exp2_parts(float2 t, const float2* __restrict__ tab, float2& Th, float2& Tl,
+                                              float2& sc)
+{
+    ff_exp2_parts(t.x, tab, Th.x, Tl.x, sc.x);
+    ff_exp2_parts(t.y, tab, Th.y, Tl.y, sc.y);
 }
 
 // 2^z for z <= 0 (float-float), Tang's table-driven reduction; tab[i] = 2^(i/256).
-__device__ __forceinline__ ff ff_exp2(ff z, const float2* __restrict__ tab)
+// Normalised: the polynomial leaves a low part of 2^-20, which a product with
+// another low part must not drop.
+__device__ __forceinline__ ff2 ff_exp2(ff2 z, const float2* __restrict__ tab)
 {
-    const bool clamp = z.h < -120.0f;
-    const float zh = clamp ? -120.0f : z.h;
-    const float zl = clamp ? 0.0f : z.l;
+    const float2 zh = vmax(z.h, -120.0f);
     // round(zh 256) sits in the low mantissa bits of zh 256 + 1.5 2^23
-    const float t = __fmaf_rn(zh, 256.0f, 12582912.0f);
-    const int ki = __float_as_int(t) - 0x4B400000;
-    const float kf = __fsub_rn(t, 12582912.0f);
-    const float fh = __fmaf_rn(kf, -0.00390625f, zh);  // zh - k/256, exact, |fh| <= 1/512
+    const float2 t = vfma(zh, vset(256.0f), vset(12582912.0f));
+    const float2 kf = vsub(t, vset(12582912.0f));
+    const float2 fh = vfma(kf, vset(-0.00390625f), zh);  // zh - k/256, exact, |fh| <= 1/512
     // u = (fh + zl) ln 2, |u| <= 0.00136
-    const float L2h = 0.693147182464599609375f, L2l = -1.904654323148236e-09f;
-    const float uh = __fmul_rn(fh, L2h);
-    float ul = __fmaf_rn(fh, L2h, -uh);
-    ul = __fmaf_rn(fh, L2l, ul);
-    ul = __fmaf_rn(zl, L2h, ul);
+    const float2 L2h = vset(0.693147182464599609375f), L2l = vset(-1.904654323148236e-09f);
+    const float2 uh = vmul(fh, L2h);
+    float2 ul = vfma(fh, L2h, vneg(uh));
+    ul = vfma(fh, L2l, ul);
+    ul = vfma(z.l, L2h, ul);
     // e^u = 1 + u + u^2 (1/2 + u/6 + u^2/24) + O(u^5)
-    float q = __fmaf_rn(uh, 1.0f / 24.0f, 1.0f / 6.0f);
-    q = __fmaf_rn(uh, q, 0.5f);
-    const float P = __fmul_rn(__fmul_rn(uh, uh), q);
-    const float s = __fadd_rn(1.0f, uh);
-    const float el = __fsub_rn(uh, __fsub_rn(s, 1.0f));
-    const float lo = __fadd_rn(el, __fadd_rn(ul, P));
-    const float2 T = tab[ki & (kFFTab - 1)];
-    const ff m = ff_mul(ff{T.x, T.y}, ff{s, lo});
-    const float sc = __int_as_float(((ki >> 8) + 127) << 23);  // 2^floor(k / 256), k >= -30720
-    return ff{__fmul_rn(m.h, sc), __fmul_rn(m.l, sc)};
+    float2 q = vfma(uh, vset(1.0f / 24.0f), vset(1.0f / 6.0f));
+    q = vfma(uh, q, vset(0.5f));
+    const float2 P = vmul(vmul(uh, uh), q);
+    const float2 s = vadd(vset(1.0f), uh);
+    const float2 el = vsub(uh, vsub(s, vset(1.0f)));
+    const float2 lo = vadd(el, vadd(ul, P));
+    float2 Th, Tl, sc;
+    ff_exp2_parts(t, tab, Th, Tl, sc);
+    const ff2 m = ff_mul(ff2{Th, Tl}, ff2{s, lo});
+    return ff_norm(ff2{vmul(m.h, sc), vmul(m.l, sc)});
 }
 
 // ---------------------------------------------------------------- constants
 
 struct FFConsts {
-    float2 kap, cz;          // kappa and -kappa log2(e)
-    float2 th1, th2;         // eps_E/eps_I, eps_I/eps_E
-    float2 om1, om2;         // 1 - th1, 1 - th2
-    float2 nk12t;            // -(4 pi x tube value of K12)
+    float4 kap, cz;          // kappa and -kappa log2(e)   (h, h, l, l)
+    float4 th1, th2;         // eps_E/eps_I, eps_I/eps_E
+    float4 om1, om2;         // 1 - th1, 1 - th2
+    float4 nk12t;            // -(4 pi x tube value of K12)
     float2 tau2, four_tau2;  // tube thresholds
     double tau2_d, four_tau2_d;
     float far_dist;          // minimum bounding-sphere gap of a far chunk pair (A)
@@ -195,16 +264,22 @@ static float2 split(double v)
     return make_float2(h, (float)(v - (double)h));
 }
 
+static float4 split2(double v)
+{
+    const float2 s = split(v);
+    return make_float4(s.x, s.x, s.y, s.y);
+}
+
 static FFConsts ff_consts(const PairConsts& k)
 {
     FFConsts c;
-    c.kap = split(k.kappa);
-    c.cz = split(-k.kappa * 1.4426950408889634074);
-    c.th1 = split(k.th1);
-    c.th2 = split(k.th2);
-    c.om1 = split(1.0 - k.th1);
-    c.om2 = split(1.0 - k.th2);
-    c.nk12t = split(-k.k12_tube);
+    c.kap = split2(k.kappa);
+    c.cz = split2(-k.kappa * 1.4426950408889634074);
+    c.th1 = split2(k.th1);
+    c.th2 = split2(k.th2);
+    c.om1 = split2(1.0 - k.th1);
+    c.om2 = split2(1.0 - k.th2);
+    c.nk12t = split2(-k.k12_tube);
     c.rule0 = (k.four_tau2 < 3.0e38) ? 1 : 0;
     c.tau2 = split(k.tau2);
     c.four_tau2 = c.rule0 ? split(k.four_tau2) : make_float2(__builtin_huge_valf(), 0.0f);
@@ -232,69 +307,180 @@ static __device__ __noinline__ bool tube_f64_ordered(const double* __restrict__ 
 
 // ---------------------------------------------------------------- pair
 
-struct FFTarget {
-    float xh0, xh1, xh2, xl0, xl1, xl2;
-    float nh0, nh1, nh2, nl0, nl1, nl2;
+// A target and a pair of sources: position, normal, a = w psi, b = w psin.
+struct FFNode {
+    ff x[3], n[3], a, b;
+};
+struct FFPair {
+    ff2 x[3], n[3], a, b;
 };
 
-// One (target <- source) interaction added to (S1, S2).  NEAR: the pair may
-// lie in the regularisation tube.
-template <bool NEAR>
-__device__ __forceinline__ void ff_pair(const FFTarget& T, const float4& F0, const float4& F1, const float4& F2,
-                                        const float4& F3, const FFConsts& k, const float2* __restrict__ tab, ff& S1,
-                                        ff& S2, const double* __restrict__ geo, int64_t i, int64_t j, int64_t N)
+// pair pr of the chunk at cb
+__device__ __forceinline__ FFPair ff_load(const float4* __restrict__ cb, int pr)
 {
-    // r = x - y: the hi parts share the grid, so their difference is exact
-    const float rh0 = __fsub_rn(T.xh0, F0.x), rh1 = __fsub_rn(T.xh1, F0.y), rh2 = __fsub_rn(T.xh2, F0.z);
-    const float rl0 = __fsub_rn(T.xl0, F1.x), rl1 = __fsub_rn(T.xl1, F1.y), rl2 = __fsub_rn(T.xl2, F1.z);
-    const ff rr = ff_norm2(rh0, rl0, rh1, rl1, rh2, rl2);
-    const ff sx = ff_dot3(rh0, rl0, rh1, rl1, rh2, rl2, T.nh0, T.nl0, T.nh1, T.nl1, T.nh2, T.nl2);
-    const ff b = ff{F2.w, F3.w};
-    if (NEAR) {
-        // rho_P^2 = |r|^2 - s_x^2 < tau^2 and |r|^2 < 4 tau^2 (tube rule 0)
-        const ff sx2 = ff_mul(sx, sx);
-        const ff rp2 = ff_sub(rr, sx2);
-        const float d1 = __fadd_rn(__fsub_rn(rp2.h, k.tau2.x), __fsub_rn(rp2.l, k.tau2.y));
-        const float d2 = __fadd_rn(__fsub_rn(rr.h, k.four_tau2.x), __fsub_rn(rr.l, k.four_tau2.y));
-        bool tube = (d1 < 0.0f) && (d2 < 0.0f);
-        const bool tie = (fabsf(d1) < 1e-9f * k.tau2.x) || (fabsf(d2) < 1e-9f * k.four_tau2.x);
-        if (tie && i < N && j < N) tube = tube_f64_ordered(geo, N, i, j, k.tau2_d, k.four_tau2_d);
-        if (tube) {
-            const ff c = ff_mul(ff_of(k.nk12t), b);
-            const ff s = two_sum(S1.h, c.h);
-            S1 = fast_two_sum(s.h, __fadd_rn(s.l, __fadd_rn(S1.l, c.l)));
-            return;
+    float4 v[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) v[c] = cb[c * kFFPairs + pr];
+    const auto lo = [](const float4& f) { return make_float2(f.x, f.y); };
+    const auto hi = [](const float4& f) { return make_float2(f.z, f.w); };
+    FFPair s;
+#pragma unroll
+    for (int f = 0; f < 2; ++f) {  // x, a then n, b
+        ff2* d = f ? s.n : s.x;
+        d[0] = ff2{lo(v[4 * f]), lo(v[4 * f + 2])};
+        d[1] = ff2{hi(v[4 * f]), hi(v[4 * f + 2])};
+        d[2] = ff2{lo(v[4 * f + 1]), lo(v[4 * f + 3])};
+        (f ? s.b : s.a) = ff2{hi(v[4 * f + 1]), hi(v[4 * f + 3])};
+    }
+    return s;
+}
+
+// Geometry of the (target T <- source s) pairs.
+struct FFGeo {
+    ff2 rr, sx, sy;
+};
+
+__device__ __forceinline__ FFGeo ff_geo(const FFNode& T, const FFPair& s)
+{
+    ff2 r[3], n[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        // r = x - y: the hi parts share the grid, so their difference is exact
+        r[c].h = vsub(vset(T.x[c].h), s.x[c].h);
+        r[c].l = vsub(vset(T.x[c].l), s.x[c].l);
+        n[c] = ff_wide(T.n[c]);
+    }
+    FFGeo g;
+    g.rr = ff_norm(ff_norm2(r));
+    g.sx = ff_norm(ff_dot3(r, n));
+    g.sy = ff_norm(ff_dot3(r, s.n));
+    return g;
+}
+
+// Factors of the two directions: y1 takes P1 s_y a - Q b, y2 takes B3 a + P2 s_x b.
+struct FFFactors {
+    ff2 P1, Q, P2, B3;
+};
+
+__device__ __forceinline__ FFFactors ff_factors(const FFGeo& G, const FFNode& T, const FFPair& s,
+                                                   const FFConsts& k, const float2* __restrict__ tab)
+{
+    const ff2 nt[3] = {ff_wide(T.n[0]), ff_wide(T.n[1]), ff_wide(T.n[2])};
+    const ff2 cc = ff_dot3(nt, s.n);
+    // 1/rho: MUFU estimate, one Newton step in float-float
+    const float2 y0 = vrsqrt(G.rr.h);
+    const float2 yy = vmul(y0, y0);  // d = |r|^2 y0^2 - 1, about 2^-21
+    const float2 d = vfma(G.rr.h, vfma(y0, y0, vneg(yy)), vfma(G.rr.l, yy, vfma(G.rr.h, yy, vset(-1.0f))));
+    const ff2 inv = fast_two_sum(y0, vmul(vmul(y0, d), vfma(vset(0.375f), d, vset(-0.5f))));
+    const ff2 rho = ff_norm(ff_mul(G.rr, inv));
+    const ff2 x = ff_mul(ff_of(k.kap), rho);
+    const ff2 E = ff_exp2(ff_mul(ff_of(k.cz), rho), tab);
+    const ff2 Ex = ff_mul(E, x);
+    // f = 1 - E (0 < E <= 1: fast two-sum of 1 and -E.h)
+    const float2 one = vset(1.0f);
+    const float2 fh = vsub(one, E.h);
+    const ff2 f{fh, vsub(vsub(vsub(one, fh), E.h), E.l)};
+    const ff2 g = ff_sub(f, Ex);                                         // 1 - A
+    const ff2 u1 = ff_add_u(ff_of(k.om1), ff_mul(ff_of(k.th1), g));  // 1 - th1 A
+    const ff2 u2 = ff_add_u(ff_of(k.om2), ff_mul(ff_of(k.th2), g));  // 1 - th2 A
+    const ff2 hb = ff_add_u(ff_mulf(g, vset(3.0f)), ff_neg(ff_mul(Ex, x)));  // 3 - B
+    const ff2 inv2 = ff_mul(inv, inv);
+    const ff2 inv3 = ff_mul(inv2, inv);
+    const ff2 br = ff_dot2_u(g, cc, ff_neg(hb), ff_mul(ff_mul(G.sx, G.sy), inv2));
+    return FFFactors{ff_mul(u1, inv3), ff_mul(f, inv), ff_mul(u2, inv3), ff_mul(br, inv3)};
+}
+
+// Forward contributions of the pairs.
+__device__ __forceinline__ void ff_forward(const FFGeo& G, const FFFactors& F, const FFPair& s, ff2& c1, ff2& c2)
+{
+    c1 = ff_dot2_u(F.P1, ff_mul(G.sy, s.a), ff_neg(F.Q), s.b);
+    c2 = ff_dot2_u(F.B3, s.a, ff_mul(F.P2, G.sx), s.b);
+}
+
+// Reverse contributions (s_x' = -s_y, s_y' = -s_x).
+__device__ __forceinline__ void ff_reverse(const FFGeo& G, const FFFactors& F, const FFNode& T, ff2& c1, ff2& c2)
+{
+    const ff2 ai = ff_wide(T.a), bi = ff_wide(T.b);
+    c1 = ff_neg(ff_dot2_u(F.P1, ff_mul(G.sx, ai), F.Q, bi));
+    c2 = ff_dot2_u(F.B3, ai, ff_neg(ff_mul(F.P2, G.sy)), bi);
+}
+
+// Tube tests of the pairs i <- j and i <- j + 16 (reverse: j <- i and j + 16 <- i);
+// sn = r . n with the target's normal.
+__device__ __forceinline__ void ff_tube(const ff2& rr, const ff2& sn, const FFConsts& k, const double* __restrict__ geo,
+                                        int64_t i, int64_t j, int64_t N, bool reverse, bool (&tube)[2])
+{
+    // rho_P^2 = |r|^2 - s_n^2 < tau^2 and |r|^2 < 4 tau^2 (tube rule 0)
+    const ff2 rp2 = ff_sub(rr, ff_mul(sn, sn));
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const ff p = ff_half(rp2, q), d = ff_half(rr, q);
+        const float d1 = __fadd_rn(__fsub_rn(p.h, k.tau2.x), __fsub_rn(p.l, k.tau2.y));
+        const float d2 = __fadd_rn(__fsub_rn(d.h, k.four_tau2.x), __fsub_rn(d.l, k.four_tau2.y));
+        tube[q] = (d1 < 0.0f) && (d2 < 0.0f);
+        if ((fabsf(d1) < 1e-9f * k.tau2.x) || (fabsf(d2) < 1e-9f * k.four_tau2.x)) {  // tie
+            const int64_t jq = j + q * kFFPairs;
+            if (i < N && jq < N)
+                tube[q] = reverse ? tube_f64_ordered(geo, N, jq, i, k.tau2_d, k.four_tau2_d)
+                                  : tube_f64_ordered(geo, N, i, jq, k.tau2_d, k.four_tau2_d);
         }
     }
-    const ff sy = ff_dot3(rh0, rl0, rh1, rl1, rh2, rl2, F2.x, F3.x, F2.y, F3.y, F2.z, F3.z);
-    const ff cc = ff_dot3(T.nh0, T.nl0, T.nh1, T.nl1, T.nh2, T.nl2, F2.x, F3.x, F2.y, F3.y, F2.z, F3.z);
-    // 1/rho: MUFU estimate, one Newton step in float-float
-    const float y0 = ptx::rsqrt_approx(rr.h);
-    const ff q = ff_mul(rr, ff{__fmul_rn(y0, y0), __fmaf_rn(y0, y0, -__fmul_rn(y0, y0))});
-    const float d = __fadd_rn(__fsub_rn(q.h, 1.0f), q.l);
-    const ff inv = ff{y0, __fmul_rn(__fmul_rn(y0, d), __fmaf_rn(0.375f, d, -0.5f))};
-    const ff rho = ff_mul(rr, inv);
-    const ff x = ff_mul(ff_of(k.kap), rho);
-    const ff E = ff_exp2(ff_mul(ff_of(k.cz), rho), tab);
-    const ff Ex = ff_mul(E, x);
-    // f = 1 - E (0 < E <= 1: fast two-sum of 1 and -E.h)
-    const float fh = __fsub_rn(1.0f, E.h);
-    const ff f = ff{fh, __fsub_rn(__fsub_rn(__fsub_rn(1.0f, fh), E.h), E.l)};
-    const ff g = ff_sub(f, Ex);                               // 1 - A
-    const ff u1 = ff_add(ff_of(k.om1), ff_mul(ff_of(k.th1), g));  // 1 - th1 A
-    const ff u2 = ff_add(ff_of(k.om2), ff_mul(ff_of(k.th2), g));  // 1 - th2 A
-    const ff hb = ff_sub(ff_mulf(g, 3.0f), ff_mul(Ex, x));     // 3 - B
-    const ff inv2 = ff_mul(inv, inv);
-    const ff inv3 = ff_mul(inv2, inv);
-    const ff a = ff{F0.w, F1.w};
-    const ff c1 = ff_sub(ff_mul(ff_mul(u1, ff_mul(sy, a)), inv3), ff_mul(ff_mul(f, inv), b));
-    const ff br = ff_sub(ff_mul(g, cc), ff_mul(hb, ff_mul(ff_mul(sx, sy), inv2)));
-    const ff c2 = ff_mul(ff_add(ff_mul(br, a), ff_mul(ff_mul(u2, sx), b)), inv3);
-    const ff s1 = two_sum(S1.h, c1.h);
-    S1 = fast_two_sum(s1.h, __fadd_rn(s1.l, __fadd_rn(S1.l, c1.l)));
-    const ff s2 = two_sum(S2.h, c2.h);
-    S2 = fast_two_sum(s2.h, __fadd_rn(s2.l, __fadd_rn(S2.l, c2.l)));
 }
+
+// Contributions inside the tube: y1 -= K12_tube b, nothing to y2.
+__device__ __forceinline__ void ff_tube_select(const bool (&tube)[2], const ff2& b, const FFConsts& k, ff2& c1, ff2& c2)
+{
+    const ff2 t = ff_mul(ff_of(k.nk12t), b);
+    c1.h = make_float2(tube[0] ? t.h.x : c1.h.x, tube[1] ? t.h.y : c1.h.y);
+    c1.l = make_float2(tube[0] ? t.l.x : c1.l.x, tube[1] ? t.l.y : c1.l.y);
+    c2.h = make_float2(tube[0] ? 0.0f : c2.h.x, tube[1] ? 0.0f : c2.h.y);
+    c2.l = make_float2(tube[0] ? 0.0f : c2.l.x, tube[1] ? 0.0f : c2.l.y);
+}
+
+// Two pairs: forward into (S1, S2) and, when rev, reverse into (R1, R2).  NEAR:
+// they may lie in the regularisation tube (nodes i <- j, j + 16; both sides are
+// evaluated and selected, the self pair among the regularised ones).
+template <bool NEAR>
+__device__ __forceinline__ void ff_pairs2(const FFNode& T, const FFPair& m, const FFConsts& k,
+                                          const float2* __restrict__ tab, bool rev, ff2& S1, ff2& S2, ff2& R1, ff2& R2,
+                                          const double* __restrict__ geo, int64_t i, int64_t j, int64_t N)
+{
+    const FFGeo G = ff_geo(T, m);
+    bool tf[2], tr[2];
+    if (NEAR) {
+        ff_tube(G.rr, G.sx, k, geo, i, j, N, false, tf);
+        if (rev) ff_tube(G.rr, G.sy, k, geo, i, j, N, true, tr);
+    }
+    const FFFactors F = ff_factors(G, T, m, k, tab);
+    ff2 c1, c2;
+    ff_forward(G, F, m, c1, c2);
+    if (NEAR) ff_tube_select(tf, m.b, k, c1, c2);
+    S1 = ff_add(S1, c1);
+    S2 = ff_add(S2, c2);
+    if (rev) {
+        ff_reverse(G, F, T, c1, c2);
+        if (NEAR) ff_tube_select(tr, ff_wide(T.b), k, c1, c2);
+        R1 = ff_add(R1, c1);
+        R2 = ff_add(R2, c2);
+    }
+}
+
+// Target i (placeholders from N on lie away from placeholder sources).
+__device__ __forceinline__ FFNode ff_target(const float* __restrict__ src, int64_t i, int64_t N)
+{
+    FFNode T;
+    const bool pad = i >= N;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        T.x[c] = pad ? ff{-kFFPad, 0.0f} : ff{src[ff_off(i, 0, c)], src[ff_off(i, 1, c)]};
+        T.n[c] = ff{src[ff_off(i, 2, c)], src[ff_off(i, 3, c)]};
+    }
+    T.a = ff{src[ff_off(i, 0, 3)], src[ff_off(i, 1, 3)]};
+    T.b = ff{src[ff_off(i, 2, 3)], src[ff_off(i, 3, 3)]};
+    return T;
+}
+
+__device__ __forceinline__ double ff_value(ff2 v) { return ((double)v.h.x + (double)v.l.x) + ((double)v.h.y + (double)v.l.y); }
 
 // ---------------------------------------------------------------- kernels
 
@@ -335,7 +521,7 @@ __global__ void __launch_bounds__(kFFThreads, 2)
 
     const int64_t t_first = s0 / s.n_stiles;
     int64_t t = t_first;
-    FFTarget T;
+    FFNode T;
     float4 tfh, tfl;  // frame of the warp's target block
     int64_t gi = 0;
     bool idle = false;
@@ -343,21 +529,7 @@ __global__ void __launch_bounds__(kFFThreads, 2)
     auto load_target = [&](int64_t tile) {
         gi = tile * kFFTTile + tid;
         idle = tile * kFFTTile + warp * kFFChunk >= N;
-        const float4 a = src[ff_off(gi, 0)], b = src[ff_off(gi, 1)];
-        const float4 c = src[ff_off(gi, 2)], e = src[ff_off(gi, 3)];
-        const bool pad = gi >= N;  // placeholder targets away from placeholder sources
-        T.xh0 = pad ? -kFFPad : a.x;
-        T.xh1 = pad ? -kFFPad : a.y;
-        T.xh2 = pad ? -kFFPad : a.z;
-        T.xl0 = pad ? 0.0f : b.x;
-        T.xl1 = pad ? 0.0f : b.y;
-        T.xl2 = pad ? 0.0f : b.z;
-        T.nh0 = c.x;
-        T.nh1 = c.y;
-        T.nh2 = c.z;
-        T.nl0 = e.x;
-        T.nl1 = e.y;
-        T.nl2 = e.z;
+        T = ff_target(reinterpret_cast<const float*>(src), gi, N);
         const int64_t blk = (tile * kFFTTile + warp * kFFChunk) / kFFChunk;
         tfh = frames[2 * blk];
         tfl = frames[2 * blk + 1];
@@ -377,7 +549,7 @@ __global__ void __launch_bounds__(kFFThreads, 2)
         const int64_t sp = u % s.n_stiles;
         const int64_t st = (sp * s.sperm) % s.n_stiles;
         if (!idle) {
-            ff S1{0.0f, 0.0f}, S2{0.0f, 0.0f};
+            ff2 S1{}, S2{}, R1{}, R2{};  // the reverse sums stay zero
             const float4* sb = &sbuf[stage][0];
 #pragma unroll 1
             for (int c = 0; c < kFFChunksPerTile; ++c) {
@@ -391,19 +563,17 @@ __global__ void __launch_bounds__(kFFThreads, 2)
                 const float4* cb = sb + c * kFFChunk * kFFNodeF4;
                 const int64_t j0 = st * kFFSTile + c * kFFChunk;
                 if (far) {
-#pragma unroll 2
-                    for (int p = 0; p < kFFChunk; ++p)
-                        ff_pair<false>(T, cb[p], cb[32 + p], cb[64 + p], cb[96 + p], k, tab, S1, S2, geo, gi, j0 + p,
-                                       N);
+#pragma unroll 1
+                    for (int p = 0; p < kFFPairs; ++p)
+                        ff_pairs2<false>(T, ff_load(cb, p), k, tab, false, S1, S2, R1, R2, geo, gi, j0 + p, N);
                 } else {
 #pragma unroll 1
-                    for (int p = 0; p < kFFChunk; ++p)
-                        ff_pair<true>(T, cb[p], cb[32 + p], cb[64 + p], cb[96 + p], k, tab, S1, S2, geo, gi, j0 + p,
-                                      N);
+                    for (int p = 0; p < kFFPairs; ++p)
+                        ff_pairs2<true>(T, ff_load(cb, p), k, tab, false, S1, S2, R1, R2, geo, gi, j0 + p, N);
                 }
             }
-            D1 += (double)S1.h + (double)S1.l;
-            D2 += (double)S2.h + (double)S2.l;
+            D1 += ff_value(S1);
+            D2 += ff_value(S2);
         }
         __syncthreads();
         if (tid == 0 && u + kFFStages < s1) {
@@ -437,117 +607,58 @@ __global__ void __launch_bounds__(kFFThreads, 2)
 //             y2_j += [br a_i - u2 s_y b_i] / rho^3
 // with br = g c - (3 - B) s_x s_y / rho^2.  Each direction takes its own tube
 // test (the reverse one on the source's normal, rho_P'^2 = |r|^2 - s_y^2).
-// 432 FP32 operations per unordered pair against 2 x 366.
+// 408 FP32 operations per unordered pair against 2 x 346.
 //
-// Per warp and source chunk the 32 lanes hold 32 targets and walk the chunk's
-// 32 sources in a staggered order (lane l takes source (l + k) mod 32 at step
-// k); the float-float reverse sums of a source ride along with it from lane to
-// lane (four shuffles a step), so after 32 steps lane l holds source l's
-// reverse sums over the warp's targets and adds them, as doubles, to the
-// reverse vector with FP64 atomics.  Forward sums and the schedule (upper
-// triangle, large and small segments, partials per (segment, row)) are those
-// of the symmetric FP32 kernel, and its fixup adds everything up.
-
-// One unordered pair: forward into (S1, S2), reverse (when rev) into (R1, R2).
-template <bool NEAR>
-__device__ __forceinline__ void ffs_pair(const FFTarget& T, ff ai, ff bi, const float4& F0, const float4& F1,
-                                         const float4& F2, const float4& F3, const FFConsts& k,
-                                         const float2* __restrict__ tab, bool rev, ff& S1, ff& S2, ff& R1, ff& R2,
-                                         const double* __restrict__ geo, int64_t i, int64_t j, int64_t N)
+// Per warp and source chunk the 32 lanes hold 32 targets; each half-warp walks
+// the chunk's 16 pairs of sources in a staggered order (lane l takes pair
+// (l + k) mod 16 at step k); the float-float reverse sums of a pair ride along
+// with it from lane to lane (four shuffles a node pair), so after 16 steps lane l
+// holds pair l mod 16's reverse sums over its half's targets; the halves are
+// added and go, as doubles, to the reverse vector with FP64 atomics.  Forward
+// sums and the schedule (upper triangle, large and small segments, partials per
+// (segment, row)) are those of the symmetric FP32 kernel, and its fixup adds
+// everything up.
+__device__ __forceinline__ ff2 ff_rotate(ff2 v, int lane)
 {
-    const float rh0 = __fsub_rn(T.xh0, F0.x), rh1 = __fsub_rn(T.xh1, F0.y), rh2 = __fsub_rn(T.xh2, F0.z);
-    const float rl0 = __fsub_rn(T.xl0, F1.x), rl1 = __fsub_rn(T.xl1, F1.y), rl2 = __fsub_rn(T.xl2, F1.z);
-    const ff rr = ff_norm2(rh0, rl0, rh1, rl1, rh2, rl2);
-    const ff sx = ff_dot3(rh0, rl0, rh1, rl1, rh2, rl2, T.nh0, T.nl0, T.nh1, T.nl1, T.nh2, T.nl2);
-    const ff sy = ff_dot3(rh0, rl0, rh1, rl1, rh2, rl2, F2.x, F3.x, F2.y, F3.y, F2.z, F3.z);
-    const ff aj = ff{F0.w, F1.w}, bj = ff{F2.w, F3.w};
-    bool tube_f = false, tube_r = false;
-    if (NEAR) {
-        const float d2 = __fadd_rn(__fsub_rn(rr.h, k.four_tau2.x), __fsub_rn(rr.l, k.four_tau2.y));
-        const bool tie2 = fabsf(d2) < 1e-9f * k.four_tau2.x;
-        const ff pf = ff_sub(rr, ff_mul(sx, sx));
-        const float d1f = __fadd_rn(__fsub_rn(pf.h, k.tau2.x), __fsub_rn(pf.l, k.tau2.y));
-        tube_f = (d1f < 0.0f) && (d2 < 0.0f);
-        if ((tie2 || fabsf(d1f) < 1e-9f * k.tau2.x) && i < N && j < N)
-            tube_f = tube_f64_ordered(geo, N, i, j, k.tau2_d, k.four_tau2_d);
-        if (rev) {
-            const ff pr = ff_sub(rr, ff_mul(sy, sy));
-            const float d1r = __fadd_rn(__fsub_rn(pr.h, k.tau2.x), __fsub_rn(pr.l, k.tau2.y));
-            tube_r = (d1r < 0.0f) && (d2 < 0.0f);
-            if ((tie2 || fabsf(d1r) < 1e-9f * k.tau2.x) && i < N && j < N)
-                tube_r = tube_f64_ordered(geo, N, j, i, k.tau2_d, k.four_tau2_d);
-        }
-        if (tube_f && (tube_r || !rev)) {  // both directions regularised (the self pair among them)
-            const ff c = ff_mul(ff_of(k.nk12t), bj);
-            const ff s = two_sum(S1.h, c.h);
-            S1 = fast_two_sum(s.h, __fadd_rn(s.l, __fadd_rn(S1.l, c.l)));
-            if (rev) {
-                const ff cr = ff_mul(ff_of(k.nk12t), bi);
-                const ff t = two_sum(R1.h, cr.h);
-                R1 = fast_two_sum(t.h, __fadd_rn(t.l, __fadd_rn(R1.l, cr.l)));
-            }
-            return;
-        }
-    }
-    const ff cc = ff_dot3(T.nh0, T.nl0, T.nh1, T.nl1, T.nh2, T.nl2, F2.x, F3.x, F2.y, F3.y, F2.z, F3.z);
-    const float y0 = ptx::rsqrt_approx(rr.h);
-    const ff q = ff_mul(rr, ff{__fmul_rn(y0, y0), __fmaf_rn(y0, y0, -__fmul_rn(y0, y0))});
-    const float d = __fadd_rn(__fsub_rn(q.h, 1.0f), q.l);
-    const ff inv = ff{y0, __fmul_rn(__fmul_rn(y0, d), __fmaf_rn(0.375f, d, -0.5f))};
-    const ff rho = ff_mul(rr, inv);
-    const ff x = ff_mul(ff_of(k.kap), rho);
-    const ff E = ff_exp2(ff_mul(ff_of(k.cz), rho), tab);
-    const ff Ex = ff_mul(E, x);
-    const float fh = __fsub_rn(1.0f, E.h);
-    const ff f = ff{fh, __fsub_rn(__fsub_rn(__fsub_rn(1.0f, fh), E.h), E.l)};
-    const ff g = ff_sub(f, Ex);
-    const ff u1 = ff_add(ff_of(k.om1), ff_mul(ff_of(k.th1), g));
-    const ff u2 = ff_add(ff_of(k.om2), ff_mul(ff_of(k.th2), g));
-    const ff hb = ff_sub(ff_mulf(g, 3.0f), ff_mul(Ex, x));
-    const ff inv2 = ff_mul(inv, inv);
-    const ff inv3 = ff_mul(inv2, inv);
-    const ff br = ff_sub(ff_mul(g, cc), ff_mul(hb, ff_mul(ff_mul(sx, sy), inv2)));
-    const ff P1 = ff_mul(u1, inv3), Q = ff_mul(f, inv), P2 = ff_mul(u2, inv3), B3 = ff_mul(br, inv3);
-    ff c1, c2;
-    if (NEAR && tube_f) {
-        c1 = ff_mul(ff_of(k.nk12t), bj);
-        c2 = ff{0.0f, 0.0f};
-    } else {
-        c1 = ff_sub(ff_mul(P1, ff_mul(sy, aj)), ff_mul(Q, bj));
-        c2 = ff_add(ff_mul(B3, aj), ff_mul(ff_mul(P2, sx), bj));
-    }
-    const ff s1 = two_sum(S1.h, c1.h);
-    S1 = fast_two_sum(s1.h, __fadd_rn(s1.l, __fadd_rn(S1.l, c1.l)));
-    const ff s2 = two_sum(S2.h, c2.h);
-    S2 = fast_two_sum(s2.h, __fadd_rn(s2.l, __fadd_rn(S2.l, c2.l)));
-    if (!rev) return;
-    ff e1, e2;
-    if (NEAR && tube_r) {
-        e1 = ff_mul(ff_of(k.nk12t), bi);
-        e2 = ff{0.0f, 0.0f};
-    } else {
-        const ff m = ff_mul(P1, ff_mul(sx, ai));
-        e1 = ff_sub(ff{-m.h, -m.l}, ff_mul(Q, bi));
-        e2 = ff_sub(ff_mul(B3, ai), ff_mul(ff_mul(P2, sy), bi));
-    }
-    const ff r1 = two_sum(R1.h, e1.h);
-    R1 = fast_two_sum(r1.h, __fadd_rn(r1.l, __fadd_rn(R1.l, e1.l)));
-    const ff r2 = two_sum(R2.h, e2.h);
-    R2 = fast_two_sum(r2.h, __fadd_rn(r2.l, __fadd_rn(R2.l, e2.l)));
+    ff2 o;
+    o.h.x = __shfl_sync(0xffffffffu, v.h.x, lane + 1, kFFPairs);
+    o.h.y = __shfl_sync(0xffffffffu, v.h.y, lane + 1, kFFPairs);
+    o.l.x = __shfl_sync(0xffffffffu, v.l.x, lane + 1, kFFPairs);
+    o.l.y = __shfl_sync(0xffffffffu, v.l.y, lane + 1, kFFPairs);
+    return o;
 }
 
-constexpr int kFFSThreads = 256;  // one target per thread; target tile = source tile (R = 1)
+// After 16 rotations lane l holds the pair l mod 16 summed over its half-warp's
+// targets: the sum over both halves of node l (first halves' lanes keep .x).
+__device__ __forceinline__ double ff_halves_sum(ff2 v, int lane)
+{
+    const bool low = lane < kFFPairs;
+    const ff keep = ff_half(v, low ? 0 : 1), give = ff_half(v, low ? 1 : 0);
+    const float gh = __shfl_xor_sync(0xffffffffu, give.h, kFFPairs);
+    const float gl = __shfl_xor_sync(0xffffffffu, give.l, kFFPairs);
+    return ((double)keep.h + (double)keep.l) + ((double)gh + (double)gl);
+}
 
-__global__ void __launch_bounds__(kFFSThreads, 2)
+// THREADS targets (one per thread) and STILE sources per step.  Small steps, as
+// a launch on a small molecule has few: 128 x 32 against 256 x 256 takes 38 us
+// for 216 at 862 nodes, 105 for 214 at 3,214, 207 for 343 at 5,014.  The CTAs of
+// an SM do not advance alike (the scheduler favours the older warps), so most of
+// the work is in small segments: at 80,358 nodes 43.1 ms with nine tenths of an
+// even share per CTA in large ones, 41.5 with half, 39.9 with one tenth.
+template <int THREADS, int STILE>
+__global__ void __launch_bounds__(THREADS, 512 / THREADS)
     pair_ffs_kernel(const float4* __restrict__ src, const float4* __restrict__ frames,
                     const float2* __restrict__ tab_g, const double* __restrict__ geo, int64_t N, int64_t n_pad,
                     SymSchedule s, FFConsts k, double* __restrict__ part, double* __restrict__ yrev,
                     unsigned* __restrict__ err, const int* __restrict__ skip)
 {
-    constexpr int TTILE = kFFSThreads;
+    constexpr int TTILE = THREADS;
+    constexpr int CHUNKS = STILE / kFFChunk;
+    constexpr uint32_t STAGE_BYTES = STILE * kFFNodeF4 * sizeof(float4);
+    constexpr uint32_t FRAME_BYTES = 2 * CHUNKS * sizeof(float4);
     if (skip != nullptr && *skip) return;
-    __shared__ __align__(128) float4 sbuf[kFFStages][kFFSTile * kFFNodeF4];
-    __shared__ __align__(16) float4 sfrm[kFFStages][2 * kFFChunksPerTile];
+    __shared__ __align__(128) float4 sbuf[kFFStages][STILE * kFFNodeF4];
+    __shared__ __align__(16) float4 sfrm[kFFStages][2 * CHUNKS];
     __shared__ float2 tab[kFFTab];
     __shared__ __align__(8) uint64_t bars[kFFStages];
     __shared__ int abort_flag;
@@ -557,7 +668,7 @@ __global__ void __launch_bounds__(kFFSThreads, 2)
     const int warp = tid >> 5;
     const int lane = tid & 31;
     unsigned long long* seg_ctr = reinterpret_cast<unsigned long long*>(yrev + 2 * n_pad);
-    for (int q = tid; q < kFFTab; q += kFFSThreads) tab[q] = tab_g[q];
+    for (int q = tid; q < kFFTab; q += THREADS) tab[q] = tab_g[q];
     if (tid == 0) {
         for (int q = 0; q < kFFStages; ++q) ptx::mbar_init(&bars[q], 1);
         ptx::fence_mbar_init();
@@ -572,13 +683,12 @@ __global__ void __launch_bounds__(kFFSThreads, 2)
         sym_locate(s, u, t, rho, pos);
         const int64_t st = s.R * t + pos;
         const int stage = (int)(n % kFFStages);
-        ptx::mbar_arrive_expect_tx(&bars[stage], kFFStageBytes + kFFFrameBytes);
-        ptx::bulk_g2s(&sbuf[stage][0], src + st * kFFSTile * kFFNodeF4, kFFStageBytes, &bars[stage]);
-        ptx::bulk_g2s(&sfrm[stage][0], frames + st * 2 * kFFChunksPerTile, kFFFrameBytes, &bars[stage]);
+        ptx::mbar_arrive_expect_tx(&bars[stage], STAGE_BYTES + FRAME_BYTES);
+        ptx::bulk_g2s(&sbuf[stage][0], src + st * STILE * kFFNodeF4, STAGE_BYTES, &bars[stage]);
+        ptx::bulk_g2s(&sfrm[stage][0], frames + st * 2 * CHUNKS, FRAME_BYTES, &bars[stage]);
     };
 
-    FFTarget T;
-    ff ai, bi;
+    FFNode T;
     float4 tfh, tfl;
     int64_t gi = 0;
     int Ablk = 0;
@@ -587,23 +697,7 @@ __global__ void __launch_bounds__(kFFSThreads, 2)
     auto load_target = [&](int64_t tile) {
         gi = tile * TTILE + tid;
         idle = tile * TTILE + warp * kFFChunk >= N;
-        const float4 a = src[ff_off(gi, 0)], b = src[ff_off(gi, 1)];
-        const float4 c = src[ff_off(gi, 2)], e = src[ff_off(gi, 3)];
-        const bool pad = gi >= N;
-        T.xh0 = pad ? -kFFPad : a.x;
-        T.xh1 = pad ? -kFFPad : a.y;
-        T.xh2 = pad ? -kFFPad : a.z;
-        T.xl0 = pad ? 0.0f : b.x;
-        T.xl1 = pad ? 0.0f : b.y;
-        T.xl2 = pad ? 0.0f : b.z;
-        T.nh0 = c.x;
-        T.nh1 = c.y;
-        T.nh2 = c.z;
-        T.nl0 = e.x;
-        T.nl1 = e.y;
-        T.nl2 = e.z;
-        ai = ff{a.w, b.w};
-        bi = ff{c.w, e.w};
+        T = ff_target(reinterpret_cast<const float*>(src), gi, N);
         Ablk = (int)((tile * TTILE + warp * kFFChunk) / kFFChunk);
         const int64_t blk = Ablk;
         tfh = frames[2 * blk];
@@ -630,11 +724,11 @@ __global__ void __launch_bounds__(kFFSThreads, 2)
             if (abort_flag) return;
             const int64_t st = s.R * t + pos;
             if (!idle) {
-                ff S1{0.0f, 0.0f}, S2{0.0f, 0.0f};
+                ff2 S1{}, S2{};
                 const float4* sb = &sbuf[stage][0];
 #pragma unroll 1
-                for (int c = 0; c < kFFChunksPerTile; ++c) {
-                    const int64_t Bc = st * kFFChunksPerTile + c;
+                for (int c = 0; c < CHUNKS; ++c) {
+                    const int64_t Bc = st * CHUNKS + c;
                     if (Bc < Ablk) continue;  // the warp holding block Bc covers this block pair
                     const bool rev = Bc > Ablk;
                     const float4 mh = sfrm[stage][2 * c], ml = sfrm[stage][2 * c + 1];
@@ -642,40 +736,37 @@ __global__ void __launch_bounds__(kFFSThreads, 2)
                     const float dy = (tfh.y - mh.y) + (tfl.y - ml.y);
                     const float dz = (tfh.z - mh.z) + (tfl.z - ml.z);
                     const float lim = k.far_dist + tfh.w + mh.w;
-                    const bool far = k.rule0 && (fmaf(dx, dx, fmaf(dy, dy, dz * dz)) >= lim * lim);
+                    const bool far = rev && k.rule0 && (fmaf(dx, dx, fmaf(dy, dy, dz * dz)) >= lim * lim);
                     const float4* cb = sb + c * kFFChunk * kFFNodeF4;
                     const int64_t j0 = Bc * kFFChunk;
-                    ff R1{0.0f, 0.0f}, R2{0.0f, 0.0f};
+                    // each half-warp walks the 16 pairs of sources, lane l taking pair
+                    // (l + step) mod 16; a pair's reverse sums go to lane - 1 of the half
+                    ff2 R1{}, R2{};
                     if (far) {
 #pragma unroll 1
-                        for (int step = 0; step < kFFChunk; ++step) {
-                            const int p = (lane + step) & (kFFChunk - 1);
-                            ffs_pair<false>(T, ai, bi, cb[p], cb[32 + p], cb[64 + p], cb[96 + p], k, tab, rev, S1, S2,
-                                            R1, R2, geo, gi, j0 + p, N);
-                            R1.h = __shfl_sync(0xffffffffu, R1.h, lane + 1);  // source p goes to lane - 1
-                            R1.l = __shfl_sync(0xffffffffu, R1.l, lane + 1);
-                            R2.h = __shfl_sync(0xffffffffu, R2.h, lane + 1);
-                            R2.l = __shfl_sync(0xffffffffu, R2.l, lane + 1);
+                        for (int step = 0; step < kFFPairs; ++step) {
+                            const int p = (lane + step) & (kFFPairs - 1);
+                            ff_pairs2<false>(T, ff_load(cb, p), k, tab, true, S1, S2, R1, R2, geo, gi, j0 + p, N);
+                            R1 = ff_rotate(R1, lane);
+                            R2 = ff_rotate(R2, lane);
                         }
                     } else {
 #pragma unroll 1
-                        for (int step = 0; step < kFFChunk; ++step) {
-                            const int p = (lane + step) & (kFFChunk - 1);
-                            ffs_pair<true>(T, ai, bi, cb[p], cb[32 + p], cb[64 + p], cb[96 + p], k, tab, rev, S1, S2,
-                                           R1, R2, geo, gi, j0 + p, N);
-                            R1.h = __shfl_sync(0xffffffffu, R1.h, lane + 1);
-                            R1.l = __shfl_sync(0xffffffffu, R1.l, lane + 1);
-                            R2.h = __shfl_sync(0xffffffffu, R2.h, lane + 1);
-                            R2.l = __shfl_sync(0xffffffffu, R2.l, lane + 1);
+                        for (int step = 0; step < kFFPairs; ++step) {
+                            const int p = (lane + step) & (kFFPairs - 1);
+                            ff_pairs2<true>(T, ff_load(cb, p), k, tab, rev, S1, S2, R1, R2, geo, gi, j0 + p, N);
+                            R1 = ff_rotate(R1, lane);
+                            R2 = ff_rotate(R2, lane);
                         }
                     }
-                    if (rev) {  // lane l holds source j0 + l's reverse sums over the warp's targets
-                        atomicAdd(yrev + j0 + lane, (double)R1.h + (double)R1.l);
-                        atomicAdd(yrev + n_pad + j0 + lane, (double)R2.h + (double)R2.l);
+                    if (rev) {
+                        // source j0 + lane's reverse sums over the warp's targets
+                        atomicAdd(yrev + j0 + lane, ff_halves_sum(R1, lane));
+                        atomicAdd(yrev + n_pad + j0 + lane, ff_halves_sum(R2, lane));
                     }
                 }
-                D1 += (double)S1.h + (double)S1.l;
-                D2 += (double)S2.h + (double)S2.l;
+                D1 += ff_value(S1);
+                D2 += ff_value(S2);
             }
             __syncthreads();
             if (tid == 0 && u + kFFStages < s1) {
@@ -744,32 +835,31 @@ __global__ void ff_pack_kernel(const double* __restrict__ geo, int64_t N, int64_
         yrev[n_pad + j] = 0.0;
         if (j == 0) *reinterpret_cast<unsigned long long*>(yrev + 2 * n_pad) = 0ull;
     }
+    float* dst = reinterpret_cast<float*>(src);
     if (j >= N) {
-        src[ff_off(j, 0)] = make_float4(kFFPad, kFFPad, kFFPad, 0.0f);
-        src[ff_off(j, 1)] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        src[ff_off(j, 2)] = make_float4(0.0f, 0.0f, 1.0f, 0.0f);
-        src[ff_off(j, 3)] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        for (int c = 0; c < 4; ++c) {
+            dst[ff_off(j, 0, c)] = c < 3 ? kFFPad : 0.0f;
+            dst[ff_off(j, 1, c)] = 0.0f;
+            dst[ff_off(j, 2, c)] = c == 2 ? 1.0f : 0.0f;
+            dst[ff_off(j, 3, c)] = 0.0f;
+        }
         return;
     }
     const double* p = in.base + (in.kidx ? (int64_t)(*in.kidx + in.koff) * in.stride : 0);
     const double cen[3] = {c0, c1, c2};
-    float xh[3], xl[3], nh[3], nl[3];
-    for (int a = 0; a < 3; ++a) {
-        const double x = geo[a * N + j] - cen[a];
-        const double xg = rint(x * grid_scale) / grid_scale;  // on the grid: exact as a float
-        xh[a] = (float)xg;
-        xl[a] = (float)(x - xg);
-        const double n = geo[(3 + a) * N + j];
-        nh[a] = (float)n;
-        nl[a] = (float)(n - (double)nh[a]);
-    }
     const double w = geo[6 * N + j];
-    const double av = w * p[j], bv = w * p[N + j];
-    const float ah = (float)av, bh = (float)bv;
-    src[ff_off(j, 0)] = make_float4(xh[0], xh[1], xh[2], ah);
-    src[ff_off(j, 1)] = make_float4(xl[0], xl[1], xl[2], (float)(av - (double)ah));
-    src[ff_off(j, 2)] = make_float4(nh[0], nh[1], nh[2], bh);
-    src[ff_off(j, 3)] = make_float4(nl[0], nl[1], nl[2], (float)(bv - (double)bh));
+    for (int a = 0; a < 4; ++a) {
+        // position and normal components, then a and b
+        const double x = a < 3 ? geo[a * N + j] - cen[a] : w * p[j];
+        const double n = a < 3 ? geo[(3 + a) * N + j] : w * p[N + j];
+        // positions: on the grid, exact as a float
+        const float xh = a < 3 ? (float)(rint(x * grid_scale) / grid_scale) : (float)x;
+        const float nh = (float)n;
+        dst[ff_off(j, 0, a)] = xh;
+        dst[ff_off(j, 1, a)] = (float)(x - (double)xh);
+        dst[ff_off(j, 2, a)] = nh;
+        dst[ff_off(j, 3, a)] = (float)(n - (double)nh);
+    }
 }
 
 // ------------------------------------------------------------------ host side
@@ -818,14 +908,17 @@ static ibim_status ff_prepare(ibim_ctx* c)
 
 ibim_status ff_prepare_context(ibim_ctx* c) { return ff_prepare(c); }
 
+constexpr int kFFSThreads = 128, kFFSSTile = 32, kFFSBigShare = 1;
+static const auto ffs_kernel = pair_ffs_kernel<kFFSThreads, kFFSSTile>;
+
 int ffs_grid_cap(ibim_ctx* c)
 {
     int occ = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, pair_ffs_kernel, kFFSThreads, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ffs_kernel, kFFSThreads, 0);
     return (occ < 1 ? 1 : occ) * c->num_sms;
 }
 
-size_t ffs_part_doubles(ibim_ctx* c) { return sym_part_doubles(c->N, kFFSThreads, kFFSTile, ffs_grid_cap(c)); }
+size_t ffs_part_doubles(ibim_ctx* c) { return sym_part_doubles(c->N, kFFSThreads, kFFSSTile, ffs_grid_cap(c), kFFSBigShare); }
 
 ibim_status ff_pack(ibim_ctx* c, VecRef in, const int* d_skip)
 {
@@ -843,8 +936,8 @@ ibim_status ff_pack(ibim_ctx* c, VecRef in, const int* d_skip)
 ibim_status ff_pairs(ibim_ctx* c, const PairConsts& k, const PairSchedule& s, const int* d_skip)
 {
     if (c->ff_symmetric) {
-        const SymSchedule ss = make_sym_schedule(c->N, kFFSThreads, kFFSTile, ffs_grid_cap(c));
-        pair_ffs_kernel<<<ss.grid, kFFSThreads, 0, c->stream>>>(
+        const SymSchedule ss = make_sym_schedule(c->N, kFFSThreads, kFFSSTile, ffs_grid_cap(c), kFFSBigShare);
+        ffs_kernel<<<ss.grid, kFFSThreads, 0, c->stream>>>(
             (const float4*)c->d_src, c->d_frames, c->d_fftab, c->d_geo64, c->N, padded_nodes(c->N), ss, ff_consts(k),
             c->d_part, c->d_yrev, c->d_err, d_skip);
     } else {
@@ -860,7 +953,7 @@ ibim_status ff_pairs(ibim_ctx* c, const PairConsts& k, const PairSchedule& s, co
 ibim_status ff_fixup(ibim_ctx* c, const PairConsts& k, const PairSchedule& s, VecRef in, OutRef out,
                      const int* d_skip)
 {
-    if (c->ff_symmetric) return sym_fixup_tiles(c, kFFSThreads, kFFSTile, ffs_grid_cap(c), k, in, out, d_skip);
+    if (c->ff_symmetric) return sym_fixup_tiles(c, kFFSThreads, kFFSSTile, ffs_grid_cap(c), k, in, out, d_skip, kFFSBigShare);
     return fixup_launch(c, k, s, kFFTTile, in, out, d_skip);
 }
 

@@ -413,11 +413,11 @@ int sym_occupancy(int v)
     return occ < 1 ? 1 : occ;
 }
 
-// Large segments hold kSymBigShare (of kSymShareDen) of an even per-CTA share;
+// Large segments hold big_share (of kSymShareDen) of an even per-CTA share;
 // the rest is cut into about kSymSmallPerCta small segments per CTA.
-constexpr int64_t kSymBigShare = 9, kSymShareDen = 10, kSymSmallPerCta = 16;
+constexpr int64_t kSymShareDen = 10, kSymSmallPerCta = 16;
 
-SymSchedule make_sym_schedule(int64_t N, int ttile, int stile, int grid_cap)
+SymSchedule make_sym_schedule(int64_t N, int ttile, int stile, int grid_cap, int big_share)
 {
     SymSchedule s;
     s.n_t = (N + ttile - 1) / ttile;
@@ -429,7 +429,7 @@ SymSchedule make_sym_schedule(int64_t N, int ttile, int stile, int grid_cap)
     int64_t g = std::min<int64_t>(grid_cap, s.total);
     if (g < 1) g = 1;
     s.nbig = g;
-    s.Lb = std::max<int64_t>(1, (kSymBigShare * s.total) / (kSymShareDen * g));  // g Lb <= total as g <= total
+    s.Lb = std::max<int64_t>(1, ((int64_t)big_share * s.total) / (kSymShareDen * g));  // g Lb <= total as g <= total
     const int64_t rest = s.total - g * s.Lb;
     s.Ls = std::max<int64_t>(1, (rest + kSymSmallPerCta * g - 1) / (kSymSmallPerCta * g));
     s.nseg = g + (rest + s.Ls - 1) / s.Ls;
@@ -438,9 +438,9 @@ SymSchedule make_sym_schedule(int64_t N, int ttile, int stile, int grid_cap)
 }
 
 // Partial slots (segment + row sequence index < nseg + n_t).
-size_t sym_part_doubles(int64_t N, int ttile, int stile, int grid_cap)
+size_t sym_part_doubles(int64_t N, int ttile, int stile, int grid_cap, int big_share)
 {
-    const SymSchedule s = make_sym_schedule(N, ttile, stile, grid_cap);
+    const SymSchedule s = make_sym_schedule(N, ttile, stile, grid_cap, big_share);
     return (size_t)(s.nseg + s.n_t) * 2 * ttile;
 }
 
@@ -485,9 +485,9 @@ ibim_status sym_fixup(ibim_ctx* c, int sv, int grid_cap, const PairConsts& k, Ve
 // y = Lambda p + (1/(4 pi)) (forward partials + reverse sums) for a symmetric
 // launch of `ttile`-target tiles on a grid of at most grid_cap CTAs.
 ibim_status sym_fixup_tiles(ibim_ctx* c, int ttile, int stile, int grid_cap, const PairConsts& k, VecRef in, OutRef out,
-                            const int* d_skip)
+                            const int* d_skip, int big_share)
 {
-    const SymSchedule s = make_sym_schedule(c->N, ttile, stile, grid_cap);
+    const SymSchedule s = make_sym_schedule(c->N, ttile, stile, grid_cap, big_share);
     static_assert(kFixParts == 4 && 128 % kFixTargets == 0, "fixup shares");
     fixup_sym_kernel<<<(unsigned)((c->N + kFixTargets - 1) / kFixTargets), kFixParts * kFixTargets, 0, c->stream>>>(
         c->d_part, s, ttile, c->N, padded_nodes(c->N), k.lambda1, k.lambda2, in, out, c->d_yrev, d_skip);

@@ -76,7 +76,7 @@ __host__ __device__ __forceinline__ void sym_row_start(const SymSchedule& s, int
     }
 }
 
-SymSchedule make_sym_schedule(int64_t N, int ttile, int stile, int grid_cap);
+SymSchedule make_sym_schedule(int64_t N, int ttile, int stile, int grid_cap, int big_share = kSymBigShare);
 
 // Float4 offset of component `comp` (0..3 = A..D) of payload pair `pr`.
 __host__ __device__ __forceinline__ int64_t sym_pair_offset(int64_t pr, int comp)
