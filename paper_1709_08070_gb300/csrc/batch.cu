@@ -947,8 +947,7 @@ ibim_status batch_solve(int nmol, ibim_ctx* const* ctxs, const ibim_phys* phys, 
         infos[i].relres = gnorm[i] > 0.0 ? beta[i] / gnorm[i] : 0.0;
         IBIM_CUDA(cudaMemcpyAsync(d_p[i], c->gm->x, sizeof(double) * 2 * c->N, cudaMemcpyDeviceToDevice, R.bs));
         double gpol = 0.0, area = 0.0;
-        IBIM_TRY(energy_launch(c, phys[i], c->gm->x, nullptr, &gpol));
-        IBIM_TRY(area_launch(c, &area));
+        IBIM_TRY(energy_launch(c, phys[i], c->gm->x, nullptr, &gpol, &area));
         infos[i].gpol = gpol;
         infos[i].gpol_kcal = gpol * kKcalPerE2A;
         infos[i].area = area;

@@ -669,8 +669,7 @@ ibim_status ibim_solve_extrapolated(ibim_ctx* c, const ibim_phys* phys, const ib
     count_launch(c);
     IBIM_CUDA(cudaGetLastError());
     double gpol = 0.0, area = 0.0;
-    IBIM_TRY(energy_launch(c, *phys, d_p, nullptr, &gpol));
-    IBIM_TRY(area_launch(c, &area));
+    IBIM_TRY(energy_launch(c, *phys, d_p, nullptr, &gpol, &area));
     info->iters = i1.iters + i2.iters;
     info->cycles = i1.cycles + i2.cycles;
     info->converged = (i1.converged && i2.converged) ? 1 : 0;

@@ -8,6 +8,13 @@ constexpr int kMaxRestart = 128;
 constexpr int kVecThreads = 256;
 constexpr int kDotGroup = 8;  // dot products a warp forms together
 
+// What the host reads of a finished cycle (pinned host memory, written by the
+// device; no answer before `done`).
+struct GmOutcome {
+    int done, k, conv;
+};
+constexpr int kStepsPerGraph = 2;  // Arnoldi steps in the captured graph and between two waits of the host
+
 struct GmState {
     int k;       // current Arnoldi step within the cycle
     int done;    // stop expanding (converged, cycle full or breakdown)
@@ -23,6 +30,7 @@ struct GmState {
     double cs[kMaxRestart], sn[kMaxRestart];
     double e[kMaxRestart + 1];
     double y[kMaxRestart];
+    GmOutcome* out;  // nullptr: not wanted (batched solves read the state itself)
     double H[(kMaxRestart + 1) * kMaxRestart];  // row-major, row stride m
     int dot_ticket[(kMaxRestart + 1 + kDotGroup - 1) / kDotGroup];  // blocks done with a group of dot products
 };
@@ -53,8 +61,10 @@ struct GmresWork {
     GmSys sys;                 // the orthogonalisation kernels' view
     GmState* st = nullptr;     // device state
     GmState* h_st = nullptr;   // pinned host mirror (small fields only are read)
+    GmOutcome* h_out = nullptr;  // pinned, behind h_st
     cudaStream_t gs = nullptr; // capture-capable stream owned by the solver
     cudaEvent_t ev = nullptr;
+    cudaEvent_t poll[2] = {nullptr, nullptr};  // behind the two latest pairs of steps
     cudaGraphExec_t exec = nullptr;
     int graph_prec = 0;
     PairConsts graph_k;

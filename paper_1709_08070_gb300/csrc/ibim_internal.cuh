@@ -246,7 +246,7 @@ ibim_status f64_apply(ibim_ctx* c, const PairConsts& k, VecRef in, OutRef out, c
 // RHS / energy / area (rhs_energy.cu)
 ibim_status rhs_launch(ibim_ctx* c, double eps_in, double* d_g);
 ibim_status energy_launch(ibim_ctx* c, const ibim_phys& p, const double* d_p, double* d_psi,
-                          double* gpol_host);
+                          double* gpol_host, double* area_host = nullptr);  // area_host: with the area, one wait
 ibim_status area_launch(ibim_ctx* c, double* area_host);
 
 // Geometry (geometry.cu)

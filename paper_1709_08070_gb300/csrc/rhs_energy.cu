@@ -187,7 +187,23 @@ __global__ void __launch_bounds__(1024)
     if (threadIdx.x == 0) out[0] = 0.5 * red[0];
 }
 
-ibim_status energy_launch(ibim_ctx* c, const ibim_phys& p, const double* d_p, double* d_psi, double* gpol_host)
+// Surface area: sum_j w_j (Sec. 3.4), deterministic two-level sum.
+__global__ void area_kernel(const double* __restrict__ w, int64_t N, double* __restrict__ out)
+{
+    __shared__ double red[1024];
+    double s = 0.0;
+    for (int64_t j = threadIdx.x; j < N; j += blockDim.x) s += w[j];
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
+        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) out[0] = red[0];
+}
+
+ibim_status energy_launch(ibim_ctx* c, const ibim_phys& p, const double* d_p, double* d_psi, double* gpol_host,
+                          double* area_host)
 {
     const int64_t N = c->N, Nc = c->Nc;
     const int atoms = Nc < 4 ? 1 : 4;
@@ -212,25 +228,17 @@ ibim_status energy_launch(ibim_ctx* c, const ibim_phys& p, const double* d_p, do
                                                                     part);
     energy_final_kernel<<<1, 1024, 0, c->stream>>>(part, nsplit, Nc, c->d_q, d_psi, c->d_red);
     count_launch(c, 2);
-    IBIM_CUDA(cudaGetLastError());
-    IBIM_CUDA(cudaMemcpyAsync(gpol_host, c->d_red, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    IBIM_CUDA(cudaStreamSynchronize(c->stream));
-    return IBIM_OK;
-}
-
-// Surface area: sum_j w_j (Sec. 3.4), deterministic two-level sum.
-__global__ void area_kernel(const double* __restrict__ w, int64_t N, double* __restrict__ out)
-{
-    __shared__ double red[1024];
-    double s = 0.0;
-    for (int64_t j = threadIdx.x; j < N; j += blockDim.x) s += w[j];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
+    if (area_host != nullptr) {
+        area_kernel<<<1, 1024, 0, c->stream>>>(c->d_geo64 + 6 * N, N, c->d_red + 1);
+        count_launch(c);
     }
-    if (threadIdx.x == 0) out[0] = red[0];
+    IBIM_CUDA(cudaGetLastError());
+    double out[2];
+    IBIM_CUDA(cudaMemcpyAsync(out, c->d_red, sizeof(double) * (area_host ? 2 : 1), cudaMemcpyDeviceToHost, c->stream));
+    IBIM_CUDA(cudaStreamSynchronize(c->stream));
+    *gpol_host = out[0];
+    if (area_host != nullptr) *area_host = out[1];
+    return IBIM_OK;
 }
 
 ibim_status area_launch(ibim_ctx* c, double* area_host)
