@@ -58,6 +58,8 @@ __global__ void __launch_bounds__(THREADS, MINB)
     constexpr int TTILE = THREADS * TPT;
     constexpr int NW = THREADS / 32;
     static_assert(TTILE <= kF32MaxTTile && STAGES <= kF32Stages, "tile, stages");
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
     if (skip != nullptr && *skip) return;
     __shared__ __align__(128) SourceStage stg[STAGES];
     __shared__ __align__(16) float4 tfrm[NW][2 * TPT];
@@ -216,6 +218,8 @@ __global__ void pack_f32_kernel(const float4* __restrict__ pos, const float4* __
                                 const double* __restrict__ w, VecRef in, int64_t N, int64_t n_pairs,
                                 float4* __restrict__ src, const int* __restrict__ skip)
 {
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
     if (skip != nullptr && *skip) return;
     const int64_t pr = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (pr >= n_pairs) return;
@@ -251,6 +255,7 @@ __global__ void __launch_bounds__(kFixShares * kFixNodes)
     fixup_kernel(const double* __restrict__ part, PairSchedule s, int ttile, int64_t N, double lambda1,
                  double lambda2, VecRef in, OutRef out, const int* __restrict__ skip)
 {
+    ptx::grid_dep_wait();
     if (skip != nullptr && *skip) return;
     __shared__ double sh[2][kFixShares][kFixNodes];
     const int tl = threadIdx.x % kFixNodes, pr = threadIdx.x / kFixNodes;
@@ -298,13 +303,14 @@ struct PairArgs {
     unsigned* err;
     const int* skip;
     Geo64 g64;
+    bool chained;
 };
 
 template <int TPT, int MINB, int THREADS, int STAGES = kF32Stages, bool FLATNEAR = false>
 static void launch_variant(const PairArgs& a, cudaStream_t stream)
 {
-    pair_f32_kernel<TPT, MINB, THREADS, STAGES, FLATNEAR><<<a.s.grid, THREADS, 0, stream>>>(
-        a.tpos, a.tnrm, a.src, a.frames, a.N, a.s, a.k, a.part, a.err, a.skip, a.g64);
+    launch_chained(pair_f32_kernel<TPT, MINB, THREADS, STAGES, FLATNEAR>, dim3(a.s.grid), THREADS, 0, stream, a.chained,
+                   a.tpos, a.tnrm, a.src, a.frames, a.N, a.s, a.k, a.part, a.err, a.skip, a.g64);
 }
 
 struct F32Variant {
@@ -435,7 +441,7 @@ ibim_status f32_pairs(ibim_ctx* c, const PairConsts& k, const PairSchedule& s, c
     IBIM_TRY(ensure(c, (void**)&c->d_part, &c->part_bytes, f32_part_doubles(c) * sizeof(double)));
     if (is_sym(c->f32_variant)) return sym_pairs(c, c->f32_variant - kNumVariants, f32_grid_cap(c), k, d_skip);
     const PairArgs a{c->d_pos32, c->d_nrm32, (const float4*)c->d_src, c->d_frames, c->N, s, f32_consts(k),
-                     c->d_part, c->d_err, d_skip, Geo64{c->d_geo64, c->d_geo64 + 3 * c->N, 1, c->N}};
+                     c->d_part, c->d_err, d_skip, Geo64{c->d_geo64, c->d_geo64 + 3 * c->N, 1, c->N}, d_skip == nullptr};
     one_directional(c).launch(a, c->stream);
     count_launch(c);
     IBIM_CUDA(cudaGetLastError());
@@ -445,8 +451,9 @@ ibim_status f32_pairs(ibim_ctx* c, const PairConsts& k, const PairSchedule& s, c
 ibim_status fixup_launch(ibim_ctx* c, const PairConsts& k, const PairSchedule& s, int ttile, VecRef in,
                          OutRef out, const int* d_skip)
 {
-    fixup_kernel<<<(unsigned)((c->N + kFixNodes - 1) / kFixNodes), kFixShares * kFixNodes, 0, c->stream>>>(
-        c->d_part, s, ttile, c->N, k.lambda1, k.lambda2, in, out, d_skip);
+    IBIM_CUDA(launch_chained(fixup_kernel, dim3((unsigned)((c->N + kFixNodes - 1) / kFixNodes)),
+                             kFixShares * kFixNodes, 0, c->stream, d_skip == nullptr, c->d_part, s, ttile, c->N, k.lambda1,
+                             k.lambda2, in, out, d_skip));
     count_launch(c);
     IBIM_CUDA(cudaGetLastError());
     return IBIM_OK;
@@ -487,7 +494,7 @@ cudaError_t launch_pair_f32_raw(const float4* tpos, const float4* tnrm, const fl
                                 int64_t N, const PairSchedule& s, const PairConsts& k, double* part, unsigned* err,
                                 cudaStream_t stream, const double* xs_aos, const double* nrm_aos)
 {
-    const PairArgs a{tpos, tnrm, src, frames, N, s, f32_consts(k), part, err, nullptr, Geo64{xs_aos, nrm_aos, 3, 1}};
+    const PairArgs a{tpos, tnrm, src, frames, N, s, f32_consts(k), part, err, nullptr, Geo64{xs_aos, nrm_aos, 3, 1}, false};
     launch_variant<kF32Tpt, 1, kF32Threads>(a, stream);
     return cudaGetLastError();
 }

@@ -75,6 +75,8 @@ __global__ void __launch_bounds__(THREADS, MINB)
     constexpr int NW = THREADS / 32;
     constexpr int STILE = CH * kChunk;
     static_assert(TTILE <= kF32MaxTTile && TTILE % STILE == 0 && kPadNodes % STILE == 0, "tiles");
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
     if (skip != nullptr && *skip) return;
     __shared__ __align__(128) SourceStageT<CH> stg[kF32Stages];
     __shared__ __align__(16) float4 tfrm[NW][2 * TPT];
@@ -267,6 +269,8 @@ __global__ void pack_sym_kernel(const float4* __restrict__ pos, const float4* __
                                 const double* __restrict__ w, VecRef in, int64_t N, int64_t n_pairs,
                                 float4* __restrict__ src, double* __restrict__ yrev, const int* __restrict__ skip)
 {
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
     if (skip != nullptr && *skip) return;
     const int64_t pr = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (pr >= n_pairs) return;
@@ -307,6 +311,7 @@ __global__ void __launch_bounds__(kFixParts * kFixTargets)
                      double lambda1, double lambda2, VecRef in, OutRef out, const double* __restrict__ yrev,
                      const int* __restrict__ skip)
 {
+    ptx::grid_dep_wait();
     if (skip != nullptr && *skip) return;
     __shared__ double sh1[kFixParts][kFixTargets], sh2[kFixParts][kFixTargets];
     const int tl = threadIdx.x % kFixTargets, pr = threadIdx.x / kFixTargets;
@@ -368,8 +373,8 @@ struct SymArgs {
 template <int TPT, int MINB, int THREADS, bool ROT, int UNR, int CH>
 static void launch_sym(const SymArgs& a, cudaStream_t st)
 {
-    pair_sym_kernel<TPT, MINB, THREADS, ROT, UNR, CH><<<a.s.grid, THREADS, 0, st>>>(
-        a.tpos, a.tnrm, a.src, a.frames, a.N, a.n_pad, a.s, a.k, a.part, a.yrev, a.err, a.skip, a.g64);
+    launch_chained(pair_sym_kernel<TPT, MINB, THREADS, ROT, UNR, CH>, dim3(a.s.grid), THREADS, 0, st, a.skip == nullptr,
+                   a.tpos, a.tnrm, a.src, a.frames, a.N, a.n_pad, a.s, a.k, a.part, a.yrev, a.err, a.skip, a.g64);
 }
 
 // scheme: 1 = warp reduction of the reverse sums, 2 = rotation (see the file comment)
@@ -489,8 +494,9 @@ ibim_status sym_fixup_tiles(ibim_ctx* c, int ttile, int stile, int grid_cap, con
 {
     const SymSchedule s = make_sym_schedule(c->N, ttile, stile, grid_cap, big_share);
     static_assert(kFixParts == 4 && 128 % kFixTargets == 0, "fixup shares");
-    fixup_sym_kernel<<<(unsigned)((c->N + kFixTargets - 1) / kFixTargets), kFixParts * kFixTargets, 0, c->stream>>>(
-        c->d_part, s, ttile, c->N, padded_nodes(c->N), k.lambda1, k.lambda2, in, out, c->d_yrev, d_skip);
+    IBIM_CUDA(launch_chained(fixup_sym_kernel, dim3((unsigned)((c->N + kFixTargets - 1) / kFixTargets)),
+                             kFixParts * kFixTargets, 0, c->stream, d_skip == nullptr, c->d_part, s, ttile, c->N,
+                             padded_nodes(c->N), k.lambda1, k.lambda2, in, out, c->d_yrev, d_skip));
     count_launch(c);
     IBIM_CUDA(cudaGetLastError());
     return IBIM_OK;
