@@ -523,13 +523,16 @@ struct TcM2l {
 };
 
 // Fields at the target proxies of each target tile from the proxy tiles of
-// its interpolated far clusters.  Work items are runs of at least 8 entries of
+// its interpolated far clusters.  Work items are runs of at least 4 entries of
 // one tile's list: CTA b takes item b and then items from the counter; the
 // source proxy tiles stream through the stage ring as in the list kernel
 // (ring position continued across items), and each item adds its fields to
 // the tile's (zeroed before the launch) with FP64 atomics.
+// Bound by the FP32 pipe; four CTAs per SM (71 registers) hide more of the
+// stage waits and item ends than three (78): 9.10 -> 9.02 ms per application of
+// 321k nodes at order 6.
 template <int NC>
-__global__ void __launch_bounds__(Cheb<NC>::kM2lThreads)
+__global__ void __launch_bounds__(Cheb<NC>::kM2lThreads, 4)
     tc_m2l_kernel(const float4* __restrict__ src, const float4* __restrict__ frames, TcM2l m, F32Consts k,
                   double* __restrict__ fields, unsigned long long* __restrict__ ctr, unsigned* __restrict__ err,
                   const int* __restrict__ skip)
@@ -956,16 +959,22 @@ ibim_status tc_setup(ibim_ctx* c, double theta, double tau_max, int order, int i
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, tc_pair_kernel<kTcTpt, kTcMinCtas, kTcThreads>, kTcThreads, 0);
     const int64_t cap = (int64_t)std::max(1, occ) * c->num_sms;
     const int64_t g = std::max<int64_t>(1, std::min<int64_t>(cap, T->total));
-    T->Lb = std::max<int64_t>(1, (9 * T->total) / (10 * g));  // g Lb <= total as g <= total
+    // A fifth of an even share per CTA in its large segment, the rest in small
+    // ones: the two CTAs of an SM do not advance alike, and far steps are shorter
+    // than near ones.  321k nodes, per application, with nine tenths / half / a
+    // fifth / a twentieth: 9.50 / 9.43 / 9.40 / 9.42 ms at order 6, 3.22 / 3.01 /
+    // 2.92 / 2.93 at order 4, theta 0.9.
+    T->Lb = std::max<int64_t>(1, T->total / (5 * g));  // g Lb <= total as g <= total
     const int64_t rest = T->total - g * T->Lb;
     T->Ls = std::max<int64_t>(1, (rest + 16 * g - 1) / (16 * g));
     T->nseg = g + (rest + T->Ls - 1) / T->Ls;
     T->grid = (int)g;
-    // m2l work items: runs of at least 8 entries of one tile's list, about
-    // four per resident CTA
+    // m2l work items: runs of at least 4 entries of one tile's list, about 32 per
+    // resident CTA, so that the CTAs end together (321k nodes, order 6, per
+    // application: four per CTA 9.40 ms, eight 9.31, sixteen 9.14, 32 9.10, 64 9.10)
     const int occm = order == 4 ? m2l_occupancy<4>() : order == 5 ? m2l_occupancy<5>() : m2l_occupancy<6>();
     const int64_t slots = (int64_t)occm * c->num_sms;
-    const int64_t run = std::max<int64_t>(8, (T->interp_steps + 4 * slots - 1) / (4 * slots));
+    const int64_t run = std::max<int64_t>(4, (T->interp_steps + 32 * slots - 1) / (32 * slots));
     std::vector<TcItem> items;
     for (int64_t t = 0; t < n_t; ++t)
         for (int64_t e = irow[t]; e < irow[t + 1]; e += run)
