@@ -44,10 +44,12 @@ WORKLOAD = {"workload": "kirkwood_sphere", "R": 20.0, "h": 0.5, "band_k": 2, "ta
 # counted; the per-chunk frame offsets and compensation add about 0.5.
 F32_OPS_PER_INTERACTION = 36
 # The symmetric variants evaluate each unordered source pair once for both
-# directions: the shared part (r, |r|^2, s_x, s_y, c, rho, E, g, the series
-# products, rho^-3, theta terms, hi, qf) is 28 lane-operations and each
-# direction's two sums 10 more, 48 for two interactions.
-F32_OPS_PER_INTERACTION_SYM = 24
+# directions, in the rotation scheme: the shared part (r 3, |r|^2 3, s_x, s_y, c
+# 3 each, the two exponent arguments 2, E x, E - 1, g 3, 3 - B 2, rho^-2 and
+# rho^-3 2, the two theta terms times rho^-3 4, the combined a-term of the second
+# sums 5, the 1/rho factor 1, products with s_x and s_y 4) is 38 lane-operations
+# and each direction's two sums 4 more, 46 for two interactions.
+F32_OPS_PER_INTERACTION_SYM = 23
 # The float-float operator (IBIM_FF, pair_ff_kernel), counted from ff_pairs2's
 # far form (lane-operations per interaction): r 6, |r|^2, s_x and s_y 31 each,
 # n.m 28, 1/rho 11, rho 7, kappa rho and the exponent argument 4 each, exp 25, E x
@@ -63,10 +65,10 @@ FFS_OPS_PER_INTERACTION = 204
 FP32_LANES_PER_SM = 128
 # dram__bytes_read.sum + dram__bytes_write.sum of one pair-kernel launch on this
 # workload, by variant (targets/thread, min CTAs/SM, threads/CTA, symmetric scheme), from
-# the ncu full-set captures summarised in profiles/pair_f32_kernel_kirkwood80k.md and
+# the ncu captures summarised in profiles/pair_f32_kernel_kirkwood80k.md and
 # profiles/pair_sym_kernel_kirkwood80k.md; None where the kernel changed after
 # its last capture.
-NCU_TRAFFIC_BYTES = {(2, 1, 512, 0): None, (2, 1, 512, 1): 7.012352e6, (2, 1, 512, 2): 7.009792e6}
+NCU_TRAFFIC_BYTES = {(2, 1, 512, 0): None, (2, 1, 512, 1): None, (2, 1, 512, 2): 7.003904e6}
 METRIC = "IBIM matvec interactions/s"
 L2_NOTE = ("GPU arm: a 256 MB buffer is written between timed steps (L2 is 129 MB); "
            "oracle arm: host cores, no GPU cache involved")

@@ -391,7 +391,8 @@ ibim_status ibim_f32_variant_info(int v, int* targets_per_thread, int* min_ctas_
                                   int* symmetric);
 
 /*
- * Autotuner: times every variant on this context's geometry with CUDA events,
+ * Autotuner: times the variants on this context's geometry with CUDA events
+ * (one application of each, more of those within a third of the best so far),
  * keeps the fastest for this context and caches it for contexts built later
  * in the process of the same geometry kind (analytic sphere, level-set
  * surface or caller-given nodes) with N in the same power-of-two bucket.  Returns the chosen
@@ -485,8 +486,8 @@ ibim_status ibim_solve_batch(int nmol, ibim_ctx* const* ctxs, const ibim_phys* p
 /*
  * Batched pair-kernel variants (tuning, not part of the paper's method):
  * one-directional kernels with one target per thread in CTAs of 512, 256 or
- * 128 threads, and a symmetric kernel (each unordered node pair of a molecule
- * evaluated once for both directions, reverse sums carried by rotating
+ * 128 threads, and symmetric kernels with one or two (each unordered node pair of
+ * a molecule evaluated once for both directions, reverse sums carried by rotating
  * accumulators as in the single-molecule symmetric kernel).  By default the
  * first batched solve of a size class times every variant on its first round
  * and keeps the fastest; ibim_set_batch_variant(v) forces variant v for later
