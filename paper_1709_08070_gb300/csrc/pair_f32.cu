@@ -48,6 +48,8 @@
 
 namespace ibim {
 
+constexpr int kSmallTTile = 64;  // targets of a small launch's CTA
+
 template <int TPT, int MINB, int THREADS, int STAGES = kF32Stages, bool FLATNEAR = false>
 __global__ void __launch_bounds__(THREADS, MINB)
     pair_f32_kernel(const float4* __restrict__ tpos, const float4* __restrict__ tnrm,
@@ -165,6 +167,126 @@ __global__ void __launch_bounds__(THREADS, MINB)
             for (int q = 0; q < TPT; ++q) {
                 dst[q * THREADS + tid] = D1[q];
                 dst[TTILE + q * THREADS + tid] = D2[q];
+            }
+            if (sp == s.n_stiles - 1 && u + 1 < s1) {
+                ++t;
+                load_targets(t);
+            }
+        }
+    }
+}
+
+// The same sums for small launches, 64 targets per CTA: GROUPS threads per target
+// share the chunks of a source tile, and as a target's sum over a chunk does not
+// depend on the others, the first of them adds the chunk sums up in order, with
+// the compensation above: the result is pair_f32_kernel's bit for bit, and the
+// chain of one step is kChunksPerTile / GROUPS chunks instead of all.
+template <int GROUPS>
+__global__ void __launch_bounds__(kSmallTTile * GROUPS, 512 / (kSmallTTile * GROUPS))
+    pair_f32_small_kernel(const float4* __restrict__ tpos, const float4* __restrict__ tnrm,
+                          const float4* __restrict__ src, const float4* __restrict__ frames, int64_t N, PairSchedule s,
+                          F32Consts k, double* __restrict__ part, unsigned* __restrict__ err,
+                          const int* __restrict__ skip, Geo64 g64)
+{
+    constexpr int TTILE = kSmallTTile;
+    constexpr int NW = TTILE * GROUPS / 32;
+    constexpr int STAGES = 2;
+    static_assert(kChunksPerTile % GROUPS == 0, "groups");
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
+    if (skip != nullptr && *skip) return;
+    __shared__ __align__(128) SourceStage stg[STAGES];
+    __shared__ __align__(16) float4 tfrm[NW][2];
+    __shared__ float2 sums[2][kChunksPerTile][TTILE];  // chunk sums of the step, steps alternating
+    __shared__ __align__(8) StagePipe pipe;
+
+    const int tid = threadIdx.x;
+    const int warp = tid >> 5;
+    const int lane = tid & 31;
+    const int tgt = tid % TTILE, grp = tid / TTILE;
+    const int64_t s0 = (int64_t)blockIdx.x * s.per_cta;
+    const int64_t s1 = (s0 + s.per_cta < s.total) ? s0 + s.per_cta : s.total;
+    if (s0 >= s1) return;
+    const bool have_frames = frames != nullptr;
+
+    if (tid == 0) pipe_init(pipe, NW);
+    __syncthreads();
+    auto issue = [&](int64_t u) {
+        const int64_t st = ((u % s.n_stiles) * s.sperm) % s.n_stiles;
+        const int stage = (int)((u - s0) % STAGES);
+        pipe_issue(pipe, stg[stage], stage, src + st * (kF32STile / 2) * kPairF4,
+                   have_frames ? frames + st * 2 * kChunksPerTile : nullptr);
+    };
+    if (tid == 0)
+        for (int q = 0; q < STAGES && s0 + q < s1; ++q) issue(s0 + q);
+
+    const int64_t t_first = s0 / s.n_stiles;
+    int64_t t = t_first;
+    Targets<1> T;
+    int64_t gi = 0;
+    bool idle = false;
+    double D1 = 0.0, D2 = 0.0;  // (of the first group)
+    auto load_targets = [&](int64_t tile) {
+        gi = tile * TTILE + tgt;
+        const int64_t blk = (tile * TTILE + (tgt & ~31)) / kChunk;
+        idle = blk * kChunk >= N;
+        const float4 a = tpos[gi];
+        const float4 b = tnrm[gi];
+        T.x[0] = make_float3(a.x, a.y, a.z);
+        T.nx[0] = f2(b.x);
+        T.ny[0] = f2(b.y);
+        T.nz[0] = f2(b.z);
+        D1 = D2 = 0.0;
+        __syncwarp();
+        if (have_frames && lane < 2) tfrm[warp][lane] = frames[2 * blk + lane];
+        __syncwarp();
+    };
+    load_targets(t);
+
+    for (int64_t u = s0; u < s1; ++u) {
+        const int stage = (int)((u - s0) % STAGES);
+        const uint32_t parity = (uint32_t)(((u - s0) / STAGES) & 1);
+        bool ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(&pipe.full[stage], parity, kWaitLimitNs));
+        const int64_t sp = u % s.n_stiles;               // position in the row
+        const int64_t st = (sp * s.sperm) % s.n_stiles;  // source tile visited there
+        float2(*sum)[TTILE] = sums[(u - s0) & 1];
+#pragma unroll 1
+        for (int c = grp; c < kChunksPerTile; c += GROUPS) {
+            float S1[1] = {0.0f}, C1[1] = {0.0f}, S2[1] = {0.0f}, C2[1] = {0.0f};
+            if (ok && !idle)
+                tile_sums<1, false, 1, true>(T, &tfrm[warp][0], have_frames, stg[stage].buf + c * kPairsPerChunk * kPairF4,
+                                             stg[stage].frm + 2 * c, k, S1, C1, S2, C2, g64, gi, 0,
+                                             st * kF32STile + c * kChunk, N);
+            sum[c][tgt] = make_float2(S1[0], S2[0]);
+        }
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(&pipe.empty[stage]);
+        // thread 0 refills the stage of step u - 1 with step u - 1 + STAGES
+        if (tid == 0 && ok && u > s0 && u - 1 + STAGES < s1) {
+            const int64_t v = u - 1 - s0;
+            ok = ptx::mbar_wait_bounded(&pipe.empty[(int)(v % STAGES)], (uint32_t)((v / STAGES) & 1), kWaitLimitNs);
+            if (ok) {
+                ptx::fence_proxy_async_smem();
+                issue(u - 1 + STAGES);
+            }
+        }
+        if (!ok && lane == 0) atomicOr(err, kDevErrTimeout);
+        if (__syncthreads_or(!ok)) return;  // the chunk sums are complete; a wait that gave up ends the CTA
+        if (grp == 0) {
+            float S1 = 0.0f, C1 = 0.0f, S2 = 0.0f, C2 = 0.0f;
+#pragma unroll
+            for (int c = 0; c < kChunksPerTile; ++c) {
+                kahan_add(S1, C1, sum[c][tgt].x);
+                kahan_add(S2, C2, sum[c][tgt].y);
+            }
+            D1 += (double)S1 - (double)C1;
+            D2 += (double)S2 - (double)C2;
+        }
+        if (sp == s.n_stiles - 1 || u + 1 == s1) {
+            if (grp == 0) {
+                double* dst = part + ((int64_t)blockIdx.x * s.max_segs + (int)(t - t_first)) * 2 * TTILE;
+                dst[tgt] = D1;
+                dst[TTILE + tgt] = D2;
             }
             if (sp == s.n_stiles - 1 && u + 1 < s1) {
                 ++t;
@@ -313,6 +435,13 @@ static void launch_variant(const PairArgs& a, cudaStream_t stream)
                    a.tpos, a.tnrm, a.src, a.frames, a.N, a.s, a.k, a.part, a.err, a.skip, a.g64);
 }
 
+template <int GROUPS>
+static void launch_small(const PairArgs& a, cudaStream_t stream)
+{
+    launch_chained(pair_f32_small_kernel<GROUPS>, dim3(a.s.grid), kSmallTTile * GROUPS, 0, stream, a.chained, a.tpos,
+                   a.tnrm, a.src, a.frames, a.N, a.s, a.k, a.part, a.err, a.skip, a.g64);
+}
+
 struct F32Variant {
     int tpt, minb, threads;
     const void* fn;
@@ -327,15 +456,18 @@ static const F32Variant kVariants[] = {
 #undef IBIM_F32_VARIANT
 // Small launches of variant 0, the choice of a context that was not tuned:
 // below kSmallSteps steps of its own kernel (about 15,000 nodes) they run
-// 64-target tiles, four times as many steps, so that the chip is filled, and the
-// branch-free near formula, as most chunk pairs are near.  The source tiles,
-// within which a target's sums are compensated, stay the same, and with them
-// the result.  Jittered-sphere clouds, own kernel against this one:
-// 300 nodes 67.5 / 33.5 us, 3,001 70.5 / 34.7, 5,000 94.7 / 62.3, 8,000 165 / 127,
-// 12,000 279 / 233; at 17,000 the two meet.
+// pair_f32_small_kernel: 64-target tiles, four times as many steps, so that the
+// chip is filled, four threads to a target, and the branch-free near formula, as
+// most chunk pairs are near.  The result is the same bit for bit.  Clouds on a
+// sphere, one application after another, one / two / four / eight threads to a
+// target: 862 nodes 20.9 / 14.8 / 14.7 / 14.6 us (the three launches take 13),
+// 3,001 31.1 / 31.0 / 30.3 / 31.1, 6,500 98 / 86 / 78 / 87, 15,000 341 / 324 / 334 /
+// 375; variant 0's own kernel took 70.5 us at 3,001 nodes and 279 at 12,000 (235 so),
+// and at 17,000 the two meet.
 constexpr int64_t kSmallSteps = 3600;
-static const F32Variant kSmallVariant = {1, 8, 64, (const void*)pair_f32_kernel<1, 8, 64, 2, true>,
-                                         launch_variant<1, 8, 64, 2, true>};
+constexpr int kSmallGroups = 4;
+static const F32Variant kSmallVariant = {1, 512 / (kSmallTTile * kSmallGroups), kSmallTTile * kSmallGroups,
+                                         (const void*)pair_f32_small_kernel<kSmallGroups>, launch_small<kSmallGroups>};
 constexpr int kNumVariants = (int)(sizeof(kVariants) / sizeof(kVariants[0]));
 
 // Variants kNumVariants.. are the symmetric kernel's (pair_sym.cu).
@@ -381,6 +513,7 @@ int f32_max_bps(int v) { return is_sym(v) ? sym_occupancy(v - kNumVariants) : oc
 // Target tile of the context's FP32 kernel.
 int f32_ttile(const ibim_ctx* c)
 {
+    if (runs_small(c->f32_variant, c->N)) return kSmallTTile;
     if (!is_sym(c->f32_variant)) return one_directional(c).threads * one_directional(c).tpt;
     int tpt, minb, threads, sym;
     f32_variant_info(c->f32_variant, &tpt, &minb, &threads, &sym);

@@ -17,6 +17,13 @@ namespace {
 std::mutex g_tune_mu;
 std::map<std::pair<int, int>, std::pair<int, int>> g_tune_cache;  // (kind, bucket) -> (variant, CTAs per SM)
 
+// Up to this many nodes (18 source tiles) only one-directional variants are
+// timed, so that small molecules' applications and solves repeat bit for bit:
+// the 512-thread symmetric variants have too few steps to win there, and the
+// smaller ones, whose reverse sums are added in a varying order, gain little on
+// variant 0's small launches (862 nodes 17 against 15 us, 3,214 28 against 32).
+constexpr int64_t kRepeatableNodes = 4608;
+
 std::atomic<uint32_t> g_loaded{0};  // variants the process has timed (bit per variant)
 
 int size_bucket(int64_t N)
@@ -93,7 +100,8 @@ extern "C" ibim_status ibim_autotune(ibim_ctx* c, const ibim_phys* phys, int* va
     const PairConsts k = make_consts(*phys);
 
     std::vector<std::pair<int, int>> cand;  // (variant, CTAs per SM; 0 = occupancy limit)
-    for (int v = f32_variant_count() - 1; v >= 0; --v) cand.push_back({v, 0});  // the symmetric ones first
+    for (int v = f32_variant_count() - 1; v >= 0; --v)  // the symmetric ones first
+        if (N > kRepeatableNodes || !f32_variant_symmetric(v)) cand.push_back({v, 0});
     // Each repetition costs about N^2 / 6e11 s; keep the whole search short.
     const double est_ms = (double)N * (double)N / 6e8;
     const int reps = est_ms > 200.0 ? 1 : 2;
