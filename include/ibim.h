@@ -392,7 +392,9 @@ ibim_status ibim_f32_variant_info(int v, int* targets_per_thread, int* min_ctas_
 
 /*
  * Autotuner: times the variants on this context's geometry with CUDA events
- * (one application of each, more of those within a third of the best so far),
+ * (one application of each, more of those within a third of the best so far; up
+ * to 4,608 nodes the one-directional ones only, so that small molecules keep a
+ * kernel whose results repeat bit for bit),
  * keeps the fastest for this context and caches it for contexts built later
  * in the process of the same geometry kind (analytic sphere, level-set
  * surface or caller-given nodes) with N in the same power-of-two bucket.  Returns the chosen
