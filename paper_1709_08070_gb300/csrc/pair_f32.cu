@@ -50,7 +50,7 @@ namespace ibim {
 
 constexpr int kSmallTTile = 64;  // targets of a small launch's CTA
 
-template <int TPT, int MINB, int THREADS, int STAGES = kF32Stages, bool FLATNEAR = false>
+template <int TPT, int MINB, int THREADS>
 __global__ void __launch_bounds__(THREADS, MINB)
     pair_f32_kernel(const float4* __restrict__ tpos, const float4* __restrict__ tnrm,
                     const float4* __restrict__ src, const float4* __restrict__ frames, int64_t N, PairSchedule s,
@@ -59,11 +59,11 @@ __global__ void __launch_bounds__(THREADS, MINB)
 {
     constexpr int TTILE = THREADS * TPT;
     constexpr int NW = THREADS / 32;
-    static_assert(TTILE <= kF32MaxTTile && STAGES <= kF32Stages, "tile, stages");
+    static_assert(TTILE <= kF32MaxTTile, "target tile");
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
     if (skip != nullptr && *skip) return;
-    __shared__ __align__(128) SourceStage stg[STAGES];
+    __shared__ __align__(128) SourceStage stg[kF32Stages];
     __shared__ __align__(16) float4 tfrm[NW][2 * TPT];
     __shared__ __align__(8) StagePipe pipe;
 
@@ -80,12 +80,12 @@ __global__ void __launch_bounds__(THREADS, MINB)
 
     auto issue = [&](int64_t u) {
         const int64_t st = ((u % s.n_stiles) * s.sperm) % s.n_stiles;
-        const int stage = (int)((u - s0) % STAGES);
+        const int stage = (int)((u - s0) % kF32Stages);
         pipe_issue(pipe, stg[stage], stage, src + st * (kF32STile / 2) * kPairF4,
                    have_frames ? frames + st * 2 * kChunksPerTile : nullptr);
     };
     if (tid == 0)
-        for (int q = 0; q < STAGES && s0 + q < s1; ++q) issue(s0 + q);
+        for (int q = 0; q < kF32Stages && s0 + q < s1; ++q) issue(s0 + q);
 
     const int64_t t_first = s0 / s.n_stiles;
     int64_t t = t_first;
@@ -121,8 +121,8 @@ __global__ void __launch_bounds__(THREADS, MINB)
     load_targets(t);
 
     for (int64_t u = s0; u < s1; ++u) {
-        const int stage = (int)((u - s0) % STAGES);
-        const uint32_t parity = (uint32_t)(((u - s0) / STAGES) & 1);
+        const int stage = (int)((u - s0) % kF32Stages);
+        const uint32_t parity = (uint32_t)(((u - s0) / kF32Stages) & 1);
         if (!__all_sync(0xffffffffu, ptx::mbar_wait_bounded(&pipe.full[stage], parity, kWaitLimitNs))) {
             if (lane == 0) atomicOr(err, kDevErrTimeout);
             return;
@@ -133,9 +133,8 @@ __global__ void __launch_bounds__(THREADS, MINB)
 #pragma unroll
         for (int q = 0; q < TPT; ++q) S1[q] = C1[q] = S2[q] = C2[q] = 0.0f;
         if (!idle)
-            tile_sums<TPT, false, kChunksPerTile, FLATNEAR>(T, &tfrm[warp][0], have_frames, stg[stage].buf,
-                                                            stg[stage].frm, k, S1, C1, S2, C2, g64, gi0, THREADS,
-                                                            st * kF32STile, N);
+            tile_sums<TPT>(T, &tfrm[warp][0], have_frames, stg[stage].buf, stg[stage].frm, k, S1, C1, S2, C2, g64, gi0,
+                           THREADS, st * kF32STile, N);
 #pragma unroll
         for (int q = 0; q < TPT; ++q) {
             D1[q] += (double)S1[q] - (double)C1[q];
@@ -143,16 +142,16 @@ __global__ void __launch_bounds__(THREADS, MINB)
         }
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(&pipe.empty[stage]);
-        // thread 0 refills the stage of step u - 1 with step u - 1 + STAGES
+        // thread 0 refills the stage of step u - 1 with step u - 1 + kF32Stages
         if (warp == 0) {
             bool ok = true;
-            if (lane == 0 && u > s0 && u - 1 + STAGES < s1) {
+            if (lane == 0 && u > s0 && u - 1 + kF32Stages < s1) {
                 const int64_t v = u - 1 - s0;
-                ok = ptx::mbar_wait_bounded(&pipe.empty[(int)(v % STAGES)], (uint32_t)((v / STAGES) & 1),
+                ok = ptx::mbar_wait_bounded(&pipe.empty[(int)(v % kF32Stages)], (uint32_t)((v / kF32Stages) & 1),
                                             kWaitLimitNs);
                 if (ok) {
                     ptx::fence_proxy_async_smem();
-                    issue(u - 1 + STAGES);
+                    issue(u - 1 + kF32Stages);
                 } else {
                     atomicOr(err, kDevErrTimeout);
                 }
@@ -428,10 +427,10 @@ struct PairArgs {
     bool chained;
 };
 
-template <int TPT, int MINB, int THREADS, int STAGES = kF32Stages, bool FLATNEAR = false>
+template <int TPT, int MINB, int THREADS>
 static void launch_variant(const PairArgs& a, cudaStream_t stream)
 {
-    launch_chained(pair_f32_kernel<TPT, MINB, THREADS, STAGES, FLATNEAR>, dim3(a.s.grid), THREADS, 0, stream, a.chained,
+    launch_chained(pair_f32_kernel<TPT, MINB, THREADS>, dim3(a.s.grid), THREADS, 0, stream, a.chained,
                    a.tpos, a.tnrm, a.src, a.frames, a.N, a.s, a.k, a.part, a.err, a.skip, a.g64);
 }
 
