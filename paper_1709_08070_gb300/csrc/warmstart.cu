@@ -22,10 +22,12 @@
 // the initial residual g - A p0 (A = Lambda + K), which is what GMRES sees:
 // unscaled, the psi block (lambda1 = (1 + eps_E/eps_I)/2, 40.5 for
 // water/protein) would be under-weighted by lambda1^2.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "ibim_internal.cuh"
@@ -44,8 +46,10 @@ constexpr int kWsParams = kOffB3 + kWsOut;  // 4930
 constexpr int kWsThreads = 128;             // prediction: nodes per block
 constexpr int kHPad = kWsH + 1;             // padded smem row (bank conflicts)
 constexpr int kTrainThreads = 256;
-constexpr int kTrainNodes = 64;             // training: nodes per tile
-constexpr int kTrainRow = kTrainNodes + 4;  // row of a transposed tile (16-byte aligned, rows four banks apart)
+constexpr int kTrainBlock = 128;            // training: nodes per block (a pair of CTAs)
+constexpr int kTrainNodes = kTrainBlock / 2;  // a CTA's half of it
+constexpr int kTrainRow = kTrainNodes + 4;  // row of a transposed half (16-byte aligned, rows four banks apart)
+constexpr int kTrainOwn = 20;               // a thread's parameters in the training kernel
 constexpr int kPartStride = kWsParams + 2;  // a CTA's gradient, 16-byte aligned
 
 static_assert(kWsParams == IBIM_WS_NPARAMS, "parameter count");
@@ -72,6 +76,8 @@ struct ibim_wsnet {
 };
 
 namespace ibim {
+
+namespace cg = cooperative_groups;
 
 // ---------------------------------------------------------------- features
 
@@ -220,11 +226,13 @@ struct TrainSmem {
     float b1[kWsH], b2[kWsH], b3[kWsOut + 2];
     float X[kWsIn][kTrainRow];       // activations transposed: [unit][node]
     float H1[kWsH][kTrainRow];
-    float H2[kWsH][kTrainRow];       // then d2
+    float H2[kWsH][kTrainRow];
     float D1[kWsH][kTrainRow];
+    float D2[kWsH][kTrainRow];
     float dO[kWsOut][kTrainRow];
     float e[kWsOut][kTrainRow];
     float wt[kTrainNodes], tgt[kWsOut][kTrainNodes];
+    float carry[kTrainOwn][kTrainThreads];  // second CTA of a pair: the first one's sums
     double loss[kTrainNodes];
 };
 
@@ -250,30 +258,48 @@ __device__ __forceinline__ float dot4(const float4& a, const float4& b, float s)
     return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, s))));
 }
 
+// s + e == a + b exactly (Knuth's two-sum); e is added to lo.
+__device__ __forceinline__ void add_exact(float& hi, float& lo, float x)
+{
+    const float s = hi + x, b = s - hi;
+    lo += (hi - (s - b)) + (x - b);
+    hi = s;
+}
+
 // Loss and gradient over a batch: node of slot s is either consecutive (first +
-// s, full-batch mode) or drawn at random.  The three 64 x 64 x 64 products of a
-// 64-node tile (layer 2 forward, its backward, its weight gradient) run as
-// register tiles of 4 x 4 per thread from shared memory, activations stored
-// transposed so that every operand is a float4; a CTA takes tiles blockIdx.x,
-// + gridDim.x, ... and keeps its weight gradients in registers, then writes
-// them as its partial gradient (summed in a fixed order by ws_update_kernel).
+// s, full-batch mode) or drawn at random.  The gradient is a sum over blocks of
+// 128 nodes: within a block every parameter's products are added node by node in
+// FP32, across blocks the sum is exact to float-float (add_exact here, then
+// ws_update_kernel) and rounded once.  The BF16 weights of the next step turn a
+// difference of one rounding into one of 2^-9 where a weight lies near a
+// boundary, so this order is part of the result (64-node tiles, summed in FP32,
+// left the results of the former one-thread-per-node kernel, FP32 atomics over
+// the same blocks in a varying order, in 4 of 16 runs of 50 steps).
+// A pair of CTAs takes a block: each its half of the nodes through the network and
+// back; the first then forms its sums and hands them over in the second's shared
+// memory, and the second goes on from them.  The products (layer 2 forward, its
+// backward, its weight gradient) run as register tiles of 4 x 4 per thread from
+// shared memory, activations stored transposed so that every operand is a float4.
+// A pair takes blocks p, p + pairs, ... and writes one partial gradient.
 // 242 MFLOP at 8,192 nodes: 3 us of the FP32 pipe; bound by the latency of its
-// eight phases.  Measured 20 us a step with the Adam kernel, launches overlapped
-// (27 us before the overlap and the transposed read of W2, whose copy stored
-// with 32-way bank conflicts; 92 us with one thread per node over shared-memory
-// rows, FP32 atomics and two memsets).
-__global__ void __launch_bounds__(kTrainThreads)
+// phases.  Measured 24 us a step with the Adam kernel, launches overlapped (92 us
+// with one thread per node, FP32 atomics and two memsets; 20 us with 64-node tiles
+// summed apart; 30 us with a whole block on one CTA of 512 threads).
+__global__ void __cluster_dims__(2) __launch_bounds__(kTrainThreads, 1)
     ws_grad_kernel(const float* __restrict__ feat, const float* __restrict__ tgt, const float* __restrict__ wt,
                    int64_t n_ex, int64_t first, int64_t count, int random, uint64_t seed, double inv_batch,
                    const __nv_bfloat16* __restrict__ wb, float* __restrict__ part, double* __restrict__ part_loss)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     TrainSmem& S = *reinterpret_cast<TrainSmem*>(smem_raw);
+    const cg::cluster_group pair = cg::this_cluster();
+    const int second = (int)pair.block_rank();
+    const int64_t npairs = gridDim.x / 2, first_block = blockIdx.x / 2;
     const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
     // four threads per node fetch its features, target and weight (zeros past the batch)
-    auto fetch = [&](int64_t tile) {
+    auto fetch = [&](int64_t block) {
         const int n = t & (kTrainNodes - 1), part4 = t / kTrainNodes;
-        const int64_t slot = tile * kTrainNodes + n;
+        const int64_t slot = block * kTrainBlock + second * kTrainNodes + n;
         const bool live = slot < count;
         int64_t i = 0;
         if (live) i = random ? (int64_t)(mix64(seed ^ (uint64_t)slot) % (uint64_t)n_ex) : first + slot;
@@ -282,8 +308,8 @@ __global__ void __launch_bounds__(kTrainThreads)
         if (part4 >= 1 && part4 <= kWsOut) S.tgt[part4 - 1][n] = live ? tgt[kWsOut * i + part4 - 1] : 0.0f;
     };
     ptx::grid_dep_launch();  // the Adam kernel may be set up; it waits for this grid
-    // this step's first tile of features while the previous Adam step finishes
-    fetch(blockIdx.x);
+    // this step's first features while the previous Adam step finishes
+    fetch(first_block);
     ptx::grid_dep_wait();
     const __nv_bfloat162* w2 = reinterpret_cast<const __nv_bfloat162*>(wb + kOffW2);
 #pragma unroll 4
@@ -304,20 +330,21 @@ __global__ void __launch_bounds__(kTrainThreads)
     }
     if (t < kWsOut) S.b3[t] = __bfloat162float(wb[kOffB3 + t]);
 
-    float gW2[4][4];                              // units ty + 16 i (layer 2) x tx + 16 j (layer 1)
-    float gW1[3] = {0.0f, 0.0f, 0.0f};            // unit t % 64, inputs t / 64 + 4 i; the bias in the last
-    float gW3 = 0.0f, gB2 = 0.0f, gB3 = 0.0f;     // t < 128: W3[t / 64][t % 64]; 128 <= t < 192: b2; t < 2: b3
-    double l = 0.0;
+    // a thread's parameters: W2, units ty + 16 i (layer 2) x tx + 16 j (layer 1); W1, unit t % 64 and inputs
+    // t / 64 + 4 i, the bias in the last; W3[t / 64][t % 64] (t < 128), b2 (t - 128 < 64) or b3 (t - 192 < 2)
+    constexpr int kW1 = 16, kRest = 19;
+    const bool ownW3 = t < 128, ownB2 = t >= 128 && t < 192, ownB3 = t >= 192 && t < 192 + kWsOut;
+    float hi[kTrainOwn], lo[kTrainOwn];  // sums over the pair's blocks
+    double l = 0.0;                      // t < 64: loss of the half's nodes t
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) gW2[i][j] = 0.0f;
+    for (int q = 0; q < kTrainOwn; ++q) hi[q] = lo[q] = 0.0f;
 
-    for (int64_t tile = blockIdx.x; tile * kTrainNodes < count; tile += gridDim.x) {
-        if (tile != blockIdx.x) {
+    for (int64_t block = first_block; block * kTrainBlock < count; block += npairs) {
+        if (block != first_block) {
             __syncthreads();
-            fetch(tile);
+            fetch(block);
         }
+        pair.barrier_arrive();  // the second CTA's hand-over buffer is free
         __syncthreads();
         float acc[4][4];  // nodes 4 ty + i, units 4 tx + j
 #pragma unroll
@@ -345,7 +372,7 @@ __global__ void __launch_bounds__(kTrainThreads)
             float s = S.b3[c];
 #pragma unroll 8
             for (int a = 0; a < kWsH; ++a) s = fmaf(S.W3[c][a], S.H2[a][n], s);
-            const float e = tile * kTrainNodes + n < count ? s - S.tgt[c][n] : 0.0f;
+            const float e = block * kTrainBlock + second * kTrainNodes + n < count ? s - S.tgt[c][n] : 0.0f;
             S.e[c][n] = e;
             S.dO[c][n] = (float)(2.0 * inv_batch) * S.wt[n] * e;
         }
@@ -354,28 +381,19 @@ __global__ void __launch_bounds__(kTrainThreads)
             const float w = S.wt[t], e0 = S.e[0][t], e1 = S.e[1][t];
             l += (double)w * ((double)e0 * e0 + (double)e1 * e1) * inv_batch;
         }
-        if (t < kWsOut * kWsH) {  // dW3[c][a] += sum_n dO[n][c] h2[n][a]
-            const int c = t / kWsH, a = t % kWsH;
-#pragma unroll 4
-            for (int n = 0; n < kTrainNodes; n += 4)
-                gW3 = dot4(*reinterpret_cast<const float4*>(&S.dO[c][n]), *reinterpret_cast<const float4*>(&S.H2[a][n]), gW3);
-        }
-        if (t < kWsOut)
-            for (int n = 0; n < kTrainNodes; ++n) gB3 += S.dO[t][n];
-        __syncthreads();
-        for (int q = t; q < kWsH * kTrainNodes; q += kTrainThreads) {  // d2 in the place of h2
+        for (int q = t; q < kWsH * kTrainNodes; q += kTrainThreads) {
             const int a = q / kTrainNodes, n = q % kTrainNodes;
             const float h = S.H2[a][n];
             float s = fmaf(S.W3[0][a], S.dO[0][n], 0.0f);
             s = fmaf(S.W3[1][a], S.dO[1][n], s);
-            S.H2[a][n] = s * (1.0f - h * h);
+            S.D2[a][n] = s * (1.0f - h * h);
         }
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
             for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
-        tile_product<kWsH>(S.H2, S.W2, ty, tx, acc);  // d1 before the derivative of tanh
+        tile_product<kWsH>(S.D2, S.W2, ty, tx, acc);  // d1 before the derivative of tanh
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const float4 h = *reinterpret_cast<const float4*>(&S.H1[4 * tx + j][4 * ty]);
@@ -383,51 +401,83 @@ __global__ void __launch_bounds__(kTrainThreads)
                 make_float4(acc[0][j] * (1.0f - h.x * h.x), acc[1][j] * (1.0f - h.y * h.y),
                             acc[2][j] * (1.0f - h.z * h.z), acc[3][j] * (1.0f - h.w * h.w));
         }
-#pragma unroll 2
-        for (int n = 0; n < kTrainNodes; n += 4) {  // dW2[a][b] += sum_n d2[n][a] h1[n][b]
-            float4 d[4], h[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                d[i] = *reinterpret_cast<const float4*>(&S.H2[ty + 16 * i][n]);
-                h[i] = *reinterpret_cast<const float4*>(&S.H1[tx + 16 * i][n]);
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) gW2[i][j] = dot4(d[i], h[j], gW2[i][j]);
-        }
-        if (t >= 2 * kWsH && t < 3 * kWsH)
-            for (int n = 0; n < kTrainNodes; ++n) gB2 += S.H2[t - 2 * kWsH][n];
         __syncthreads();
-        {  // dW1[a][b] += sum_n d1[n][a] x[n][b], the bias as one more input
-            const int a = t % kWsH, b0 = t / kWsH;
+        pair.barrier_wait();
+        // the block's sums, node by node: the first CTA's from zero, the second's from the first's
+        float g[kTrainOwn];
+        auto sums = [&]() {
+#pragma unroll 2
+            for (int n = 0; n < kTrainNodes; n += 4) {  // dW2[a][b] = sum_n d2[n][a] h1[n][b]
+                float4 d[4], h[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    d[i] = *reinterpret_cast<const float4*>(&S.D2[ty + 16 * i][n]);
+                    h[i] = *reinterpret_cast<const float4*>(&S.H1[tx + 16 * i][n]);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) g[4 * i + j] = dot4(d[i], h[j], g[4 * i + j]);
+            }
 #pragma unroll 4
-            for (int n = 0; n < kTrainNodes; n += 4) {
-                const float4 d = *reinterpret_cast<const float4*>(&S.D1[a][n]);
+            for (int n = 0; n < kTrainNodes; n += 4) {  // dW1[a][b] = sum_n d1[n][a] x[n][b], the bias as one more input
+                const float4 d = *reinterpret_cast<const float4*>(&S.D1[t % kWsH][n]);
 #pragma unroll
                 for (int i = 0; i < 3; ++i) {
-                    const int b = b0 + 4 * i;
-                    if (b < kWsIn) gW1[i] = dot4(d, *reinterpret_cast<const float4*>(&S.X[b][n]), gW1[i]);
-                    else if (b == kWsIn) gW1[i] += (d.x + d.y) + (d.z + d.w);
+                    const int b = t / kWsH + 4 * i;
+                    if (b < kWsIn) g[kW1 + i] = dot4(d, *reinterpret_cast<const float4*>(&S.X[b][n]), g[kW1 + i]);
+                    else if (b == kWsIn) g[kW1 + i] = (((g[kW1 + i] + d.x) + d.y) + d.z) + d.w;
                 }
             }
+            if (ownW3)  // dW3[c][a] = sum_n dO[n][c] h2[n][a]
+#pragma unroll 4
+                for (int n = 0; n < kTrainNodes; n += 4)
+                    g[kRest] = dot4(*reinterpret_cast<const float4*>(&S.dO[t / kWsH][n]),
+                                    *reinterpret_cast<const float4*>(&S.H2[t % kWsH][n]), g[kRest]);
+            else if (ownB2 || ownB3) {
+                const float* row = ownB2 ? S.D2[t - 128] : S.dO[t - 192];
+#pragma unroll 8
+                for (int n = 0; n < kTrainNodes; ++n) g[kRest] += row[n];
+            }
+        };
+        if (!second) {
+#pragma unroll
+            for (int q = 0; q < kTrainOwn; ++q) g[q] = 0.0f;
+            sums();
+            float* carry = pair.map_shared_rank(&S.carry[0][0], 1);
+#pragma unroll
+            for (int q = 0; q < kTrainOwn; ++q) carry[q * kTrainThreads + t] = g[q];
+        }
+        pair.sync();
+        if (second) {
+#pragma unroll
+            for (int q = 0; q < kTrainOwn; ++q) g[q] = S.carry[q][t];
+            sums();
+#pragma unroll
+            for (int q = 0; q < kTrainOwn; ++q) add_exact(hi[q], lo[q], g[q]);
         }
     }
 
-    float* g = part + (int64_t)blockIdx.x * kPartStride;
+    // the pair's partial gradient; with several blocks the low parts as a second one
+    auto store = [&](float* p, const float (&v)[kTrainOwn]) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) g[kOffW2 + (ty + 16 * i) * kWsH + tx + 16 * j] = gW2[i][j];
+            for (int j = 0; j < 4; ++j) p[kOffW2 + (ty + 16 * i) * kWsH + tx + 16 * j] = v[4 * i + j];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        const int a = t % kWsH, b = t / kWsH + 4 * i;
-        if (b < kWsIn) g[kOffW1 + a * kWsIn + b] = gW1[i];
-        else if (b == kWsIn) g[kOffB1 + a] = gW1[i];
+        for (int i = 0; i < 3; ++i) {
+            const int a = t % kWsH, b = t / kWsH + 4 * i;
+            if (b < kWsIn) p[kOffW1 + a * kWsIn + b] = v[kW1 + i];
+            else if (b == kWsIn) p[kOffB1 + a] = v[kW1 + i];
+        }
+        if (ownW3) p[kOffW3 + t] = v[kRest];
+        if (ownB2) p[kOffB2 + t - 128] = v[kRest];
+        if (ownB3) p[kOffB3 + t - 192] = v[kRest];
+    };
+    if (second) {
+        store(part + first_block * kPartStride, hi);
+        if (count > npairs * kTrainBlock) store(part + (npairs + first_block) * kPartStride, lo);
     }
-    if (t < kWsOut * kWsH) g[kOffW3 + t] = gW3;
-    if (t >= 2 * kWsH && t < 3 * kWsH) g[kOffB2 + t - 2 * kWsH] = gB2;
-    if (t < kWsOut) g[kOffB3 + t] = gB3;
     if (t < kTrainNodes) S.loss[t] = l;
     for (int o = kTrainNodes / 2; o > 0; o >>= 1) {
         __syncthreads();
@@ -436,36 +486,38 @@ __global__ void __launch_bounds__(kTrainThreads)
     if (t == 0) part_loss[blockIdx.x] = S.loss[0];
 }
 
-// Sums the CTAs' partial gradients (kSumParts threads per parameter over fixed
-// shares) and losses; with adam, one Adam step (Kingma and Ba 2015) on the FP32
+// Sums the partial gradients (kSumParts threads per parameter over fixed shares,
+// exact to float-float) and the CTAs' losses; with adam, one Adam step (Kingma and Ba 2015) on the FP32
 // master weights, which refreshes the BF16 copy; else the gradient goes to grad.
 constexpr int kSumParts = 8, kSumParams = 32;
 __global__ void __launch_bounds__(kSumParts * kSumParams)
-    ws_update_kernel(const float* __restrict__ part, const double* __restrict__ part_loss, int nparts, int adam,
+    ws_update_kernel(const float* __restrict__ part, const double* __restrict__ part_loss, int nparts, int ctas, int adam,
                      float* __restrict__ w, float* __restrict__ m, float* __restrict__ v, __nv_bfloat16* __restrict__ wb,
                      float lr, float b1, float b2, float c1, float c2, float* __restrict__ grad,
                      double* __restrict__ loss)
 {
-    __shared__ float sh[kSumParts][kSumParams];
+    __shared__ double sh[kSumParts][kSumParams];
     ptx::grid_dep_launch();  // the next step's gradient may be set up; it waits for this grid
     ptx::grid_dep_wait();
     const int ql = threadIdx.x % kSumParams, pr = threadIdx.x / kSumParams;
     const int q = blockIdx.x * kSumParams + ql;
-    float s = 0.0f;
+    float hi = 0.0f, lo = 0.0f;
     if (q < kWsParams) {
 #pragma unroll 8
-        for (int p = pr; p < nparts; p += kSumParts) s += part[(int64_t)p * kPartStride + q];
+        for (int p = pr; p < nparts; p += kSumParts) add_exact(hi, lo, part[(int64_t)p * kPartStride + q]);
     }
-    sh[pr][ql] = s;
+    double d = (double)hi + (double)lo;
+    sh[pr][ql] = d;
     if (blockIdx.x == 0 && threadIdx.x < 32) {
-        double d = 0.0;
-        for (int p = threadIdx.x; p < nparts; p += 32) d += part_loss[p];
-        for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-        if (threadIdx.x == 0) *loss = d;
+        double v = 0.0;
+        for (int p = threadIdx.x; p < ctas; p += 32) v += part_loss[p];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (threadIdx.x == 0) *loss = v;
     }
     __syncthreads();
     if (pr != 0 || q >= kWsParams) return;
-    for (int p = 1; p < kSumParts; ++p) s += sh[p][ql];
+    for (int p = 1; p < kSumParts; ++p) d += sh[p][ql];
+    const float s = (float)d;
     if (!adam) {
         grad[q] = s;
         return;
@@ -486,11 +538,13 @@ __global__ void ws_to_bf16_kernel(const float* __restrict__ w, __nv_bfloat16* __
 }
 
 static size_t grad_smem() { return sizeof(TrainSmem); }
-// CTAs of a training launch: one per SM, each over its share of the tiles
+// CTAs of a training launch: a pair for each block, at most one CTA per SM
 static unsigned grad_ctas(const ibim_wsnet* n, int64_t count)
 {
-    return (unsigned)std::min<int64_t>(n->num_sms, (count + kTrainNodes - 1) / kTrainNodes);
+    return 2u * (unsigned)std::min<int64_t>(std::max(1, n->num_sms / 2), (count + kTrainBlock - 1) / kTrainBlock);
 }
+// partial gradients of such a launch (see ws_grad_kernel)
+static int grad_nparts(unsigned ctas, int64_t count) { return (int)ctas / 2 * (count > (int64_t)ctas * kTrainNodes ? 2 : 1); }
 // the partial gradients behind the gradient, the partial losses behind the loss
 static float* grad_parts(const ibim_wsnet* n) { return n->d_g + kPartStride; }
 static double* loss_parts(const ibim_wsnet* n) { return n->d_loss + 2; }
@@ -590,8 +644,8 @@ ibim_status ibim_wsnet_create(uint64_t seed, void* stream, ibim_wsnet** out)
     if (e == cudaSuccess) e = cudaMalloc((void**)&n->d_m, sizeof(float) * kWsParams);
     if (e == cudaSuccess) e = cudaMalloc((void**)&n->d_v, sizeof(float) * kWsParams);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n->num_sms, cudaDevAttrMultiProcessorCount, n->device);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&n->d_g, sizeof(float) * kPartStride * (1 + (size_t)n->num_sms));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&n->d_loss, sizeof(double) * (2 + (size_t)n->num_sms));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&n->d_g, sizeof(float) * kPartStride * (2 + (size_t)n->num_sms));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&n->d_loss, sizeof(double) * (3 + (size_t)n->num_sms));
     if (e == cudaSuccess) e = cudaMalloc((void**)&n->d_scal, sizeof(double) * 4);
     if (e == cudaSuccess) e = cudaMemcpyAsync(n->d_w, w.data(), sizeof(float) * kWsParams, cudaMemcpyHostToDevice, n->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(n->d_m, 0, sizeof(float) * kWsParams, n->stream);
@@ -731,7 +785,7 @@ ibim_status ibim_wsnet_gradient(ibim_wsnet* n, int64_t first, int64_t count, dou
                                                                     0, 0, 1.0 / (double)count, n->d_wb, grad_parts(n),
                                                                     loss_parts(n));
     ws_update_kernel<<<(kWsParams + kSumParams - 1) / kSumParams, kSumParts * kSumParams, 0, n->stream>>>(
-        grad_parts(n), loss_parts(n), (int)ctas, 0, n->d_w, n->d_m, n->d_v, n->d_wb, 0.0f, 0.0f, 0.0f, 1.0f, 1.0f,
+        grad_parts(n), loss_parts(n), grad_nparts(ctas, count), (int)ctas, 0, n->d_w, n->d_m, n->d_v, n->d_wb, 0.0f, 0.0f, 0.0f, 1.0f, 1.0f,
         n->d_g, n->d_loss);
     IBIM_CUDA(cudaGetLastError());
     IBIM_CUDA(cudaMemcpyAsync(h_grad, n->d_g, sizeof(float) * kWsParams, cudaMemcpyDeviceToHost, n->stream));
@@ -777,7 +831,7 @@ ibim_status ibim_wsnet_train(ibim_wsnet* n, int steps, int batch_nodes, double l
                                      loss_parts(n)));
         const float c1 = (float)(1.0 - pow(b1, (double)n->step)), c2 = (float)(1.0 - pow(b2, (double)n->step));
         IBIM_CUDA(cudaLaunchKernelEx(&sum_cfg, ws_update_kernel, (const float*)grad_parts(n),
-                                     (const double*)loss_parts(n), (int)ctas, 1, n->d_w, n->d_m, n->d_v, n->d_wb,
+                                     (const double*)loss_parts(n), grad_nparts(ctas, batch_nodes), (int)ctas, 1, n->d_w, n->d_m, n->d_v, n->d_wb,
                                      (float)lr, (float)b1, (float)b2, c1, c2, n->d_g, n->d_loss));
     }
     if (last_loss) {
