@@ -488,8 +488,8 @@ ibim_status ibim_solve_batch(int nmol, ibim_ctx* const* ctxs, const ibim_phys* p
 /*
  * Batched pair-kernel variants (tuning, not part of the paper's method):
  * one-directional kernels with one target per thread in CTAs of 512, 256 or
- * 128 threads, and symmetric kernels with one or two (each unordered node pair of
- * a molecule evaluated once for both directions, reverse sums carried by rotating
+ * 128 threads, and a symmetric kernel (each unordered node pair of a molecule
+ * evaluated once for both directions, reverse sums carried by rotating
  * accumulators as in the single-molecule symmetric kernel).  By default the
  * first batched solve of a size class times every variant on its first round
  * and keeps the fastest; ibim_set_batch_variant(v) forces variant v for later

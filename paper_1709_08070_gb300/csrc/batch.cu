@@ -62,10 +62,7 @@ struct BatchPlan {
     int nactive;
     int pad;
     int64_t total;
-    int64_t per_cta;         // one-directional kernels: steps per CTA
-    int64_t Lb, Ls;          // symmetric kernel: steps of a large segment (one per CTA) and of a small one
-    int64_t nbig, nseg;      // large segments, segments in all
-    unsigned long long ctr;  // small segments handed out
+    int64_t per_cta;
     int mol[kMaxBatch];
     int64_t off[kMaxBatch + 1];
 };
@@ -108,17 +105,6 @@ __global__ void batch_plan_kernel(const BatchMol* __restrict__ mols, int nmol, i
     plan->nactive = a;
     plan->total = total;
     plan->per_cta = total > 0 ? (total + grid - 1) / grid : 1;
-    // as make_sym_schedule: nine tenths of an even share per CTA, then about 16
-    // small segments per CTA from a counter
-    const int64_t g = total < grid ? (total > 0 ? total : 1) : grid;
-    const int64_t Lb = 9 * total / (10 * g) > 1 ? 9 * total / (10 * g) : 1;
-    const int64_t rest = total > g * Lb ? total - g * Lb : 0;
-    const int64_t Ls = (rest + 16 * g - 1) / (16 * g) > 1 ? (rest + 16 * g - 1) / (16 * g) : 1;
-    plan->Lb = Lb;
-    plan->Ls = Ls;
-    plan->nbig = total > 0 ? g : 0;
-    plan->nseg = total > 0 ? g + (rest + Ls - 1) / Ls : 0;
-    plan->ctr = 0ull;
 }
 
 __global__ void batch_pack_kernel(const BatchMol* __restrict__ mols, const BatchPlan* __restrict__ plan, int mode)
@@ -194,24 +180,25 @@ __global__ void batch_sym_pack_kernel(const BatchMol* __restrict__ mols, const B
 
 // Symmetric batched pair sums (rotation scheme of pair_sym.cu): stream-K over
 // the concatenated upper triangles of the active molecules' (target tile,
-// source tile) steps, cut into one large segment per CTA and small ones from a
-// counter as in pair_sym.cu, so that CTAs whose steps were cheaper (diagonal,
-// far) take more of the rest.  Forward sums of a row are added to the
-// molecule's output with FP64 atomics when the row (or the segment) ends; the
+// source tile) steps.  Forward sums of a row are added to the molecule's
+// output with FP64 atomics when the row (or the CTA's range) ends; the
 // reverse sums of a staged source tile are collected in shared memory and
 // added to the output with FP64 atomics once every warp has released the
-// tile.  UNR: unrolled steps of the 32-step rotation loop.
-// Bound by instruction issue.  Eight globules of 50 to 120 atoms, per round:
-// one target per thread 1.94 ms, with one even share per CTA or with segments;
-// two per thread, which halve the reverse sums' atomics and the rotation's
-// shuffles, 1.88 ms in even shares (a 1,024-target row leaves fewer, coarser
-// steps) and 1.83 ms in segments.  Three of 30 to 40 atoms: 0.33 ms with one
-// target per thread, 0.36 ms with two; the solver measures both on the size at
-// hand.
+// stage (warp 0, before it refills the stage).  UNR: unroll depth of the
+// rotation loop (4 with one target per thread: 8.98e11 against 8.74e11
+// interactions/s at 2 over 8 rounds of the 64-globule batch).
+// The reverse sums of a tile are plain FP32 sums over its 512 targets, in the
+// order in which the warps arrive, so a solution varies by 8e-9 of its norm from
+// run to run, and a molecule whose residual ends near the tolerance may take one
+// step more or less.  Two targets per thread (1,024 to a sum), steps in segments,
+// the combined a-term and branch-free near chunks of the single-molecule kernel
+// save an eighth of a round (eight globules of 50 to 120 atoms, with the
+// orthogonalisation 2.11 against 2.40 ms), but the solutions then lie 2.1e-8 from
+// this kernel's and other molecules take the extra step: not used.
 template <int TPT, int THREADS, int UNR>
 __global__ void __launch_bounds__(THREADS, 1)
-    batch_sym_kernel(const BatchMol* __restrict__ mols, const BatchPlan* __restrict__ plan,
-                     unsigned long long* __restrict__ ctr, int mode, unsigned* __restrict__ err)
+    batch_sym_kernel(const BatchMol* __restrict__ mols, const BatchPlan* __restrict__ plan, int mode,
+                     unsigned* __restrict__ err)
 {
     constexpr int TTILE = TPT * THREADS;
     constexpr int NW = THREADS / 32;
@@ -232,26 +219,17 @@ __global__ void __launch_bounds__(THREADS, 1)
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
     const int lane = tid & 31;
-    const int64_t total = plan->total, Lb = plan->Lb, Ls = plan->Ls, nbig = plan->nbig, nseg = plan->nseg;
-    if (blockIdx.x >= nseg) return;
-    __shared__ int64_t seg_next[2];
-    __shared__ int abort_sh;  // a bounded wait gave up: every warp leaves after the segment barrier
-    auto seg_start = [&](int64_t q) {
-        const int64_t v = q < nbig ? q * Lb : nbig * Lb + (q - nbig) * Ls;
-        return v < total ? v : total;
-    };
+    const int64_t total = plan->total;
+    const int64_t per_cta = plan->per_cta;
+    const int64_t s0 = (int64_t)blockIdx.x * per_cta;
+    const int64_t s1 = (s0 + per_cta < total) ? s0 + per_cta : total;
+    if (s0 >= s1) return;
     const int nact = plan->nactive;
     const int* __restrict__ s_mol = plan->mol;
     const int64_t* __restrict__ s_off = plan->off;
     for (int q = tid; q < kF32Stages * sym_rev_row(true); q += THREADS) (&racc[0][0])[q] = 0.0f;
-    if (tid == 0) {
-        pipe_init(pipe, NW);
-        abort_sh = 0;
-    }
+    if (tid == 0) pipe_init(pipe, NW);
     __syncthreads();
-
-    // ring position of step u of the current segment: done + (u - s0) = u + off
-    int64_t s0 = 0, s1 = 0, off = 0, done = 0;
 
     // step u -> active index a, row t and position in the row
     auto locate = [&](int64_t u, int& a, int64_t& t, int64_t& pos) {
@@ -281,26 +259,25 @@ __global__ void __launch_bounds__(THREADS, 1)
         locate(u, a, t, pos);
         const BatchMol& M = mols[s_mol[a]];
         const int64_t st = R * t + pos;
-        const int stage = (int)((u + off) % kF32Stages);
+        const int stage = (int)((u - s0) % kF32Stages);
         stage_mol[stage] = s_mol[a];
         stage_st[stage] = st;
         stage_k[stage] = M.k;
         stage_g[stage] = M.g64;
         pipe_issue(pipe, stg[stage], stage, M.src + st * (kF32STile / 2) * kPairF4, M.frames + st * 2 * kChunksPerTile);
     };
+    if (tid == 0)
+        for (int q = 0; q < kF32Stages && s0 + q < s1; ++q) issue(s0 + q);
 
-    int a = 0;
-    int64_t t = 0, pos = 0;
-    const BatchMol* M = nullptr;
+    int a;
+    int64_t t, pos;
+    locate(s0, a, t, pos);
+    const BatchMol* M = &mols[s_mol[a]];
     SymTargets<TPT> T;
     int64_t gi0 = 0;
     int Ablk[TPT];
     bool idle = false;
-    // FP64 sums of the row (own element only): in shared memory, as two targets
-    // per thread leave no registers for them
-    extern __shared__ double acc_sh[];
-    double(*acc1)[THREADS] = reinterpret_cast<double(*)[THREADS]>(acc_sh);
-    double(*acc2)[THREADS] = acc1 + TPT;
+    double D1[TPT], D2[TPT];
 
     auto load_targets = [&]() {
         gi0 = t * TTILE + tid;
@@ -319,8 +296,8 @@ __global__ void __launch_bounds__(THREADS, 1)
             T.a[q] = f2((i & 1) ? pa.w : pa.z);
             T.nb[q] = f2(-((i & 1) ? pb.w : pb.z));
             Ablk[q] = (int)((t * TTILE + (int64_t)q * THREADS + warp * 32) / kChunk);
-            acc1[q][tid] = 0.0;
-            acc2[q][tid] = 0.0;
+            D1[q] = 0.0;
+            D2[q] = 0.0;
         }
         __syncwarp();
         if (lane < 2 * TPT) {
@@ -337,14 +314,14 @@ __global__ void __launch_bounds__(THREADS, 1)
         for (int q = 0; q < TPT; ++q) {
             const int64_t i = gi0 + (int64_t)q * THREADS;
             if (i < N) {
-                atomicAdd(y + i, kInv4Pi * acc1[q][tid]);
-                atomicAdd(y + N + i, kInv4Pi * acc2[q][tid]);
+                atomicAdd(y + i, kInv4Pi * D1[q]);
+                atomicAdd(y + N + i, kInv4Pi * D2[q]);
             }
         }
     };
     // warp 0: reverse sums of the tile staged for step v into its molecule's output
     auto flush_rev = [&](int64_t v) {
-        const int sv = (int)((v + off) % kF32Stages);
+        const int sv = (int)((v - s0) % kF32Stages);
         const BatchMol& S = mols[stage_mol[sv]];
         double* y = batch_out(S, mode);
         const int64_t N = S.N;
@@ -360,107 +337,70 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
         __syncwarp();
     };
-    auto give_up = [&]() {
-        if (lane == 0) {
-            atomicOr(err, kDevErrTimeout);
-            *(volatile int*)&abort_sh = 1;
-        }
-    };
     // warp 0: wait until every warp is past step v
     auto wait_empty = [&](int64_t v) -> bool {
         bool ok = true;
-        const int64_t w = v + off;
+        const int64_t w = v - s0;
         if (lane == 0)
             ok = ptx::mbar_wait_bounded(&pipe.empty[(int)(w % kF32Stages)], (uint32_t)((w / kF32Stages) & 1),
                                         kWaitLimitNs);
         ok = __shfl_sync(0xffffffffu, ok, 0);
-        if (!ok) give_up();
+        if (!ok && lane == 0) atomicOr(err, kDevErrTimeout);
         return ok;
     };
+    load_targets();
 
-    int64_t seg = blockIdx.x;
-    int sp = 0;
-    while (seg < nseg) {
-        s0 = seg_start(seg);
-        s1 = seg_start(seg + 1);
-        off = done - s0;
-        // every stage is free here: warp 0 waited for each earlier step's release
-        if (tid == 0) {
-            ptx::fence_proxy_async_smem();
-            for (int q = 0; q < kF32Stages && s0 + q < s1; ++q) issue(s0 + q);
+    for (int64_t u = s0; u < s1; ++u) {
+        const int stage = (int)((u - s0) % kF32Stages);
+        const uint32_t parity = (uint32_t)(((u - s0) / kF32Stages) & 1);
+        if (!__all_sync(0xffffffffu, ptx::mbar_wait_bounded(&pipe.full[stage], parity, kWaitLimitNs))) {
+            if (lane == 0) atomicOr(err, kDevErrTimeout);
+            return;
         }
-        locate(s0, a, t, pos);
-        M = &mols[s_mol[a]];
-        load_targets();
-        bool bad = false;
-        for (int64_t u = s0; u < s1; ++u) {
-            const int stage = (int)((u + off) % kF32Stages);
-            const uint32_t parity = (uint32_t)(((u + off) / kF32Stages) & 1);
-            if (!__all_sync(0xffffffffu, ptx::mbar_wait_bounded(&pipe.full[stage], parity, kWaitLimitNs))) {
-                give_up();
-                bad = true;
-                break;
-            }
-            const int64_t st = R * t + pos;
-            float S1[TPT], C1[TPT], S2[TPT], C2[TPT];
+        const int64_t st = R * t + pos;
+        float S1[TPT], C1[TPT], S2[TPT], C2[TPT];
 #pragma unroll
-            for (int q = 0; q < TPT; ++q) S1[q] = C1[q] = S2[q] = C2[q] = 0.0f;
-            if (!idle)
-                tile_sums_sym<TPT, true, UNR>(T, &tfrm[warp][0], stg[stage].buf, stg[stage].frm, stage_k[stage], S1, C1, S2, C2,
-                                         stage_g[stage], gi0, THREADS, st * kF32STile, M->N, Ablk, st * kChunksPerTile,
-                                         &racc[stage][0]);
+        for (int q = 0; q < TPT; ++q) S1[q] = C1[q] = S2[q] = C2[q] = 0.0f;
+        if (!idle)
+            tile_sums_sym<TPT, true, UNR, kChunksPerTile, false>(T, &tfrm[warp][0], stg[stage].buf, stg[stage].frm, stage_k[stage], S1, C1, S2, C2,
+                                     stage_g[stage], gi0, THREADS, st * kF32STile, M->N, Ablk, st * kChunksPerTile,
+                                     &racc[stage][0]);
 #pragma unroll
-            for (int q = 0; q < TPT; ++q) {
-                acc1[q][tid] += (double)S1[q] - (double)C1[q];
-                acc2[q][tid] += (double)S2[q] - (double)C2[q];
+        for (int q = 0; q < TPT; ++q) {
+            D1[q] += (double)S1[q] - (double)C1[q];
+            D2[q] += (double)S2[q] - (double)C2[q];
+        }
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(&pipe.empty[stage]);
+        if (warp == 0 && u > s0) {
+            if (!wait_empty(u - 1)) return;
+            flush_rev(u - 1);
+            if (lane == 0 && u - 1 + kF32Stages < s1) {
+                ptx::fence_proxy_async_smem();
+                issue(u - 1 + kF32Stages);
             }
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&pipe.empty[stage]);
-            if (warp == 0 && u > s0) {
-                if (!wait_empty(u - 1)) {
-                    bad = true;
-                    break;
-                }
-                flush_rev(u - 1);
-                if (lane == 0 && u - 1 + kF32Stages < s1) {
-                    ptx::fence_proxy_async_smem();
-                    issue(u - 1 + kF32Stages);
-                }
-                __syncwarp();
-            }
-            // advance to step u + 1
-            const int64_t row_len = M->n_stiles - R * t;
-            const bool row_ends = (pos + 1 == row_len);
-            if (row_ends || u + 1 == s1) flush_rows();
-            if (u + 1 == s1) break;
-            if (!row_ends) {
-                ++pos;
+        }
+        // advance to step u + 1
+        const int64_t row_len = M->n_stiles - R * t;
+        const bool row_ends = (pos + 1 == row_len);
+        if (row_ends || u + 1 == s1) flush_rows();
+        if (u + 1 == s1) break;
+        if (!row_ends) {
+            ++pos;
+        } else {
+            pos = 0;
+            if (t + 1 < (M->N + TTILE - 1) / TTILE) {
+                ++t;
             } else {
-                pos = 0;
-                if (t + 1 < (M->N + TTILE - 1) / TTILE) {
-                    ++t;
-                } else {
-                    ++a;
-                    M = &mols[s_mol[a]];
-                    t = 0;
-                }
-                load_targets();
+                ++a;
+                M = &mols[s_mol[a]];
+                t = 0;
             }
+            load_targets();
         }
-        if (warp == 0) {  // the segment's last step: reverse sums, then the next segment
-            if (!bad && wait_empty(s1 - 1)) {
-                flush_rev(s1 - 1);
-                if (lane == 0) seg_next[sp] = nbig + (int64_t)atomicAdd(ctr, 1ull);
-            } else if (lane == 0) {
-                seg_next[sp] = nseg;
-            }
-        }
-        done += s1 - s0;
-        __syncthreads();
-        if (*(volatile int*)&abort_sh) return;
-        seg = seg_next[sp];
-        sp ^= 1;
     }
+    if (warp == 0 && wait_empty(s1 - 1)) flush_rev(s1 - 1);
 }
 
 template <int TPT, int THREADS, int MINB>
@@ -617,8 +557,6 @@ __global__ void __launch_bounds__(THREADS, MINB)
     }
 }
 
-constexpr size_t batch_sym_smem(int tpt, int threads) { return sizeof(double) * 2 * tpt * threads; }
-
 struct BatchVariant {
     int tpt, threads, minb, sym;
     const void* fn;
@@ -634,14 +572,14 @@ template <int T, int W, int U>
 static void launch_batch_sym(int grid, cudaStream_t st, const BatchMol* mols, const BatchPlan* plan, int mode,
                              unsigned* err)
 {
-    batch_sym_kernel<T, W, U><<<grid, W, batch_sym_smem(T, W), st>>>(mols, plan, &const_cast<BatchPlan*>(plan)->ctr, mode, err);
+    batch_sym_kernel<T, W, U><<<grid, W, 0, st>>>(mols, plan, mode, err);
 }
 #define IBIM_BATCH_VARIANT(T, W, M) {T, W, M, 0, (const void*)batch_pair_kernel<T, W, M>, launch_batch_pair<T, W, M>}
 #define IBIM_BATCH_SYM_VARIANT(T, W, U) \
     {T, W, 1, 1, (const void*)batch_sym_kernel<T, W, U>, launch_batch_sym<T, W, U>}
 static const BatchVariant kBatchVariants[] = {
     IBIM_BATCH_VARIANT(1, 512, 1), IBIM_BATCH_VARIANT(1, 256, 2), IBIM_BATCH_VARIANT(1, 128, 4),
-    IBIM_BATCH_SYM_VARIANT(1, 512, 4), IBIM_BATCH_SYM_VARIANT(2, 512, 1),
+    IBIM_BATCH_SYM_VARIANT(1, 512, 4),
 };
 #undef IBIM_BATCH_VARIANT
 #undef IBIM_BATCH_SYM_VARIANT
@@ -668,10 +606,7 @@ struct BatchRun {
     {
         variant = v;
         int occ = 0;
-        const BatchVariant& b = kBatchVariants[v];
-        const size_t smem = b.sym ? batch_sym_smem(b.tpt, b.threads) : 0;
-        if (smem) cudaFuncSetAttribute(b.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, b.fn, b.threads, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kBatchVariants[v].fn, kBatchVariants[v].threads, 0);
         grid = (occ < 1 ? 1 : occ) * sms;
     }
     ~BatchRun()

@@ -158,6 +158,45 @@ __device__ __forceinline__ void pair_far_sym(float2 Xx, float2 Xy, float2 Xz, fl
     r2 = __fmul2_rn(P, __ffma2_rn(sy, nv, __fmul2_rn(g, __fmul2_rn(ai, cc))));
 }
 
+// Both directions' sums of a pair.  Forward, with the source's weights (a, b) and
+// those that a regularised direction keeps (bt in the second sum, qf the 1/rho
+// factor); reverse likewise with the target's (nb = -b_i), accumulated: nR1 -=
+// first sum, R2 += second.
+// COMMON: the a-part of the second sum is the same in both directions,
+// W = [g c - (3 - B) s_x s_y / rho^2] / rho^3, formed once.  Otherwise each
+// direction forms its product with s_x or s_y.
+template <bool COMMON>
+__device__ __forceinline__ void sym_add(float2 P, float2 g, float2 hn, float2 inv2, float2 sx, float2 sy, float2 cc,
+                                        float2 Pu1, float2 Pu2, float2 a, float2 b, float2 bt, float2 qf, float2 ai,
+                                        float2 nb, float2 nbt, float2 qfr, float2& t1, float2& t2, float2& nR1,
+                                        float2& R2)
+{
+    if (COMMON) {
+        const float2 W = __fmul2_rn(P, __ffma2_rn(__fmul2_rn(hn, inv2), __fmul2_rn(sx, sy), __fmul2_rn(g, cc)));
+        t1 = __ffma2_rn(__fmul2_rn(Pu1, sy), a, t1);
+        t1 = __ffma2_rn(qf, b, t1);
+        t2 = __ffma2_rn(__fmul2_rn(Pu2, sx), bt, t2);
+        t2 = __ffma2_rn(W, a, t2);
+        nR1 = __ffma2_rn(__fmul2_rn(Pu1, sx), ai, nR1);
+        nR1 = __ffma2_rn(qfr, nb, nR1);
+        R2 = __ffma2_rn(__fmul2_rn(Pu2, sy), nbt, R2);
+        R2 = __ffma2_rn(W, ai, R2);
+    } else {
+        const float2 Pgc = __fmul2_rn(__fmul2_rn(P, g), cc);
+        const float2 Phi = __fmul2_rn(hn, __fmul2_rn(inv2, P));
+        const float2 sa = __fmul2_rn(a, sy);
+        t1 = __ffma2_rn(Pu1, sa, t1);
+        t1 = __ffma2_rn(qf, b, t1);
+        t2 = __ffma2_rn(sx, __ffma2_rn(Phi, sa, __fmul2_rn(Pu2, bt)), t2);
+        t2 = __ffma2_rn(Pgc, a, t2);
+        const float2 psa = __fmul2_rn(ai, sx);
+        nR1 = __ffma2_rn(Pu1, psa, nR1);
+        nR1 = __ffma2_rn(qfr, nb, nR1);
+        R2 = __ffma2_rn(sy, __ffma2_rn(Phi, psa, __fmul2_rn(Pu2, nbt)), R2);
+        R2 = __ffma2_rn(Pgc, ai, R2);
+    }
+}
+
 // pair_far_sym with the reverse sums accumulated into (nR1, R2) (rotation
 // scheme): nR1 -= first reverse sum, R2 += second.  The a-part of the second sum
 // is the same in both directions, W = [g c - (3 - B) s_x s_y / rho^2] / rho^3:
@@ -169,6 +208,8 @@ __device__ __forceinline__ void pair_far_sym(float2 Xx, float2 Xy, float2 Xz, fl
 // 35.76 / 5.19 ms per application, 36.73 / 5.33 with 48 operations (each direction
 // its own s_x s_y product) and two MUFU; rho^-2 by a hardware reciprocal as well
 // (45 operations) 36.01 / 5.22.
+// COMMON false (the batched kernel, see there): the 48 operations and two MUFU.
+template <bool COMMON>
 __device__ __forceinline__ void pair_far_sym_acc(float2 Xx, float2 Xy, float2 Xz, float2 nx, float2 ny, float2 nz,
                                                  float2 ai, float2 nbi, const float4& A, const float4& B,
                                                  const float4& C, const float4& D, const FarConsts& c, float2& t1,
@@ -193,7 +234,8 @@ __device__ __forceinline__ void pair_far_sym_acc(float2 Xx, float2 Xy, float2 Xz
     cc = __ffma2_rn(ny, my, cc);
     cc = __ffma2_rn(nz, mz, cc);
     const float2 inv = make_float2(ptx::rsqrt_approx(rr.x), ptx::rsqrt_approx(rr.y));
-    const float2 rho = make_float2(ptx::sqrt_approx(rr.x), ptx::sqrt_approx(rr.y));
+    const float2 rho =
+        COMMON ? make_float2(ptx::sqrt_approx(rr.x), ptx::sqrt_approx(rr.y)) : __fmul2_rn(rr, inv);
     const float2 ea = __fmul2_rn(rho, c.kl2e);
     const float2 xn = __fmul2_rn(rho, c.nkappa);
     const float2 E = make_float2(ptx::ex2_approx(ea.x), ptx::ex2_approx(ea.y));
@@ -205,18 +247,8 @@ __device__ __forceinline__ void pair_far_sym_acc(float2 Xx, float2 Xy, float2 Xz
     const float2 P = __fmul2_rn(inv2, inv);
     const float2 Pu1 = __fmul2_rn(P, __ffma2_rn(c.th1, g, c.omth1));
     const float2 Pu2 = __fmul2_rn(P, __ffma2_rn(c.th2, g, c.omth2));
-    const float2 W = __fmul2_rn(P, __ffma2_rn(__fmul2_rn(hn, inv2), __fmul2_rn(sx, sy), __fmul2_rn(g, cc)));
     const float2 qf = __fmul2_rn(fn, inv);
-    // forward
-    t1 = __ffma2_rn(__fmul2_rn(Pu1, sy), aj, t1);
-    t1 = __ffma2_rn(qf, bj, t1);
-    t2 = __ffma2_rn(__fmul2_rn(Pu2, sx), bj, t2);
-    t2 = __ffma2_rn(W, aj, t2);
-    // reverse, accumulated
-    nR1 = __ffma2_rn(__fmul2_rn(Pu1, sx), ai, nR1);
-    nR1 = __ffma2_rn(qf, nbi, nR1);
-    R2 = __ffma2_rn(__fmul2_rn(Pu2, sy), nbi, R2);
-    R2 = __ffma2_rn(W, ai, R2);
+    sym_add<COMMON>(P, g, hn, inv2, sx, sy, cc, Pu1, Pu2, aj, bj, bj, qf, ai, nbi, nbi, qf, t1, t2, nR1, R2);
 }
 
 // Near pairs in the rotation scheme, both directions, packed over the two
@@ -237,7 +269,7 @@ __device__ __forceinline__ void pair_far_sym_acc(float2 Xx, float2 Xy, float2 Xz
 // without FLAT in the rare case that it lies in the band.  80k-node sphere with
 // every chunk near (tube rule 1): 8.6 ms flat, 9.4 ms with the branches.
 // i: the target's node index, j: the first source's.
-template <bool FLAT>
+template <bool FLAT, bool COMMON>
 __device__ __forceinline__ void pair_near_sym_acc(float2 Xx, float2 Xy, float2 Xz, float2 nx, float2 ny, float2 nz,
                                                   float2 ai, float2 nbi, const float4& A, const float4& B,
                                                   const float4& C, const float4& D, const FarConsts& c,
@@ -326,24 +358,15 @@ __device__ __forceinline__ void pair_near_sym_acc(float2 Xx, float2 Xy, float2 X
     const float2 P = __fmul2_rn(inv2, inv);
     const float2 Pu1 = __fmul2_rn(P, __ffma2_rn(c.th1, g, c.omth1));
     const float2 Pu2 = __fmul2_rn(P, __ffma2_rn(c.th2, g, c.omth2));
-    const float2 W = __fmul2_rn(P, __ffma2_rn(__fmul2_rn(hn, inv2), __fmul2_rn(sx, sy), __fmul2_rn(g, cc)));
     const float2 qf = __fmul2_rn(fn, inv);
-    // forward; a regularised pair adds -K12_tube b only
+    // a regularised direction adds -K12_tube b only
     const float2 ajf = make_float2(tf0 ? 0.0f : aj.x, tf1 ? 0.0f : aj.y);
     const float2 bjt = make_float2(tf0 ? 0.0f : bj.x, tf1 ? 0.0f : bj.y);
     const float2 qff = make_float2(tf0 ? -k.k12t : qf.x, tf1 ? -k.k12t : qf.y);
-    t1 = __ffma2_rn(__fmul2_rn(Pu1, sy), ajf, t1);
-    t1 = __ffma2_rn(qff, bj, t1);
-    t2 = __ffma2_rn(__fmul2_rn(Pu2, sx), bjt, t2);
-    t2 = __ffma2_rn(W, ajf, t2);
-    // reverse, accumulated (nbi = -b_i)
     const float2 air = make_float2(tr0 ? 0.0f : ai.x, tr1 ? 0.0f : ai.y);
     const float2 nbt = make_float2(tr0 ? 0.0f : nbi.x, tr1 ? 0.0f : nbi.y);
     const float2 qfr = make_float2(tr0 ? -k.k12t : qf.x, tr1 ? -k.k12t : qf.y);
-    nR1 = __ffma2_rn(__fmul2_rn(Pu1, sx), air, nR1);
-    nR1 = __ffma2_rn(qfr, nbi, nR1);
-    R2 = __ffma2_rn(__fmul2_rn(Pu2, sy), nbt, R2);
-    R2 = __ffma2_rn(W, air, R2);
+    sym_add<COMMON>(P, g, hn, inv2, sx, sy, cc, Pu1, Pu2, ajf, bj, bjt, qff, air, nbi, nbt, qfr, t1, t2, nR1, R2);
 }
 
 // One ordered near pair (target <- source), scalar: tube test on the target's
@@ -485,12 +508,14 @@ __device__ __forceinline__ void warp_sum4_add(float v0, float v1, float v2, floa
 // pair_near_sym_acc, decided per target slot (each slot's 32 targets are one
 // block of the warp, so the choice is warp-uniform; inactive slots are
 // skipped there); otherwise the warp reduction, near chunks by the scalar
-// near_pair_sym.  UNR: unroll depth of the rotation loop over far chunks.
+// near_pair_sym.  UNR: unroll depth of the rotation loop over far chunks.  COMMON:
+// the arithmetic of pair_far_sym_acc; without it near chunks have no branch-free
+// form either.
 // Measured on the 80k-node sphere when the pair took 48 operations and near
 // chunks a scalar path: two targets per thread run fastest at 1 (5.65 ms; 5.72 at
 // 2, spills at 4), one target per thread at 4 (5.86 ms; 6.11 at 2, 6.22 at 1); at
 // these depths now 5.16 and 5.60 ms.
-template <int TPT, bool ROT, int UNR = 2, int CH = kChunksPerTile>
+template <int TPT, bool ROT, int UNR = 2, int CH = kChunksPerTile, bool COMMON = true>
 __device__ __forceinline__ void tile_sums_sym(const SymTargets<TPT>& T, const float4* tfrm, const float4* sb,
                                               const float4* sfrm, const F32Consts& k, float (&S1)[TPT],
                                               float (&C1)[TPT], float (&S2)[TPT], float (&C2)[TPT],
@@ -565,7 +590,7 @@ __device__ __forceinline__ void tile_sums_sym(const SymTargets<TPT>& T, const fl
                         const float4 A = cb[p], B = cb[P + p], C = cb[2 * P + p], D = cb[3 * P + p];
 #pragma unroll
                         for (int q = 0; q < TPT; ++q)
-                            pair_far_sym_acc(Xx[q], Xy[q], Xz[q], T.nx[q], T.ny[q], T.nz[q], aq[q], nbq[q], A, B, C,
+                            pair_far_sym_acc<COMMON>(Xx[q], Xy[q], Xz[q], T.nx[q], T.ny[q], T.nz[q], aq[q], nbq[q], A, B, C,
                                              D, fc, t1[q], t2[q], nR1, R2);
                         // pair p goes to lane hl - 1 at the next step: its sums follow it
                         nR1.x = __shfl_sync(0xffffffffu, nR1.x, nxt, P);
@@ -578,7 +603,7 @@ __device__ __forceinline__ void tile_sums_sym(const SymTargets<TPT>& T, const fl
                     float tmin = __builtin_huge_valf();
                     auto near_loop = [&](auto flat) {
                         constexpr bool FLAT = decltype(flat)::value;
-#pragma unroll(FLAT && TPT == 1 ? 2 : 1)
+#pragma unroll(TPT == 1 && (FLAT || !COMMON) ? 2 : 1)
                         for (int step = 0; step < P; ++step) {
                             const int p = (hl + step) & (P - 1);
                             const float4 A = cb[p], B = cb[P + p], C = cb[2 * P + p], D = cb[3 * P + p];
@@ -586,10 +611,10 @@ __device__ __forceinline__ void tile_sums_sym(const SymTargets<TPT>& T, const fl
                             for (int q = 0; q < TPT; ++q) {
                                 if (!act[q]) continue;
                                 if (TPT > 1 && farq[q])  // (one slot: this loop runs near chunks only)
-                                    pair_far_sym_acc(Xx[q], Xy[q], Xz[q], T.nx[q], T.ny[q], T.nz[q], aq[q], nbq[q], A,
+                                    pair_far_sym_acc<COMMON>(Xx[q], Xy[q], Xz[q], T.nx[q], T.ny[q], T.nz[q], aq[q], nbq[q], A,
                                                      B, C, D, fc, t1[q], t2[q], nR1, R2);
                                 else
-                                    pair_near_sym_acc<FLAT>(Xx[q], Xy[q], Xz[q], T.nx[q], T.ny[q], T.nz[q], aq[q],
+                                    pair_near_sym_acc<FLAT, COMMON>(Xx[q], Xy[q], Xz[q], T.nx[q], T.ny[q], T.nz[q], aq[q],
                                                           nbq[q], A, B, C, D, fc, k, t1[q], t2[q], nR1, R2, tmin, g64,
                                                           gi0 + (int64_t)q * qstride, jc + 2 * p, N);
                             }
@@ -599,8 +624,9 @@ __device__ __forceinline__ void tile_sums_sym(const SymTargets<TPT>& T, const fl
                             R2.y = __shfl_sync(0xffffffffu, R2.y, nxt, P);
                         }
                     };
-                    near_loop(std::true_type{});
-                    if (__any_sync(0xffffffffu, tmin < kTieBand * k.tau2)) {  // a tie: the chunk again, decided in FP64
+                    if (COMMON) near_loop(std::true_type{});
+                    // (with COMMON only after a tie: the chunk again, decided in FP64)
+                    if (!COMMON || __any_sync(0xffffffffu, tmin < kTieBand * k.tau2)) {
                         nR1 = R2 = make_float2(0.0f, 0.0f);
 #pragma unroll
                         for (int q = 0; q < TPT; ++q) t1[q] = t2[q] = make_float2(0.0f, 0.0f);
