@@ -178,6 +178,9 @@ ibim_status ibim_get_jacobian(const ibim_ctx* ctx, double* J);
  *   y2_i = lambda2 psin_i + sum_j [K21(i,j) w_j psi_j - K22(i,j) w_j psin_j]
  * d_in, d_out: device, 2N doubles each, must not overlap.  Asynchronous on
  * the context stream.  precision: IBIM_F64, IBIM_FF, IBIM_F32C or IBIM_F32T.
+ * The first application on a context allocates the workspaces of all precisions
+ * (later ones can be captured into a CUDA graph), the first in IBIM_F64 another
+ * 2.6 KB per node, also while the calling thread captures.
  */
 ibim_status ibim_matvec(ibim_ctx* ctx, const ibim_phys* phys, int precision, const double* d_in,
                         double* d_out);

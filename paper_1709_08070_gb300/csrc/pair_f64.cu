@@ -262,12 +262,20 @@ __global__ void __launch_bounds__(kF64Parts * kF64Nodes)
 size_t f64_src_bytes(int64_t N) { return (size_t)f64_plan(N).n_chunks * kF64Chunk * 8 * sizeof(double); }
 
 // The partial sums of the FP64 path (kept apart from the other paths' buffer:
-// they take 2.6 KB per node and are allocated on the first FP64 application).
+// they take 2.6 KB per node and are allocated on the first FP64 application, once
+// per context).  That application may be one that the caller captures after
+// applications of another precision: the relaxed mode lets this thread allocate
+// meanwhile, and the buffer is an ordinary one that outlives the graph.
 ibim_status f64_prepare(ibim_ctx* c)
 {
+    if (c->d_part64 != nullptr) return IBIM_OK;
     const F64Plan p = f64_plan(c->N);
-    return ensure(c, (void**)&c->d_part64, &c->part64_bytes,
-                  sizeof(double) * (kF64Head + (size_t)p.items * 4 * p.m * kF64Chunk));
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    IBIM_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+    const ibim_status s = ensure(c, (void**)&c->d_part64, &c->part64_bytes,
+                                 sizeof(double) * (kF64Head + (size_t)p.items * 4 * p.m * kF64Chunk));
+    IBIM_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));  // the thread's own mode again
+    return s;
 }
 
 ibim_status f64_apply(ibim_ctx* c, const PairConsts& k, VecRef in, OutRef out, const int* d_skip)
