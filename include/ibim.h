@@ -400,9 +400,10 @@ ibim_status ibim_f32_variant_info(int v, int* targets_per_thread, int* min_ctas_
  * kernel whose results repeat bit for bit),
  * keeps the fastest for this context and caches it for contexts built later
  * in the process of the same geometry kind (analytic sphere, level-set
- * surface or caller-given nodes) with N in the same power-of-two bucket.  Returns the chosen
- * variant, its resident CTAs per SM and its time per application (outputs
- * may be NULL).  Synchronises; call it outside any stream capture.
+ * surface or caller-given nodes) with N in the same power-of-two bucket and on
+ * the same side of that limit.  Returns the chosen variant, its resident CTAs per
+ * SM and its time per application (outputs may be NULL).  Synchronises; call it
+ * outside any stream capture.
  */
 ibim_status ibim_autotune(ibim_ctx* ctx, const ibim_phys* phys, int* variant, int* ctas_per_sm, double* best_ms);
 

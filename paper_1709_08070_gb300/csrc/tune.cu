@@ -1,12 +1,14 @@
 // Autotuner of the FP32 pair-sum kernel: measures each variant (targets per
 // thread x CTAs per SM) on a context's own geometry with CUDA events and keeps
-// the fastest, cached per (geometry kind, problem-size bucket floor(log2 N))
+// the fastest, cached per (geometry kind, problem-size bucket floor(log2 N), and
+// whether N lies in the repeatable range below)
 // for contexts built later in the process: an analytic sphere, a level-set
 // surface and a caller's node cloud of the same size have different near-field
 // shares, so one kind's choice is not applied to another.
 #include <atomic>
 #include <map>
 #include <mutex>
+#include <tuple>
 #include <vector>
 
 #include "ibim_internal.cuh"
@@ -15,7 +17,7 @@ namespace ibim {
 
 namespace {
 std::mutex g_tune_mu;
-std::map<std::pair<int, int>, std::pair<int, int>> g_tune_cache;  // (kind, bucket) -> (variant, CTAs per SM)
+std::map<std::tuple<int, int, bool>, std::pair<int, int>> g_tune_cache;  // cache_key -> (variant, CTAs per SM)
 
 // Up to this many nodes (18 source tiles) only one-directional variants are
 // timed, so that small molecules' applications and solves repeat bit for bit:
@@ -40,7 +42,12 @@ int geometry_kind(const ibim_ctx* c)
     return c->band_eps > 0.0 ? 1 : 0;
 }
 
-std::pair<int, int> cache_key(const ibim_ctx* c) { return {geometry_kind(c), size_bucket(c->N)}; }
+// The repeatable range ends inside a bucket: its two parts have different
+// candidates and keep their own choices.
+std::tuple<int, int, bool> cache_key(const ibim_ctx* c)
+{
+    return {geometry_kind(c), size_bucket(c->N), c->N <= kRepeatableNodes};
+}
 
 __global__ void fill_kernel(double* __restrict__ p, int64_t n)
 {
