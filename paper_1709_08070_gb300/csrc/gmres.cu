@@ -606,7 +606,8 @@ static ibim_status capture_step(ibim_ctx* c, const PairConsts& k, int precision)
     IBIM_TRY(ensure_operator_workspaces(c));
     if (precision == IBIM_F64) IBIM_TRY(f64_prepare(c));
     if (w->graph_valid && w->graph_prec == precision && memcmp(&w->graph_k, &k, sizeof(k)) == 0 &&
-        w->graph_generation == c->ws_generation && w->graph_variant == c->f32_variant && w->graph_bps == c->f32_bps)
+        w->graph_generation == c->ws_generation && w->graph_variant == c->f32_variant && w->graph_bps == c->f32_bps &&
+        w->graph_ff == c->ff_symmetric)
         return IBIM_OK;
     if (w->exec) {
         cudaGraphExecDestroy(w->exec);
@@ -634,6 +635,7 @@ static ibim_status capture_step(ibim_ctx* c, const PairConsts& k, int precision)
     w->graph_generation = c->ws_generation;
     w->graph_variant = c->f32_variant;
     w->graph_bps = c->f32_bps;
+    w->graph_ff = c->ff_symmetric;
     return IBIM_OK;
 }
 

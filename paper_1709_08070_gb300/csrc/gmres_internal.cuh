@@ -71,6 +71,7 @@ struct GmresWork {
     uint64_t graph_generation = 0;  // workspace generation the graph was captured with
     int graph_variant = -1;         // FP32 pair-kernel variant and CTAs per SM captured in the graph
     int graph_bps = -1;
+    int graph_ff = -1;              // float-float kernel captured in the graph
     bool graph_valid = false;
 };
 
