@@ -158,43 +158,27 @@ __device__ __forceinline__ void pair_far_sym(float2 Xx, float2 Xy, float2 Xz, fl
     r2 = __fmul2_rn(P, __ffma2_rn(sy, nv, __fmul2_rn(g, __fmul2_rn(ai, cc))));
 }
 
-// Both directions' sums of a pair.  Forward, with the source's weights (a, b) and
-// those that a regularised direction keeps (bt in the second sum, qf the 1/rho
-// factor); reverse likewise with the target's (nb = -b_i), accumulated: nR1 -=
-// first sum, R2 += second.
-// COMMON: the a-part of the second sum is the same in both directions,
-// W = [g c - (3 - B) s_x s_y / rho^2] / rho^3, formed once.  Otherwise each
-// direction forms its product with s_x or s_y.
-template <bool COMMON>
-__device__ __forceinline__ void sym_add(float2 P, float2 g, float2 hn, float2 inv2, float2 sx, float2 sy, float2 cc,
-                                        float2 Pu1, float2 Pu2, float2 a, float2 b, float2 bt, float2 qf, float2 ai,
-                                        float2 nb, float2 nbt, float2 qfr, float2& t1, float2& t2, float2& nR1,
-                                        float2& R2)
+// Both directions' sums of a pair, each direction forming its products with s_x or
+// s_y.  Forward, with the source's weights (a, b) and what a regularised direction
+// keeps of them (bt in the second sum, qf the 1/rho factor); reverse likewise with
+// the target's (nb = -b_i), accumulated: nR1 -= first sum, R2 += second.
+__device__ __forceinline__ void sym_add_apart(float2 P, float2 g, float2 hn, float2 inv2, float2 sx, float2 sy,
+                                              float2 cc, float2 Pu1, float2 Pu2, float2 a, float2 b, float2 bt,
+                                              float2 qf, float2 ai, float2 nb, float2 nbt, float2 qfr, float2& t1,
+                                              float2& t2, float2& nR1, float2& R2)
 {
-    if (COMMON) {
-        const float2 W = __fmul2_rn(P, __ffma2_rn(__fmul2_rn(hn, inv2), __fmul2_rn(sx, sy), __fmul2_rn(g, cc)));
-        t1 = __ffma2_rn(__fmul2_rn(Pu1, sy), a, t1);
-        t1 = __ffma2_rn(qf, b, t1);
-        t2 = __ffma2_rn(__fmul2_rn(Pu2, sx), bt, t2);
-        t2 = __ffma2_rn(W, a, t2);
-        nR1 = __ffma2_rn(__fmul2_rn(Pu1, sx), ai, nR1);
-        nR1 = __ffma2_rn(qfr, nb, nR1);
-        R2 = __ffma2_rn(__fmul2_rn(Pu2, sy), nbt, R2);
-        R2 = __ffma2_rn(W, ai, R2);
-    } else {
-        const float2 Pgc = __fmul2_rn(__fmul2_rn(P, g), cc);
-        const float2 Phi = __fmul2_rn(hn, __fmul2_rn(inv2, P));
-        const float2 sa = __fmul2_rn(a, sy);
-        t1 = __ffma2_rn(Pu1, sa, t1);
-        t1 = __ffma2_rn(qf, b, t1);
-        t2 = __ffma2_rn(sx, __ffma2_rn(Phi, sa, __fmul2_rn(Pu2, bt)), t2);
-        t2 = __ffma2_rn(Pgc, a, t2);
-        const float2 psa = __fmul2_rn(ai, sx);
-        nR1 = __ffma2_rn(Pu1, psa, nR1);
-        nR1 = __ffma2_rn(qfr, nb, nR1);
-        R2 = __ffma2_rn(sy, __ffma2_rn(Phi, psa, __fmul2_rn(Pu2, nbt)), R2);
-        R2 = __ffma2_rn(Pgc, ai, R2);
-    }
+    const float2 Pgc = __fmul2_rn(__fmul2_rn(P, g), cc);
+    const float2 Phi = __fmul2_rn(hn, __fmul2_rn(inv2, P));
+    const float2 sa = __fmul2_rn(a, sy);
+    t1 = __ffma2_rn(Pu1, sa, t1);
+    t1 = __ffma2_rn(qf, b, t1);
+    t2 = __ffma2_rn(sx, __ffma2_rn(Phi, sa, __fmul2_rn(Pu2, bt)), t2);
+    t2 = __ffma2_rn(Pgc, a, t2);
+    const float2 psa = __fmul2_rn(ai, sx);
+    nR1 = __ffma2_rn(Pu1, psa, nR1);
+    nR1 = __ffma2_rn(qfr, nb, nR1);
+    R2 = __ffma2_rn(sy, __ffma2_rn(Phi, psa, __fmul2_rn(Pu2, nbt)), R2);
+    R2 = __ffma2_rn(Pgc, ai, R2);
 }
 
 // pair_far_sym with the reverse sums accumulated into (nR1, R2) (rotation
@@ -247,8 +231,23 @@ __device__ __forceinline__ void pair_far_sym_acc(float2 Xx, float2 Xy, float2 Xz
     const float2 P = __fmul2_rn(inv2, inv);
     const float2 Pu1 = __fmul2_rn(P, __ffma2_rn(c.th1, g, c.omth1));
     const float2 Pu2 = __fmul2_rn(P, __ffma2_rn(c.th2, g, c.omth2));
+    if (!COMMON) {
+        const float2 qf = __fmul2_rn(fn, inv);
+        sym_add_apart(P, g, hn, inv2, sx, sy, cc, Pu1, Pu2, aj, bj, bj, qf, ai, nbi, nbi, qf, t1, t2, nR1, R2);
+        return;
+    }
+    const float2 W = __fmul2_rn(P, __ffma2_rn(__fmul2_rn(hn, inv2), __fmul2_rn(sx, sy), __fmul2_rn(g, cc)));
     const float2 qf = __fmul2_rn(fn, inv);
-    sym_add<COMMON>(P, g, hn, inv2, sx, sy, cc, Pu1, Pu2, aj, bj, bj, qf, ai, nbi, nbi, qf, t1, t2, nR1, R2);
+    // forward
+    t1 = __ffma2_rn(__fmul2_rn(Pu1, sy), aj, t1);
+    t1 = __ffma2_rn(qf, bj, t1);
+    t2 = __ffma2_rn(__fmul2_rn(Pu2, sx), bj, t2);
+    t2 = __ffma2_rn(W, aj, t2);
+    // reverse, accumulated
+    nR1 = __ffma2_rn(__fmul2_rn(Pu1, sx), ai, nR1);
+    nR1 = __ffma2_rn(qf, nbi, nR1);
+    R2 = __ffma2_rn(__fmul2_rn(Pu2, sy), nbi, R2);
+    R2 = __ffma2_rn(W, ai, R2);
 }
 
 // Near pairs in the rotation scheme, both directions, packed over the two
@@ -358,15 +357,30 @@ __device__ __forceinline__ void pair_near_sym_acc(float2 Xx, float2 Xy, float2 X
     const float2 P = __fmul2_rn(inv2, inv);
     const float2 Pu1 = __fmul2_rn(P, __ffma2_rn(c.th1, g, c.omth1));
     const float2 Pu2 = __fmul2_rn(P, __ffma2_rn(c.th2, g, c.omth2));
+    const float2 W = __fmul2_rn(P, __ffma2_rn(__fmul2_rn(hn, inv2), __fmul2_rn(sx, sy), __fmul2_rn(g, cc)));
     const float2 qf = __fmul2_rn(fn, inv);
-    // a regularised direction adds -K12_tube b only
+    // forward; a regularised pair adds -K12_tube b only
     const float2 ajf = make_float2(tf0 ? 0.0f : aj.x, tf1 ? 0.0f : aj.y);
     const float2 bjt = make_float2(tf0 ? 0.0f : bj.x, tf1 ? 0.0f : bj.y);
     const float2 qff = make_float2(tf0 ? -k.k12t : qf.x, tf1 ? -k.k12t : qf.y);
+    if (COMMON) {
+        t1 = __ffma2_rn(__fmul2_rn(Pu1, sy), ajf, t1);
+        t1 = __ffma2_rn(qff, bj, t1);
+        t2 = __ffma2_rn(__fmul2_rn(Pu2, sx), bjt, t2);
+        t2 = __ffma2_rn(W, ajf, t2);
+    }
+    // reverse, accumulated (nbi = -b_i)
     const float2 air = make_float2(tr0 ? 0.0f : ai.x, tr1 ? 0.0f : ai.y);
     const float2 nbt = make_float2(tr0 ? 0.0f : nbi.x, tr1 ? 0.0f : nbi.y);
     const float2 qfr = make_float2(tr0 ? -k.k12t : qf.x, tr1 ? -k.k12t : qf.y);
-    sym_add<COMMON>(P, g, hn, inv2, sx, sy, cc, Pu1, Pu2, ajf, bj, bjt, qff, air, nbi, nbt, qfr, t1, t2, nR1, R2);
+    if (!COMMON) {
+        sym_add_apart(P, g, hn, inv2, sx, sy, cc, Pu1, Pu2, ajf, bj, bjt, qff, air, nbi, nbt, qfr, t1, t2, nR1, R2);
+        return;
+    }
+    nR1 = __ffma2_rn(__fmul2_rn(Pu1, sx), air, nR1);
+    nR1 = __ffma2_rn(qfr, nbi, nR1);
+    R2 = __ffma2_rn(__fmul2_rn(Pu2, sy), nbt, R2);
+    R2 = __ffma2_rn(W, air, R2);
 }
 
 // One ordered near pair (target <- source), scalar: tube test on the target's
