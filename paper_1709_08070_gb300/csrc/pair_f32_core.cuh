@@ -192,18 +192,20 @@ static __device__ __noinline__ bool tube_f64(const Geo64& g, int64_t i, int64_t 
 // FP32 tube test defers to tube_f64.
 constexpr float kTieBand = 1e-5f;
 
-// Margins of the tube test, packed: p = tau^2 - rho^2 (to which s_x^2 is added:
-// positive inside the tangent-plane cylinder) and q = (4 tau^2 - rho^2) / 4
-// (+inf for tube rule 1), so that both have the tie band kTieBand tau^2.
-struct TubeTest {
-    float2 p, q;
-};
-__device__ __forceinline__ TubeTest tube_margins(float2 rr, const F32Consts& k)
+// Margins of the tube test, packed, both with the tie band kTieBand tau^2:
+// tau^2 - rho_P^2 (positive inside the tangent-plane cylinder; s = r . n with the
+// direction's normal) and (4 tau^2 - rho^2) / 4 (+inf for tube rule 1).  Their
+// signs are those of the comparisons rho_P^2 < tau^2 and rho^2 < 4 tau^2:
+// rho_P^2 = rho^2 - s^2 is rounded once, and as there (tau^2 - rho^2 first would
+// lose half a unit of rho^2, which under rule 1 can be far above tau^2).
+__device__ __forceinline__ float2 plane_margin(float2 rr, float2 s, const F32Consts& k)
 {
-    TubeTest t;
-    t.p = __ffma2_rn(rr, f2(-1.0f), f2(k.tau2));
-    t.q = __ffma2_rn(rr, f2(-0.25f), f2(0.25f * k.four_tau2));
-    return t;
+    const float2 rp = __ffma2_rn(make_float2(-s.x, -s.y), s, rr);
+    return __fadd2_rn(f2(k.tau2), make_float2(-rp.x, -rp.y));
+}
+__device__ __forceinline__ float2 ball_margin(float2 rr, const F32Consts& k)
+{
+    return __ffma2_rn(rr, f2(-0.25f), f2(0.25f * k.four_tau2));
 }
 
 // g from its series (g_series, both lanes at once) and fn = -(1 - E) = E xn - g
@@ -234,8 +236,10 @@ __device__ __forceinline__ void series_where_small(float2 xn, float2 En, const F
 // the 1/rho factor of the first sum.  rho^2 is kept >= 1e-12, so that
 // coincident nodes (the self pair among them, always in the tube) leave
 // every product finite.  A test within kTieBand of a threshold has to be
-// decided in FP64 (tube_f64, which the FP32 test agrees with outside the
-// band).  Without FLAT that is done on the spot, by a branch, and the series by
+// decided in FP64 (tube_f64; outside the band the FP32 test agrees with it as long
+// as rho^2 is of tau^2's size, as under rule 0, where a decision at larger rho is
+// the ball's; under rule 1 the rounding of rho^2 exceeds the band from about 10 tau
+// on, and a pair that close to the cylinder falls as FP32 has it).  Without FLAT that is done on the spot, by a branch, and the series by
 // another; FLAT has no branch and keeps the smallest distance to a threshold in
 // tmin: the caller repeats the chunk without FLAT when it lies in the band.
 // (One-directional kernel, 5k-node sphere, almost every chunk near: 79 us flat,
@@ -267,11 +271,10 @@ __device__ __forceinline__ void pair_near2(float2 Xx, float2 Xy, float2 Xz, floa
     ca = __ffma2_rn(nz, mz, ca);
     bool t0, t1b;
     if (FLAT) {
-        const TubeTest tt = tube_margins(rr, k);
-        const float2 mf = __ffma2_rn(sx, sx, tt.p);
-        t0 = (mf.x > 0.0f) & (tt.q.x > 0.0f);
-        t1b = (mf.y > 0.0f) & (tt.q.y > 0.0f);
-        tmin = fminf(tmin, fminf(fminf(fabsf(mf.x), fabsf(tt.q.x)), fminf(fabsf(mf.y), fabsf(tt.q.y))));
+        const float2 mf = plane_margin(rr, sx, k), mq = ball_margin(rr, k);
+        t0 = (mf.x > 0.0f) & (mq.x > 0.0f);
+        t1b = (mf.y > 0.0f) & (mq.y > 0.0f);
+        tmin = fminf(tmin, fminf(fminf(fabsf(mf.x), fabsf(mq.x)), fminf(fabsf(mf.y), fabsf(mq.y))));
     } else {
         const float2 rp = __ffma2_rn(__fmul2_rn(sx, c.neg1), sx, rr);
         t0 = (rp.x < k.tau2) & (rr.x < k.four_tau2);

@@ -260,8 +260,8 @@ __device__ __forceinline__ void pair_far_sym_acc(float2 Xx, float2 Xy, float2 Xz
 // of its 1/rho factor, so the products with the powers of 1/rho stay shared.
 // rho^2 is kept >= 1e-12, so that coincident nodes (the self pair among
 // them, always in the tube) leave every product finite.
-// A test within kTieBand of a threshold has to be decided in FP64 (tube_f64,
-// which the FP32 tests agree with outside the band).  Without FLAT the four
+// A test within kTieBand of a threshold has to be decided in FP64 (tube_f64; see
+// pair_near2).  Without FLAT the four
 // tests are decided on the spot, by a branch, and the series are another two
 // branches; FLAT has none (the series is formed packed and selected) and keeps
 // the smallest distance to a threshold in tmin: the caller repeats the chunk
@@ -296,16 +296,14 @@ __device__ __forceinline__ void pair_near_sym_acc(float2 Xx, float2 Xy, float2 X
     cc = __ffma2_rn(nz, mz, cc);
     bool tf0, tf1, tr0, tr1;
     if (FLAT) {
-        // the signs of tau^2 - rho_P^2 and of (4 tau^2 - rho^2) / 4
-        const TubeTest tt = tube_margins(rr, k);
-        const float2 mf = __ffma2_rn(sx, sx, tt.p), mr = __ffma2_rn(sy, sy, tt.p);
-        const bool in0 = tt.q.x > 0.0f, in1 = tt.q.y > 0.0f;
+        const float2 mf = plane_margin(rr, sx, k), mr = plane_margin(rr, sy, k), mq = ball_margin(rr, k);
+        const bool in0 = mq.x > 0.0f, in1 = mq.y > 0.0f;
         tf0 = (mf.x > 0.0f) & in0;
         tf1 = (mf.y > 0.0f) & in1;
         tr0 = (mr.x > 0.0f) & in0;
         tr1 = (mr.y > 0.0f) & in1;
-        const float d0 = fminf(fminf(fabsf(mf.x), fabsf(mr.x)), fabsf(tt.q.x));
-        const float d1 = fminf(fminf(fabsf(mf.y), fabsf(mr.y)), fabsf(tt.q.y));
+        const float d0 = fminf(fminf(fabsf(mf.x), fabsf(mr.x)), fabsf(mq.x));
+        const float d1 = fminf(fminf(fabsf(mf.y), fabsf(mr.y)), fabsf(mq.y));
         tmin = fminf(tmin, fminf(d0, d1));
     } else {
         // tube tests: forward (f) on rho^2 - s_x^2, reverse (r) on rho^2 - s_y^2
