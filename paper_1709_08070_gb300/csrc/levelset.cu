@@ -87,7 +87,7 @@ __global__ void vdw_kernel(LsGrid g, CellList cl, const Atom* __restrict__ atoms
                     const float v = sqrtf(d0 * d0 + d1 * d1 + d2 * d2) - q.w;
                     if (pass == 0) {
                         f32 = fminf(f32, v);
-                    } else if (v <= f32) {
+                    } else if (!(v > f32)) {  // (also where FP32 gives no number)
                         const Atom z = atoms[a];
                         const double e0 = x0 - z.x, e1 = x1 - z.y, e2 = x2 - z.z;
                         f = fmin(f, sqrt(e0 * e0 + e1 * e1 + e2 * e2) - z.r);
@@ -561,11 +561,12 @@ ibim_status build_levelset(ibim_ctx* c, int64_t Na, const double* z, const doubl
 
     // FP32 copies relative to the cell origin; a distance minus radius formed
     // from them is within `margin` of the FP64 one (coordinates, radius and
-    // square root each within 2^-24 of at most the cell list's diagonal)
+    // square root each within 2^-24 of at most the cell list's diagonal); where
+    // squares of the coordinates would leave FP32's range, every atom is taken
     std::vector<float4> atoms32(Na);
     double diag = rmax;
     for (int a = 0; a < 3; ++a) diag += cl.cs * (cl.nc[a] + 2);
-    const float margin = (float)(16.0 * diag / 16777216.0);
+    const float margin = diag < 1e18 ? (float)(16.0 * diag / 16777216.0) : INFINITY;
     for (int64_t k = 0; k < Na; ++k)
         atoms32[k] = make_float4((float)(atoms[k].x - cl.co[0]), (float)(atoms[k].y - cl.co[1]),
                                  (float)(atoms[k].z - cl.co[2]), (float)atoms[k].r);
