@@ -147,14 +147,14 @@ __device__ __forceinline__ void weno_pair(const LsGrid& g, const double* __restr
 // c_i / (s_i + e)^2 are multiplied through by the three squares, so that one
 // reciprocal serves them all; smoothness and e carry a common factor 4.
 __device__ __forceinline__ double weno5_scaled(double v1, double v2, double v3, double v4, double v5, double q1,
-                                               double q2, double q3)
+                                               double q2, double q3, double floor4)
 {
     const double g1 = v2 - v1, g2 = v3 - v2, g3 = v4 - v3, g4 = v5 - v4;
     const double d1 = g2 - g1, d2 = g3 - g2, d3 = g4 - g3;
     const double e1 = fma(3.0, g2, -g1), e2 = g2 + g3, e3 = fma(-3.0, g3, g4);
     const double m = max_abs64(max_abs64(max_abs64(v1, v2), max_abs64(v3, v4)), v5);
     // 4 (1e-6 m^2 + tiny); the floor keeps the products below normal numbers
-    const double e = max_abs64(4e-6 * m * m, 4e-56);
+    const double e = max_abs64(4e-6 * m * m, floor4);
     const double t1 = fma(13.0 / 3.0 * d1, d1, fma(e1, e1, e));
     const double t2 = fma(13.0 / 3.0 * d2, d2, fma(e2, e2, e));
     const double t3 = fma(13.0 / 3.0 * d3, d3, fma(e3, e3, e));
@@ -181,11 +181,11 @@ struct AxisSides {
     double m1, m2, m3, p1;   // 6 h q: backward (m1, m2, m3), forward (p1, m3, m2)
 };
 
-__device__ __forceinline__ double weno_side(const AxisSides& A, bool back)
+__device__ __forceinline__ double weno_side(const AxisSides& A, bool back, double floor4)
 {
     const double w = weno5_scaled(back ? A.D[0] : A.D[5], back ? A.D[1] : A.D[4], back ? A.D[2] : A.D[3],
                                   back ? A.D[3] : A.D[2], back ? A.D[4] : A.D[1], back ? A.m1 : A.p1,
-                                  back ? A.m2 : A.m3, back ? A.m3 : A.m2);
+                                  back ? A.m2 : A.m3, back ? A.m3 : A.m2, floor4);
     return __longlong_as_double(back ? neg_bits(w) : pos_bits(w));
 }
 
@@ -214,7 +214,7 @@ __global__ void ls_sign_kernel(int64_t M, double h, const double* __restrict__ p
 __global__ void __launch_bounds__(kStageThreads)
     ls_stage_kernel(LsGrid g, const double* __restrict__ in, const double* __restrict__ base,
                     const double* __restrict__ sgn, double* __restrict__ out, double a, double b, double dt,
-                    double inv6h)
+                    double inv6h, double floor4)
 {
     constexpr int kQueue = 3 * kStageThreads;
     __shared__ double queue[8][kQueue];  // v1..v5, q1..q3 of a second evaluation; its value comes back in [0]
@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(kStageThreads)
         long long best = 0;
         slot[ax] = -1;
         if (max(bm, bp) > 0) {
-            best = max(0ll, pos_bits(weno_side(A, back)));
+            best = max(0ll, pos_bits(weno_side(A, back, floor4)));
             if (min(bm, bp) > best && live) {
                 const int e = atomicAdd(&queued, 1);
                 slot[ax] = e;
@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(kStageThreads)
     const int nq = queued;
     for (int e = threadIdx.x; e < nq; e += kStageThreads)
         queue[0][e] = weno5_scaled(queue[0][e], queue[1][e], queue[2][e], queue[3][e], queue[4][e], queue[5][e],
-                                   queue[6][e], queue[7][e]);
+                                   queue[6][e], queue[7][e], floor4);
     if (nq > 0) __syncthreads();
     if (!live) return;
     double s = 0.0;
@@ -618,6 +618,9 @@ ibim_status build_levelset(ibim_ctx* c, int64_t Na, const double* z, const doubl
     const unsigned nb = (unsigned)((M + bs - 1) / bs);
     const unsigned ns = (unsigned)((M + kStageThreads - 1) / kStageThreads);
     const double inv6h = 1.0 / (6.0 * h);
+    // floor of the WENO weights: 1e-25 of a slope, whatever the unit of length, as
+    // long as its fourth power is a normal number
+    const double floor4 = std::max(4e-56 * (4.0 * h * h), 1e-75);
     vdw_kernel<<<nb, bs, 0, c->stream>>>(g, cl, d_atoms, d_atoms32, d_start, L, probe, margin, d_phi);
     count_launch(c);
     LS_CUDA(cudaGetLastError());
@@ -627,10 +630,10 @@ ibim_status build_levelset(ibim_ctx* c, int64_t Na, const double* z, const doubl
         const int steps = (int)ceil(probe / (0.5 * h));
         const double dt = probe / steps;
         for (int s = 0; s < steps; ++s) {
-            ls_stage_kernel<<<ns, kStageThreads, 0, c->stream>>>(g, d_phi, d_phi, nullptr, d_t1, 0.0, 1.0, dt, inv6h);
-            ls_stage_kernel<<<ns, kStageThreads, 0, c->stream>>>(g, d_t1, d_phi, nullptr, d_t2, 0.75, 0.25, dt, inv6h);
+            ls_stage_kernel<<<ns, kStageThreads, 0, c->stream>>>(g, d_phi, d_phi, nullptr, d_t1, 0.0, 1.0, dt, inv6h, floor4);
+            ls_stage_kernel<<<ns, kStageThreads, 0, c->stream>>>(g, d_t1, d_phi, nullptr, d_t2, 0.75, 0.25, dt, inv6h, floor4);
             ls_stage_kernel<<<ns, kStageThreads, 0, c->stream>>>(g, d_t2, d_phi, nullptr, d_phi, 1.0 / 3.0, 2.0 / 3.0, dt,
-                                                                 inv6h);
+                                                                 inv6h, floor4);
             count_launch(c, 3);
         }
         LS_CUDA(cudaGetLastError());
@@ -675,10 +678,10 @@ ibim_status build_levelset(ibim_ctx* c, int64_t Na, const double* z, const doubl
         ls_sign_kernel<<<nb, bs, 0, c->stream>>>(M, h, d_phi, d_sgn);
         count_launch(c);
         for (int s = 0; s < steps; ++s) {
-            ls_stage_kernel<<<ns, kStageThreads, 0, c->stream>>>(g, d_phi, d_phi, d_sgn, d_t1, 0.0, 1.0, dt, inv6h);
-            ls_stage_kernel<<<ns, kStageThreads, 0, c->stream>>>(g, d_t1, d_phi, d_sgn, d_t2, 0.75, 0.25, dt, inv6h);
+            ls_stage_kernel<<<ns, kStageThreads, 0, c->stream>>>(g, d_phi, d_phi, d_sgn, d_t1, 0.0, 1.0, dt, inv6h, floor4);
+            ls_stage_kernel<<<ns, kStageThreads, 0, c->stream>>>(g, d_t1, d_phi, d_sgn, d_t2, 0.75, 0.25, dt, inv6h, floor4);
             ls_stage_kernel<<<ns, kStageThreads, 0, c->stream>>>(g, d_t2, d_phi, d_sgn, d_phi, 1.0 / 3.0, 2.0 / 3.0, dt,
-                                                                 inv6h);
+                                                                 inv6h, floor4);
             count_launch(c, 3);
         }
         LS_CUDA(cudaGetLastError());

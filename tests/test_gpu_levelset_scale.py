@@ -15,7 +15,7 @@ if not torch.cuda.is_available():  # pragma: no cover
 from paper_1709_08070_gb300 import ibim  # noqa: E402
 
 
-@pytest.mark.parametrize("power", [-33, 40, 64, 100])
+@pytest.mark.parametrize("power", [-60, -33, 40, 64, 100])
 def test_phi_scales_with_the_unit_of_length(power):
     z, r, _ = inputs.globule_atoms(25, seed=3)
     phis = []
