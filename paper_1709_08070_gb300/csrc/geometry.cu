@@ -8,7 +8,7 @@
 #include <math.h>
 
 #include <algorithm>
-#include <system_error>
+#include <exception>
 #include <thread>
 #include <vector>
 
@@ -284,7 +284,7 @@ void rcb_split(RcbNode* v, int64_t n, int spare)
             std::thread right;
             try {
                 right = std::thread(rcb_split, v + k, n - k, (spare - 1) / 2);
-            } catch (const std::system_error&) {  // no thread to be had: this one does both
+            } catch (const std::exception&) {  // no thread (or no memory for one): this one does both
                 rcb_split(v + k, n - k, 0);
             }
             rcb_split(v, k, (spare - 1) - (spare - 1) / 2);
