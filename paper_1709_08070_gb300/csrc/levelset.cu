@@ -14,8 +14,9 @@
 //                                             grad = (p_- + p_+)/2 (WENO5),
 //                                             x* = x - phi n, w = delta_eps(phi) h^3
 // The grid is origin-free: node (i, j, k) sits at h (lo + (i, j, k)).  The
-// file is compiled without FMA contraction so that the stencil arithmetic
-// rounds like plain C.
+// file is compiled without FMA contraction, so that the band's stencil arithmetic
+// and the last line of a stage round like plain C; the stages' WENO evaluation
+// names its fma() calls.
 #include <math.h>
 
 #include <algorithm>

@@ -178,8 +178,9 @@ __global__ void __launch_bounds__(THREADS, MINB)
 // The same sums for small launches, 64 targets per CTA: GROUPS threads per target
 // share the chunks of a source tile, and as a target's sum over a chunk does not
 // depend on the others, the first of them adds the chunk sums up in order, with
-// the compensation above: the result is pair_f32_kernel's bit for bit, and the
-// chain of one step is kChunksPerTile / GROUPS chunks instead of all.
+// the compensation above: a target's sum over a source tile is pair_f32_kernel's
+// bit for bit, and the chain of one step is kChunksPerTile / GROUPS chunks instead
+// of all.
 template <int GROUPS>
 __global__ void __launch_bounds__(kSmallTTile * GROUPS, 512 / (kSmallTTile * GROUPS))
     pair_f32_small_kernel(const float4* __restrict__ tpos, const float4* __restrict__ tnrm,
@@ -457,8 +458,9 @@ static const F32Variant kVariants[] = {
 // below kSmallSteps steps of its own kernel (about 15,000 nodes) they run
 // pair_f32_small_kernel: 64-target tiles, four times as many steps, so that the
 // chip is filled, four threads to a target, and the branch-free near formula, as
-// most chunk pairs are near.  The result is the same bit for bit.  Clouds on a
-// sphere, one application after another, one / two / four / eight threads to a
+// most chunk pairs are near.  The tile sums are the same bit for bit; they fall to
+// other CTAs than with 256-target tiles, so their FP64 sums group differently (1e-16
+// of the result), and each launch repeats itself.  Clouds on a sphere, one application after another, one / two / four / eight threads to a
 // target: 862 nodes 20.9 / 14.8 / 14.7 / 14.6 us (the three launches take 13),
 // 3,001 31.1 / 31.0 / 30.3 / 31.1, 6,500 98 / 86 / 78 / 87, 15,000 341 / 324 / 334 /
 // 375; variant 0's own kernel took 70.5 us at 3,001 nodes and 279 at 12,000 (235 so),

@@ -389,10 +389,9 @@ struct SymVariant {
 // The last three, with smaller source tiles and target tiles, are for small
 // molecules: a launch of 512-target tiles on 5,000 nodes has 110 steps for 152
 // SMs.  Measured per application (us; the best of the first four, then these):
-// 862 nodes 66 / 21.7 33 63; 4,982 68 / 50.8 56 67; 12,754 201 / 198 186 191;
-// 21,651 467 / 531 504 445; 37,657 1245 / 1515 1417 1244; 80,358 5334 / 6459
+// 4,982 nodes 68 / 50.8 56 67; 12,754 201 / 198 186 191; 21,651 467 / 531 504 445; 37,657 1245 / 1515 1417 1244; 80,358 5334 / 6459
 // 6102 5583 (the smaller target tile reads every source more often).  The
-// autotuner picks.
+// autotuner picks, above 4,608 nodes.
 static const SymVariant kSymVariants[] = {
     IBIM_SYM_VARIANT(2, 1, 512, false, 2, 8), IBIM_SYM_VARIANT(1, 1, 512, false, 2, 8),
     IBIM_SYM_VARIANT(2, 1, 512, true, 1, 8),  IBIM_SYM_VARIANT(1, 1, 512, true, 4, 8),

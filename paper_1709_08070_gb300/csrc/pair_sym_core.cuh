@@ -526,7 +526,7 @@ __device__ __forceinline__ void warp_sum4_add(float v0, float v1, float v2, floa
 // Measured on the 80k-node sphere when the pair took 48 operations and near
 // chunks a scalar path: two targets per thread run fastest at 1 (5.65 ms; 5.72 at
 // 2, spills at 4), one target per thread at 4 (5.86 ms; 6.11 at 2, 6.22 at 1); at
-// these depths now 5.16 and 5.60 ms.
+// these depths now 5.17 and 5.60 ms.
 template <int TPT, bool ROT, int UNR = 2, int CH = kChunksPerTile, bool COMMON = true>
 __device__ __forceinline__ void tile_sums_sym(const SymTargets<TPT>& T, const float4* tfrm, const float4* sb,
                                               const float4* sfrm, const F32Consts& k, float (&S1)[TPT],
